@@ -1,0 +1,133 @@
+// dg_f64.cuh -- FP64 building blocks for the narrow FP64 pipe of sm_103a.
+//
+// The chip executes two FP64 operations per SM and cycle (a warp-wide DADD, DMUL,
+// DFMA or DSETP holds a sub-partition's pipe for 64 cycles), so the FP64 kernels are
+// bound by the number of FP64 instructions.  What can run elsewhere does: seeds come
+// from the special-function unit (rcp.approx / rsqrt.approx on the high word),
+// comparisons, exponents and tables from the integer pipe.
+//   rcpv     1/x: one cubically convergent step r (1 + e + e^2), e = 1 - x r, from the
+//            ~20-bit seed: 3 FP64 operations, within about 1 ulp.
+//   rsqrt64, sqrtv: one cubic (Householder) step y (1 + e/2 + 3e^2/8), e = 1 - x y^2:
+//            5 FP64 operations.
+//   pow_m1   x^z and x^z - 1 by log2 and exp2 with a table of 2^(i/64) and Taylor
+//            polynomials on the remainders (|ln| <= 0.0055): about 22 operations;
+//            x^z - 1 keeps its relative accuracy near x = 1.
+#pragma once
+
+#include <cuda_runtime.h>
+
+namespace dgk {
+
+// x > 0 and not NaN (+inf is positive), without a comparison on the FP64 pipe.
+__device__ __forceinline__ bool posv(double x) {
+  return (unsigned long long)(__double_as_longlong(x) - 1) < 0x7ff0000000000000ull;
+}
+__device__ __forceinline__ bool posv(float x) { return x > 0.0f; }
+
+// a > b for positive a and b (or a NaN on neither side).
+__device__ __forceinline__ bool gt_pos(double a, double b) {
+  return __double_as_longlong(a) > __double_as_longlong(b);
+}
+
+// The exponent of x is in [2, 2044]: neither x nor 1/x is zero, subnormal, infinite
+// or NaN, and the refinement of a seed is safe.
+__device__ __forceinline__ bool refinable(double x) {
+  return ((((unsigned)__double2hiint(x) >> 20) & 0x7ffu) - 2u) <= 2042u;
+}
+
+// 1/x.  Outside the refinable range the seed is the result (1/0 = inf, 1/inf = 0,
+// NaN; results below 2^-1022 flush to zero).
+__device__ __forceinline__ double rcpv(double x) {
+  double r;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
+  const double e = fma(-x, r, 1.0);
+  const double y = fma(r, fma(e, e, e), r);
+  return refinable(x) ? y : r;
+}
+
+// 1/sqrt(x), x positive and refinable.
+__device__ __forceinline__ double rsqrt64(double x) {
+  double y;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  const double e = fma(-(x * y), y, 1.0);
+  return fma(y * e, fma(0.375, e, 0.5), y);
+}
+
+// sqrt(x), x >= 0 (zero, subnormal, infinite and NaN x are returned as they are;
+// a negative x gives a NaN).
+__device__ __forceinline__ double sqrt64(double x) {
+  double y;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  const double t = x * y;
+  const double e = fma(-t, y, 1.0);
+  const double s = fma(t * e, fma(0.375, e, 0.5), t);
+  return refinable(x) ? s : x;
+}
+
+// 2^(i/64), i = 0 .. 64, rounded to FP64.
+__device__ const double kExp2Tab[65] = {
+    0x1.0000000000000p+0, 0x1.02c9a3e778061p+0, 0x1.059b0d3158574p+0,
+    0x1.0874518759bc8p+0, 0x1.0b5586cf9890fp+0, 0x1.0e3ec32d3d1a2p+0,
+    0x1.11301d0125b51p+0, 0x1.1429aaea92de0p+0, 0x1.172b83c7d517bp+0,
+    0x1.1a35beb6fcb75p+0, 0x1.1d4873168b9aap+0, 0x1.2063b88628cd6p+0,
+    0x1.2387a6e756238p+0, 0x1.26b4565e27cddp+0, 0x1.29e9df51fdee1p+0,
+    0x1.2d285a6e4030bp+0, 0x1.306fe0a31b715p+0, 0x1.33c08b26416ffp+0,
+    0x1.371a7373aa9cbp+0, 0x1.3a7db34e59ff7p+0, 0x1.3dea64c123422p+0,
+    0x1.4160a21f72e2ap+0, 0x1.44e086061892dp+0, 0x1.486a2b5c13cd0p+0,
+    0x1.4bfdad5362a27p+0, 0x1.4f9b2769d2ca7p+0, 0x1.5342b569d4f82p+0,
+    0x1.56f4736b527dap+0, 0x1.5ab07dd485429p+0, 0x1.5e76f15ad2148p+0,
+    0x1.6247eb03a5585p+0, 0x1.6623882552225p+0, 0x1.6a09e667f3bcdp+0,
+    0x1.6dfb23c651a2fp+0, 0x1.71f75e8ec5f74p+0, 0x1.75feb564267c9p+0,
+    0x1.7a11473eb0187p+0, 0x1.7e2f336cf4e62p+0, 0x1.82589994cce13p+0,
+    0x1.868d99b4492edp+0, 0x1.8ace5422aa0dbp+0, 0x1.8f1ae99157736p+0,
+    0x1.93737b0cdc5e5p+0, 0x1.97d829fde4e50p+0, 0x1.9c49182a3f090p+0,
+    0x1.a0c667b5de565p+0, 0x1.a5503b23e255dp+0, 0x1.a9e6b5579fdbfp+0,
+    0x1.ae89f995ad3adp+0, 0x1.b33a2b84f15fbp+0, 0x1.b7f76f2fb5e47p+0,
+    0x1.bcc1e904bc1d2p+0, 0x1.c199bdd85529cp+0, 0x1.c67f12e57d14bp+0,
+    0x1.cb720dcef9069p+0, 0x1.d072d4a07897cp+0, 0x1.d5818dcfba487p+0,
+    0x1.da9e603db3285p+0, 0x1.dfc97337b9b5fp+0, 0x1.e502ee78b3ff6p+0,
+    0x1.ea4afa2a490dap+0, 0x1.efa1bee615a27p+0, 0x1.f50765b6e4540p+0,
+    0x1.fa7c1819e90d8p+0, 0x1.0000000000000p+1};
+
+// x^z for x positive and refinable and |z| <= 4; returns x^z - 1 and, in w, x^z.
+//   x = 2^(e+1) h, h in [1/2, 1);  k = 64 (1 + log2 h) to the nearest integer (FP32);
+//   r = h 2^((64-k)/64) - 1, |r| < 0.0056;  log2 x = (64 e + k)/64 + log2(1 + r);
+//   z log2 x = n/64 + f, |f| <= 1/128;  x^z = 2^(n/64) 2^f.
+// log2(1 + r) and 2^f - 1 by Taylor polynomials of degree 7 and 6 (truncation
+// 2e-17 and 5e-18 relative): the table-driven scheme of Tang (ACM TOMS 1989, 1990).
+__device__ __forceinline__ double pow_m1(double x, double z, double& w) {
+  const int hx = __double2hiint(x), lx = __double2loint(x);
+  const int e = (hx >> 20) - 1023;
+  const float m = __int_as_float(0x3f800000 | ((hx & 0x000fffff) << 3) | ((unsigned)lx >> 29));
+  int k = __float2int_rn(64.0f * __log2f(m));
+  k = k < 0 ? 0 : (k > 64 ? 64 : k);
+  const double h = __hiloint2double((hx & 0x000fffff) | 0x3fe00000, lx);
+  const double r = fma(h, __ldg(&kExp2Tab[64 - k]), -1.0);
+  double q = 0.2060992915555662;
+  q = fma(q, r, -0.2404491734814939);
+  q = fma(q, r, 0.28853900817779266);
+  q = fma(q, r, -0.36067376022224085);
+  q = fma(q, r, 0.4808983469629878);
+  q = fma(q, r, -0.7213475204444817);
+  q = fma(q, r, 1.4426950408889634);
+  // integers to FP64 by the 1.5 * 2^52 shift
+  constexpr double shift = 6755399441055744.0;
+  const double nk = __hiloint2double(0x43380000 + ((64 * e + k) >> 31), 64 * e + k) - shift;
+  const double y = fma(z * 0.015625, nk, z * (q * r));
+  const double ys = fma(y, 64.0, shift);
+  const int n = __double2loint(ys);
+  const double f = fma(ys - shift, -0.015625, y);
+  double p = 0.0001540353039338161;
+  p = fma(p, f, 0.0013333558146428443);
+  p = fma(p, f, 0.009618129107628477);
+  p = fma(p, f, 0.05550410866482158);
+  p = fma(p, f, 0.24022650695910072);
+  p = fma(p, f, 0.6931471805599453);
+  p *= f;
+  const double t0 = __ldg(&kExp2Tab[n & 63]);
+  const double t = __hiloint2double(__double2hiint(t0) + ((n >> 6) << 20), __double2loint(t0));
+  w = fma(t, p, t);
+  return fma(t, p, t - 1.0);
+}
+
+}  // namespace dgk

@@ -873,6 +873,7 @@ Stage2DArgs<TS> stage_args(const AdjointCall& c, const Work& w, StateBuf<TS> in,
   a.dx = c.dx; a.dy = c.dy;
   a.gamma = c.gamma; a.cfl = 0.3; a.dt_override = dt; a.limiter = c.limiter;
   a.gas.set(c.gamma);
+  a.geo.set(c.dx, c.dy);
   a.in = in; a.base = base; a.out = out;
   a.lim_sl = nullptr;
   a.ctl = w.ctl;

@@ -16,6 +16,10 @@ struct BatchProb {
   int pad;
   long ncell;
   double dx, dy;
+  Geo2D<double> geo64;  // the constants of the cell in the kernel's arithmetic type
+  Geo2D<float> geo32;
+  __device__ __forceinline__ const Geo2D<double>& geo(double) const { return geo64; }
+  __device__ __forceinline__ const Geo2D<float>& geo(float) const { return geo32; }
   long c0_off, sl_off;
 };
 

@@ -250,6 +250,7 @@ cudaError_t launch_stage_t(dg_ctx* c, int stage, int in, int base, int out, doub
       a.dx = p.dx; a.dy = p.dy;
       a.gamma = c->gamma; a.cfl = c->cfl; a.dt_override = dtov; a.limiter = c->limiter;
       a.gas.set(c->gamma);
+      a.geo.set(p.dx, p.dy);
       a.in = sbuf<TS>(c, in, p);
       a.base = sbuf<TS>(c, base, p);
       a.out = sbuf<TS>(c, out, p);
@@ -266,6 +267,7 @@ cudaError_t launch_stage_t(dg_ctx* c, int stage, int in, int base, int out, doub
       a.dx = p.dx; a.dy = p.dy; a.dz = p.dz;
       a.gamma = c->gamma; a.cfl = c->cfl; a.dt_override = dtov; a.limiter = c->limiter;
       a.gas.set(c->gamma);
+      a.geo.set(p.dx, p.dy, p.dz);
       a.in = sbuf<TS>(c, in, p);
       a.base = sbuf<TS>(c, base, p);
       a.out = sbuf<TS>(c, out, p);
@@ -300,6 +302,7 @@ cudaError_t launch_mh_t(dg_ctx* c, int a, int b, double dtov) {
       s.dx = p.dx; s.dy = p.dy; s.dz = p.dz;
       s.gamma = c->gamma; s.cfl = c->cfl; s.dt_override = dtov; s.limiter = c->limiter;
       s.gas.set(c->gamma);
+      s.geo.set(p.dx, p.dy, p.dz);
       s.in = sbuf<TS>(c, a, p);
       s.base = s.in;
       s.out = sbuf<TS>(c, b, p);
@@ -315,6 +318,7 @@ cudaError_t launch_mh_t(dg_ctx* c, int a, int b, double dtov) {
     s.dx = p.dx; s.dy = p.dy;
     s.gamma = c->gamma; s.cfl = c->cfl; s.dt_override = dtov; s.limiter = c->limiter;
     s.gas.set(c->gamma);
+    s.geo.set(p.dx, p.dy);
     s.in = sbuf<TS>(c, a, p);
     s.base = s.in;
     s.out = sbuf<TS>(c, b, p);
@@ -652,6 +656,8 @@ dg_status build_batch(dg_ctx* c) {
       b.ncell = p.ncell;
       b.dx = p.dx;
       b.dy = p.dy;
+      b.geo64.set(p.dx, p.dy);
+      b.geo32.set(p.dx, p.dy);
       b.c0_off = (long)p.c0_off;
       b.sl_off = (long)p.sl_off;
       begin += b.ntiles;

@@ -48,6 +48,58 @@ template <class T> __device__ __forceinline__ const Gas<T>& gas_of(const GasPair
 template <> __device__ __forceinline__ const Gas<double>& gas_of<double>(const GasPair& g) { return g.d; }
 template <> __device__ __forceinline__ const Gas<float>& gas_of<float>(const GasPair& g) { return g.f; }
 
+// Geometry of a 2D cell and the constants of its right-hand side, formed once on the
+// host in FP64 (a division per thread and constant costs 8 to 10 instructions, on the
+// narrow pipe in FP64).
+template <class T>
+struct Geo2D {
+  T dx, dy;
+  T hx, hy;    // half cell sizes
+  T ox, oy;    // Gauss point offsets, d / (2 sqrt 3)
+  T ix, iy;    // 1/dx, 1/dy
+  T i2x, i2y;  // 1/(2 dx), 1/(2 dy)
+  T c3x, c3y;  // 3/dx^2, 3/dy^2
+  T r3;        // sqrt3/(dx dy)
+  T ax, ay;    // sqrt3/(dx^2+dy^2) * dy/dx, * dx/dy
+  __host__ void set(double x, double y) {
+    dx = T(x); dy = T(y);
+    hx = T(0.5 * x); hy = T(0.5 * y);
+    ox = T(x * 0.28867513459481288225); oy = T(y * 0.28867513459481288225);
+    ix = T(1.0 / x); iy = T(1.0 / y);
+    i2x = T(0.5 / x); i2y = T(0.5 / y);
+    c3x = T(3.0 / (x * x)); c3y = T(3.0 / (y * y));
+    r3 = T(1.7320508075688772935 / (x * y));
+    const double a = 1.7320508075688772935 / (x * x + y * y);
+    ax = T(a * (y / x)); ay = T(a * (x / y));
+  }
+};
+
+// The same for a 3D cell (indices: axis; e1, e2 the transverse axes of d in order).
+template <class T>
+struct Geo3D {
+  T h[3], hh[3], oo[3];  // cell size, half, Gauss point offset
+  T ih[3];               // 1/h
+  T c0[3];               // 1/(4 h_d)
+  T cs[3];               // 3/(2 h_d^2)
+  T ce[3][3];            // sqrt3/(2 h_e h_d)
+  // (a10, a11) = f[0..1] . (P, Q) and f[2..3] . (P, Q), with P = hx2 rxx - hy2 ryy and
+  // Q = hx2 rxx - hz2 rzz: the inverse of the coupled mass block
+  T h2[3], f[4];
+  __host__ void set(double x, double y, double z) {
+    const double d[3] = {x, y, z};
+    for (int a = 0; a < 3; ++a) {
+      h[a] = T(d[a]); hh[a] = T(0.5 * d[a]); oo[a] = T(d[a] * 0.28867513459481288225);
+      ih[a] = T(1.0 / d[a]);
+      c0[a] = T(0.25 / d[a]);
+      cs[a] = T(1.5 / (d[a] * d[a]));
+      h2[a] = T(d[a] * d[a]);
+      for (int e = 0; e < 3; ++e) ce[a][e] = T(0.86602540378443864676 / (d[e] * d[a]));
+    }
+    const double A = x * x + y * y, B = x * x + z * z, det = A * B - x * x * x * x;
+    f[0] = T(B / det); f[1] = T(-x * x / det); f[2] = T(-x * x / det); f[3] = T(A / det);
+  }
+};
+
 // Phase profiling of the stage kernels, compiled in only by the profiling build
 // (-DDG_PHASE_PROFILE; the normal build has no stamps).  Thread 0 of every CTA
 // stamps clock64() at the end of each phase -- after the barrier that closes it,
@@ -85,6 +137,7 @@ struct Stage2DArgs {
   double dx, dy;
   double gamma, cfl, dt_override;
   GasPair gas;
+  Geo2D<TS> geo;
   int limiter;
   StateBuf<TS> in;    // stage input (V^n in stage 1, V^1 in stage 2)
   StateBuf<TS> base;  // V^n (stage 2 only)
@@ -108,6 +161,7 @@ struct Stage3DArgs {
   double dx, dy, dz;
   double gamma, cfl, dt_override;
   GasPair gas;
+  Geo3D<TS> geo;
   int limiter;
   StateBuf<TS> in;
   StateBuf<TS> base;

@@ -115,7 +115,7 @@ __device__ __forceinline__ Dn<T, N> operator/(T a, const Dn<T, N>& b) {
 template <class T, int N>
 __device__ __forceinline__ Dn<T, N> dsqrt(const Dn<T, N>& a) {
   Dn<T, N> r;
-  r.v = rsqrtv(a.v);
+  r.v = sqrtv(a.v);
   T k = r.v > T(0) ? T(0.5) / r.v : T(0);
 #pragma unroll
   for (int i = 0; i < N; ++i) r.d[i] = a.d[i] * k;
@@ -159,6 +159,22 @@ __device__ __forceinline__ Dn<T, N>& operator+=(Dn<T, N>& a, const Dn<T, N>& b) 
 }
 template <class T, int N>
 __device__ __forceinline__ Dn<T, N> rsqrtv(const Dn<T, N>& a) { return dsqrt(a); }
+template <class T, int N>
+__device__ __forceinline__ Dn<T, N> sqrtv(const Dn<T, N>& a) { return dsqrt(a); }
+template <class T, int N>
+__device__ __forceinline__ Dn<T, N> rcpv(const Dn<T, N>& a) { return T(1) / a; }
+template <class T, int N>
+__device__ __forceinline__ Dn<T, N> rsqrtp(const Dn<T, N>& a) { return T(1) / dsqrt(a); }
+template <class T, int N>
+__device__ __forceinline__ bool posv(const Dn<T, N>& a) { return posv(a.v); }
+template <class T, int N>
+__device__ __forceinline__ bool negv(const Dn<T, N>& a) { return a.v < T(0); }
+template <class T, int N>
+__device__ __forceinline__ bool gt_pos(const Dn<T, N>& a, const Dn<T, N>& b) { return a.v > b.v; }
+template <class T, int N>
+struct Tiny<Dn<T, N>> {
+  static constexpr T v = Tiny<T>::v;
+};
 template <class T, int N>
 struct Prec<Dn<T, N>> {
   static constexpr T newton_tol = Prec<T>::newton_tol;

@@ -7,7 +7,7 @@
 // comparisons, exponents and tables from the integer pipe.
 //   rcpv     1/x: one cubically convergent step r (1 + e + e^2), e = 1 - x r, from the
 //            ~20-bit seed: 3 FP64 operations, within about 1 ulp.
-//   rsqrt64, sqrtv: one cubic (Householder) step y (1 + e/2 + 3e^2/8), e = 1 - x y^2:
+//   rsqrt64, sqrt64: one cubic (Householder) step y (1 + e/2 + 3e^2/8), e = 1 - x y^2:
 //            5 FP64 operations.
 //   pow_m1   x^z and x^z - 1 by log2 and exp2 with a table of 2^(i/64) and Taylor
 //            polynomials on the remainders (|ln| <= 0.0055): about 22 operations;
@@ -28,6 +28,44 @@ __device__ __forceinline__ bool posv(float x) { return x > 0.0f; }
 __device__ __forceinline__ bool gt_pos(double a, double b) {
   return __double_as_longlong(a) > __double_as_longlong(b);
 }
+__device__ __forceinline__ bool gt_pos(float a, float b) { return a > b; }
+
+// x < 0 by the sign bit (-0 counts as negative).
+__device__ __forceinline__ bool negv(double x) { return __double2hiint(x) < 0; }
+__device__ __forceinline__ bool negv(float x) { return x < 0.0f; }
+
+// Running maximum and minimum of a few values.  FP64 compares the integer images that
+// order like the doubles: no comparison on the FP64 pipe.
+template <class T>
+struct Extremes {
+  T hi, lo;
+  __device__ __forceinline__ explicit Extremes(T x) : hi(x), lo(x) {}
+  __device__ __forceinline__ void add(T x) {
+    hi = x > hi ? x : hi;
+    lo = x < lo ? x : lo;
+  }
+  __device__ __forceinline__ void add(T x, T y) { add(x); add(y); }
+  __device__ __forceinline__ T max() const { return hi; }
+  __device__ __forceinline__ T min() const { return lo; }
+};
+template <>
+struct Extremes<double> {
+  long long hi, lo;
+  __device__ __forceinline__ static long long image(long long b) {
+    return b ^ (long long)((unsigned long long)(b >> 63) >> 1);
+  }
+  __device__ __forceinline__ explicit Extremes(double x) {
+    hi = lo = image(__double_as_longlong(x));
+  }
+  __device__ __forceinline__ void add(double x) {
+    const long long k = image(__double_as_longlong(x));
+    hi = k > hi ? k : hi;
+    lo = k < lo ? k : lo;
+  }
+  __device__ __forceinline__ void add(double x, double y) { add(x); add(y); }
+  __device__ __forceinline__ double max() const { return __longlong_as_double(image(hi)); }
+  __device__ __forceinline__ double min() const { return __longlong_as_double(image(lo)); }
+};
 
 // The exponent of x is in [2, 2044]: neither x nor 1/x is zero, subnormal, infinite
 // or NaN, and the refinement of a seed is safe.
@@ -64,6 +102,63 @@ __device__ __forceinline__ double sqrt64(double x) {
   return refinable(x) ? s : x;
 }
 
+// FP32: three-operand minimum and maximum (a NaN operand is passed over, as by the
+// comparisons of the general form).
+template <>
+struct Extremes<float> {
+  float hi, lo;
+  __device__ __forceinline__ explicit Extremes(float x) { hi = lo = x; }
+  __device__ __forceinline__ void add(float x, float y) {
+    asm("max.f32 %0, %1, %2, %3;" : "=f"(hi) : "f"(hi), "f"(x), "f"(y));
+    asm("min.f32 %0, %1, %2, %3;" : "=f"(lo) : "f"(lo), "f"(x), "f"(y));
+  }
+  __device__ __forceinline__ float max() const { return hi; }
+  __device__ __forceinline__ float min() const { return lo; }
+};
+
+// The same operations of the FP32 path: one special-function instruction each (1 to 2
+// ulp).  The flushing forms leave out the scaling that subnormal operands would need
+// (3 more instructions a call): the averages are flushed when they are converted.
+__device__ __forceinline__ float rcpv(float x) {
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+}
+__device__ __forceinline__ float sqrtv(float x) {
+  float r;
+  asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+}
+__device__ __forceinline__ float rsqrtp(float x) {
+  float r;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+}
+__device__ __forceinline__ float ex2v(float x) {
+  float r;
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+}
+__device__ __forceinline__ float lg2v(float x) {
+  float r;
+  asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+}
+__device__ __forceinline__ double sqrtv(double x) { return sqrt64(x); }
+__device__ __forceinline__ double rsqrtp(double x) { return rsqrt64(x); }
+
+// The smallest normal number of a type: slopes below it count as zero.
+template <class T>
+struct Tiny;
+template <>
+struct Tiny<double> {
+  static constexpr double v = 2.2250738585072014e-308;
+};
+template <>
+struct Tiny<float> {
+  static constexpr float v = 1.17549435e-38f;
+};
+
 // 2^(i/64), i = 0 .. 64, rounded to FP64.
 __device__ const double kExp2Tab[65] = {
     0x1.0000000000000p+0, 0x1.02c9a3e778061p+0, 0x1.059b0d3158574p+0,
@@ -99,7 +194,7 @@ __device__ __forceinline__ double pow_m1(double x, double z, double& w) {
   const int hx = __double2hiint(x), lx = __double2loint(x);
   const int e = (hx >> 20) - 1023;
   const float m = __int_as_float(0x3f800000 | ((hx & 0x000fffff) << 3) | ((unsigned)lx >> 29));
-  int k = __float2int_rn(64.0f * __log2f(m));
+  int k = __float2int_rn(64.0f * lg2v(m));
   k = k < 0 ? 0 : (k > 64 ? 64 : k);
   const double h = __hiloint2double((hx & 0x000fffff) | 0x3fe00000, lx);
   const double r = fma(h, __ldg(&kExp2Tab[64 - k]), -1.0);

@@ -94,7 +94,7 @@ __device__ __forceinline__ void mh_grads2d(const Gas<TC>& G, const TC* hh, const
   }
   const bool limit = limiter != 0;
   const TC rho = W[0], vx = W[1], vy = W[2];
-  const TC inv = TC(1) / rho;
+  const TC inv = rcpv(rho);
   TC gr[2], gvx[2], gvy[2], gp[2], gbx[2], gby[2];
   if (EQ == 1) {
     gbx[0] = s[10]; gbx[1] = s[8];
@@ -115,14 +115,11 @@ __device__ __forceinline__ void mh_grads2d(const Gas<TC>& G, const TC* hh, const
     TC hi[NP], lo[NP];
 #pragma unroll
     for (int q = 0; q < NP; ++q) {
-      TC a = W[q], b = W[q];
+      Extremes<TC> ex(W[q]);
 #pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        a = Wn[k][q] > a ? Wn[k][q] : a;
-        b = Wn[k][q] < b ? Wn[k][q] : b;
-      }
-      hi[q] = a;
-      lo[q] = b;
+      for (int k = 0; k < 4; k += 2) ex.add(Wn[k][q], Wn[k + 1][q]);
+      hi[q] = ex.max();
+      lo[q] = ex.min();
     }
     ar = limiter_alpha<TC, 2>(W[0], hi[0], lo[0], gr, hh);
     avx = limiter_alpha<TC, 2>(W[1], hi[1], lo[1], gvx, hh);
@@ -160,7 +157,7 @@ __device__ __forceinline__ void mh_grads2d(const Gas<TC>& G, const TC* hh, const
 template <int EQ, class TC>
 __device__ __forceinline__ void mh_rates2d(const Gas<TC>& G, const TC* W, const TC* g, TC* Wt) {
   const TC rho = W[0], vx = W[1], vy = W[2], p = W[3];
-  const TC inv = TC(1) / rho;
+  const TC inv = rcpv(rho);
   const TC divv = g[2] + g[5];
   Wt[0] = -(vx * g[0] + vy * g[1]) - rho * divv;
   Wt[3] = -(vx * g[6] + vy * g[7]) - G.g * p * divv;
@@ -195,7 +192,7 @@ template <int EQ, class TC>
 __device__ __forceinline__ void prim_flux2d(const Gas<TC>& G, const TC* W, TC* Fx, TC* Fy,
                                             unsigned& err) {
   const TC rho = W[0], vx = W[1], vy = W[2], p = W[3];
-  if (!(rho > TC(0) && p > TC(0))) err |= ERR_NONPHYS;
+  if (!(posv(rho) && posv(p))) err |= ERR_NONPHYS;
   TC bx = TC(0), by = TC(0), b2h = TC(0);
   if (EQ == 1) { bx = W[4]; by = W[5]; b2h = TC(0.5) * (bx * bx + by * by); }
   const TC mx = rho * vx, my = rho * vy;
@@ -282,8 +279,8 @@ __device__ __forceinline__ void mh2d_compute(const Stage2DArgs<TS>& A, int i0, i
   }
   __syncthreads();
 
-  const TC dx = Cvt<TC>::to_tc(A.dx), dy = Cvt<TC>::to_tc(A.dy);
-  TC hh[2] = {TC(0.5) * dx, TC(0.5) * dy};
+  const Geo2D<TS>& geo = A.geo;
+  const TC hh[2] = {geo.hx, geo.hy};
 
   // ---- 2. gradients, limiter and half-step prediction on the tile and its ring
   for (int r1 = tid; r1 < R1; r1 += NT) {
@@ -310,7 +307,7 @@ __device__ __forceinline__ void mh2d_compute(const Stage2DArgs<TS>& A, int i0, i
   __syncthreads();  // the primitives are dead from here: their space takes the fluxes
 
   // ---- 3. faces: Riemann fluxes of the predicted states, each face once
-  const TC ox = dx * TC(0.28867513459481288225), oy = dy * TC(0.28867513459481288225);
+  const TC ox = geo.ox, oy = geo.oy;
   for (int e = tid; e < NGF * (NFX + NFY); e += NT) {
     const bool xf = e < NGF * NFX;
     const int ee = xf ? e : e - NGF * NFX;
@@ -381,9 +378,8 @@ __device__ __forceinline__ void mh2d_compute(const Stage2DArgs<TS>& A, int i0, i
       Dxm[q] = Dxp[q] = Dym[q] = Dyp[q] = TC(0);
     }
   }
-  const TC inv2dx = TC(0.5) / dx, inv2dy = TC(0.5) / dy;
-  const TC c3x = TC(3) / (dx * dx), c3y = TC(3) / (dy * dy);
-  const TC r3 = TC(1.7320508075688772935) / (dx * dy);
+  const TC inv2dx = geo.i2x, inv2dy = geo.i2y;
+  const TC c3x = geo.c3x, c3y = geo.c3y, r3 = geo.r3;
   TC rc0[NV], rs[NS];
 #pragma unroll
   for (int v = 0; v < 4; ++v) {
@@ -396,8 +392,7 @@ __device__ __forceinline__ void mh2d_compute(const Stage2DArgs<TS>& A, int i0, i
     rc0[5] = -(Sxp[4] - Sxm[4]) * inv2dx;
     rs[8] = c3y * (sFy[4] - (Syp[4] + Sym[4]));
     rs[9] = c3x * (sFx[4] - (Sxp[4] + Sxm[4]));
-    const TC ca3 = TC(1.7320508075688772935) / (dx * dx + dy * dy);
-    rs[10] = ca3 * ((dy / dx) * (Dxp[4] - Dxm[4]) - (dx / dy) * (Dyp[4] - Dym[4]));
+    rs[10] = geo.ax * (Dxp[4] - Dxm[4]) - geo.ay * (Dyp[4] - Dym[4]);
   }
 
   // U^{n+1} = U^n + dt L, U^n the limited step input
@@ -413,7 +408,7 @@ __device__ __forceinline__ void mh2d_compute(const Stage2DArgs<TS>& A, int i0, i
 #pragma unroll
     for (int k = 0; k < NS; ++k) A.out.sl[k * ncell + gc] = (TS)os[k];
   }
-  courant_commit2d<EQ, TC, TS, NT>(A, G, owner, o0, dx, dy, dt, nblk, err, S);
+  courant_commit2d<EQ, TC, TS, NT>(A, G, owner, o0, dt, nblk, err, S);
 }
 
 template <int EQ, class TC, class TS, int TX, int TY, int NGF, bool WENO>

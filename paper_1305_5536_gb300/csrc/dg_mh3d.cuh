@@ -53,7 +53,7 @@ __device__ __forceinline__ void mh_grads3d(const Gas<TC>& G, const TC* hh, const
     return;
   }
   const bool limit = limiter != 0;
-  const TC rho = W[0], inv = TC(1) / rho;
+  const TC rho = W[0], inv = rcpv(rho);
   const TC v[3] = {W[1], W[2], W[3]};
   const TC v2h = TC(0.5) * (v[0] * v[0] + v[1] * v[1] + v[2] * v[2]);
 #pragma unroll
@@ -70,13 +70,10 @@ __device__ __forceinline__ void mh_grads3d(const Gas<TC>& G, const TC* hh, const
   if (!limit) return;
 #pragma unroll
   for (int q = 0; q < 5; ++q) {
-    TC hi = W[q], lo = W[q];
+    Extremes<TC> ex(W[q]);
 #pragma unroll
-    for (int k = 0; k < 6; ++k) {
-      hi = Wn[k][q] > hi ? Wn[k][q] : hi;
-      lo = Wn[k][q] < lo ? Wn[k][q] : lo;
-    }
-    const TC a = limiter_alpha<TC, 3>(W[q], hi, lo, g + 3 * q, hh);
+    for (int k = 0; k < 6; k += 2) ex.add(Wn[k][q], Wn[k + 1][q]);
+    const TC a = limiter_alpha<TC, 3>(W[q], ex.max(), ex.min(), g + 3 * q, hh);
 #pragma unroll
     for (int d = 0; d < 3; ++d) g[3 * q + d] *= a;
   }
@@ -106,7 +103,7 @@ __device__ __forceinline__ void mh_cons3d(const Gas<TC>& G, const TC* W, const T
 
 template <class TC>
 __device__ __forceinline__ void mh_rates3d(const Gas<TC>& G, const TC* W, const TC* g, TC* Wt) {
-  const TC rho = W[0], inv = TC(1) / rho, p = W[4];
+  const TC rho = W[0], inv = rcpv(rho), p = W[4];
   const TC v[3] = {W[1], W[2], W[3]};
   const TC divv = g[3] + g[7] + g[11];
   Wt[0] = -(v[0] * g[0] + v[1] * g[1] + v[2] * g[2]) - rho * divv;
@@ -132,7 +129,7 @@ template <class TC>
 __device__ __forceinline__ void prim_flux3d(const Gas<TC>& G, const TC* W, int d, TC* F,
                                             unsigned& err) {
   const TC rho = W[0], p = W[4];
-  if (!(rho > TC(0) && p > TC(0))) err |= ERR_NONPHYS;
+  if (!(posv(rho) && posv(p))) err |= ERR_NONPHYS;
   const TC m[3] = {rho * W[1], rho * W[2], rho * W[3]};
   const TC vd = W[1 + d];
   const TC E = p * G.inv_gm1 + TC(0.5) * (m[0] * W[1] + m[1] * W[2] + m[2] * W[3]);
@@ -165,9 +162,8 @@ __device__ __forceinline__ void face_flux_prim3d(const Gas<TC>& G, int d, const 
 // side (gather3d with four equal Gauss-point fluxes) for NV variables.
 template <int D, class TC, int NV = 5>
 __device__ __forceinline__ void gather3d_centroid(const TC* s_f, int FMAX, int fm, int fp,
-                                                  const TC* hd, TC* rc0, TC* rs) {
-  const TC c0f = TC(1) / hd[D];
-  const TC csf = TC(6) / (hd[D] * hd[D]);
+                                                  const Geo3D<TC>& geo, TC* rc0, TC* rs) {
+  const TC c0f = geo.ih[D], csf = TC(4) * geo.cs[D];
 #pragma unroll
   for (int v = 0; v < NV; ++v) {
     const TC m = s_f[v * FMAX + fm], p = s_f[v * FMAX + fp];
@@ -239,11 +235,9 @@ __global__ void __launch_bounds__(TX * TY * TZ) mh3d_kernel(const Stage3DArgs<TS
   cp_async_wait_all();
   __syncthreads();
 
-  const TC dx = Cvt<TC>::to_tc(A.dx), dy = Cvt<TC>::to_tc(A.dy), dz = Cvt<TC>::to_tc(A.dz);
-  const TC hh[3] = {TC(0.5) * dx, TC(0.5) * dy, TC(0.5) * dz};
-  const TC oo[3] = {dx * TC(0.28867513459481288225), dy * TC(0.28867513459481288225),
-                    dz * TC(0.28867513459481288225)};
-  const TC hd[3] = {dx, dy, dz};
+  const Geo3D<TS>& geo = A.geo;
+  const TC hh[3] = {geo.hh[0], geo.hh[1], geo.hh[2]};
+  const TC oo[3] = {geo.oo[0], geo.oo[1], geo.oo[2]};
 
   // ---- 2. gradients, limiter, half-step prediction on the halo-1 box
   for (int r1 = tid; r1 < R1; r1 += NT) {
@@ -300,7 +294,7 @@ __global__ void __launch_bounds__(TX * TY * TZ) mh3d_kernel(const Stage3DArgs<TS
 #pragma unroll
     for (int v = 0; v < 5; ++v)
 #pragma unroll
-      for (int d = 0; d < 3; ++d) rs[3 * v + d] = TC(1.5) / (hd[d] * hd[d]) * sF[d][v];
+      for (int d = 0; d < 3; ++d) rs[3 * v + d] = geo.cs[d] * sF[d][v];
   }
 
   // ---- 4. faces, one orientation at a time (rolled loop: one copy of the solver)
@@ -338,13 +332,13 @@ __global__ void __launch_bounds__(TX * TY * TZ) mh3d_kernel(const Stage3DArgs<TS
       const int fm = (lz * FY + ly) * FX + lx;
       const int fp = fm + (d == 0 ? 1 : (d == 1 ? FX : FX * FY));
       if (NPT == 4) {
-        if (d == 0) gather3d<0, TC>(s_f, FMAX, fm, fp, hd, rc0, rs);
-        else if (d == 1) gather3d<1, TC>(s_f, FMAX, fm, fp, hd, rc0, rs);
-        else gather3d<2, TC>(s_f, FMAX, fm, fp, hd, rc0, rs);
+        if (d == 0) gather3d<0, TC>(s_f, FMAX, fm, fp, geo, rc0, rs);
+        else if (d == 1) gather3d<1, TC>(s_f, FMAX, fm, fp, geo, rc0, rs);
+        else gather3d<2, TC>(s_f, FMAX, fm, fp, geo, rc0, rs);
       } else {
-        if (d == 0) gather3d_centroid<0, TC>(s_f, FMAX, fm, fp, hd, rc0, rs);
-        else if (d == 1) gather3d_centroid<1, TC>(s_f, FMAX, fm, fp, hd, rc0, rs);
-        else gather3d_centroid<2, TC>(s_f, FMAX, fm, fp, hd, rc0, rs);
+        if (d == 0) gather3d_centroid<0, TC>(s_f, FMAX, fm, fp, geo, rc0, rs);
+        else if (d == 1) gather3d_centroid<1, TC>(s_f, FMAX, fm, fp, geo, rc0, rs);
+        else gather3d_centroid<2, TC>(s_f, FMAX, fm, fp, geo, rc0, rs);
       }
     }
     __syncthreads();
@@ -386,8 +380,9 @@ __global__ void __launch_bounds__(TX * TY * TZ) mh3d_kernel(const Stage3DArgs<TS
 #pragma unroll
     for (int v = 0; v < 5; ++v) c[v] = Cvt<TC>::to_tc(o0[v]);
     prims3d<TC>(G, c, W, err);
-    TC cs = sqrt(G.g * W[4] / W[0]);
-    sp = (fabs(W[1]) + cs) / dx + (fabs(W[2]) + cs) / dy + (fabs(W[3]) + cs) / dz;
+    TC cs = sqrtv(G.g * W[4] * rcpv(W[0]));
+    sp = (fabs(W[1]) + cs) * geo.ih[0] + (fabs(W[2]) + cs) * geo.ih[1] +
+         (fabs(W[3]) + cs) * geo.ih[2];
     if (!courant_ok(sp, W[0], W[4])) { err |= ERR_NONPHYS; sp = TC(0); }
   }
 #pragma unroll

@@ -49,7 +49,7 @@ __host__ __device__ constexpr size_t mh3m_smem_bytes() {
 template <class TC>
 __device__ __forceinline__ void prim_grads3m(const Gas<TC>& G, const TC* W, const TC* s,
                                              const TC (*gB)[3], TC* g) {
-  const TC rho = W[0], inv = TC(1) / rho;
+  const TC rho = W[0], inv = rcpv(rho);
   const TC v[3] = {W[1], W[2], W[3]};
   const TC v2h = TC(0.5) * (v[0] * v[0] + v[1] * v[1] + v[2] * v[2]);
 #pragma unroll
@@ -95,7 +95,7 @@ __device__ __forceinline__ void mh_cons3m(const Gas<TC>& G, const TC* W, const T
 template <class TC>
 __device__ __forceinline__ void mh_rates3m(const Gas<TC>& G, const TC* W, const TC* g,
                                            const TC (*gB)[3], TC* Wt) {
-  const TC rho = W[0], inv = TC(1) / rho, p = W[4];
+  const TC rho = W[0], inv = rcpv(rho), p = W[4];
   const TC v[3] = {W[1], W[2], W[3]};
   const TC B[3] = {W[5], W[6], W[7]};
   const TC divv = g[3] + g[7] + g[11];
@@ -135,7 +135,7 @@ template <class TC>
 __device__ __forceinline__ void prim_flux3m(const Gas<TC>& G, const TC* W, int d, TC* F,
                                             unsigned& err) {
   const TC rho = W[0], p = W[4];
-  if (!(rho > TC(0) && p > TC(0))) err |= ERR_NONPHYS;
+  if (!(posv(rho) && posv(p))) err |= ERR_NONPHYS;
   const TC v[3] = {W[1], W[2], W[3]};
   const TC B[3] = {W[5], W[6], W[7]};
   const TC b2h = TC(0.5) * (B[0] * B[0] + B[1] * B[1] + B[2] * B[2]);
@@ -216,11 +216,9 @@ __global__ void __launch_bounds__(TX * TY * TZ) mh3m_kernel(const Stage3DArgs<TS
   cp_async_wait_all();
   __syncthreads();
 
-  const TC dx = Cvt<TC>::to_tc(A.dx), dy = Cvt<TC>::to_tc(A.dy), dz = Cvt<TC>::to_tc(A.dz);
-  const TC hh[3] = {TC(0.5) * dx, TC(0.5) * dy, TC(0.5) * dz};
-  const TC oo[3] = {dx * TC(0.28867513459481288225), dy * TC(0.28867513459481288225),
-                    dz * TC(0.28867513459481288225)};
-  const TC hd[3] = {dx, dy, dz};
+  const Geo3D<TS>& geo = A.geo;
+  const TC hh[3] = {geo.hh[0], geo.hh[1], geo.hh[2]};
+  const TC oo[3] = {geo.oo[0], geo.oo[1], geo.oo[2]};
 
   // ---- 2. limiter, primitive gradients, half-step prediction on the halo-1 box
   for (int r1 = tid; r1 < R1; r1 += NT) {
@@ -275,7 +273,7 @@ __global__ void __launch_bounds__(TX * TY * TZ) mh3m_kernel(const Stage3DArgs<TS
     for (int d = 0; d < 3; ++d) {
       TC F[8];
       prim_flux3m<TC>(G, W, d, F, err);
-      const TC w = TC(1.5) / (hd[d] * hd[d]);
+      const TC w = geo.cs[d];
 #pragma unroll
       for (int v = 0; v < 8; ++v) rs[3 * v + d] += w * F[v];
     }
@@ -318,25 +316,25 @@ __global__ void __launch_bounds__(TX * TY * TZ) mh3m_kernel(const Stage3DArgs<TS
       const TC* s_fb = s_f + 5 * FMAX * NPT;  // the three field components
       if (NPT == 4) {
         if (d == 0) {
-          gather3d<0, TC>(s_f, FMAX, fm, fp, hd, rc0, rs);
-          gather3d<0, TC, 3>(s_fb, FMAX, fm, fp, hd, rc0 + 5, rs + 15);
+          gather3d<0, TC>(s_f, FMAX, fm, fp, geo, rc0, rs);
+          gather3d<0, TC, 3>(s_fb, FMAX, fm, fp, geo, rc0 + 5, rs + 15);
         } else if (d == 1) {
-          gather3d<1, TC>(s_f, FMAX, fm, fp, hd, rc0, rs);
-          gather3d<1, TC, 3>(s_fb, FMAX, fm, fp, hd, rc0 + 5, rs + 15);
+          gather3d<1, TC>(s_f, FMAX, fm, fp, geo, rc0, rs);
+          gather3d<1, TC, 3>(s_fb, FMAX, fm, fp, geo, rc0 + 5, rs + 15);
         } else {
-          gather3d<2, TC>(s_f, FMAX, fm, fp, hd, rc0, rs);
-          gather3d<2, TC, 3>(s_fb, FMAX, fm, fp, hd, rc0 + 5, rs + 15);
+          gather3d<2, TC>(s_f, FMAX, fm, fp, geo, rc0, rs);
+          gather3d<2, TC, 3>(s_fb, FMAX, fm, fp, geo, rc0 + 5, rs + 15);
         }
       } else {
         if (d == 0) {
-          gather3d_centroid<0, TC>(s_f, FMAX, fm, fp, hd, rc0, rs);
-          gather3d_centroid<0, TC, 3>(s_fb, FMAX, fm, fp, hd, rc0 + 5, rs + 15);
+          gather3d_centroid<0, TC>(s_f, FMAX, fm, fp, geo, rc0, rs);
+          gather3d_centroid<0, TC, 3>(s_fb, FMAX, fm, fp, geo, rc0 + 5, rs + 15);
         } else if (d == 1) {
-          gather3d_centroid<1, TC>(s_f, FMAX, fm, fp, hd, rc0, rs);
-          gather3d_centroid<1, TC, 3>(s_fb, FMAX, fm, fp, hd, rc0 + 5, rs + 15);
+          gather3d_centroid<1, TC>(s_f, FMAX, fm, fp, geo, rc0, rs);
+          gather3d_centroid<1, TC, 3>(s_fb, FMAX, fm, fp, geo, rc0 + 5, rs + 15);
         } else {
-          gather3d_centroid<2, TC>(s_f, FMAX, fm, fp, hd, rc0, rs);
-          gather3d_centroid<2, TC, 3>(s_fb, FMAX, fm, fp, hd, rc0 + 5, rs + 15);
+          gather3d_centroid<2, TC>(s_f, FMAX, fm, fp, geo, rc0, rs);
+          gather3d_centroid<2, TC, 3>(s_fb, FMAX, fm, fp, geo, rc0 + 5, rs + 15);
         }
       }
     }
@@ -345,7 +343,7 @@ __global__ void __launch_bounds__(TX * TY * TZ) mh3m_kernel(const Stage3DArgs<TS
   TC rsl[23];
 #pragma unroll
   for (int k = 0; k < 15; ++k) rsl[k] = rs[k];
-  field_rhs3m<TC>(rs, hd, rsl + 15);
+  field_rhs3m<TC>(rs, geo, rsl + 15);
 
   // ---- 5. update of the limited coefficients, Courant speed of the new state
   const int gi = i0 + lx, gj = j0 + ly, gk = k0 + lz;
@@ -387,9 +385,9 @@ __global__ void __launch_bounds__(TX * TY * TZ) mh3m_kernel(const Stage3DArgs<TS
     for (int v = 0; v < 8; ++v) c[v] = Cvt<TC>::to_tc(o0[v]);
     prims3m<TC>(G, c, W, err);
     const TC b2 = W[5] * W[5] + W[6] * W[6] + W[7] * W[7];
-    sp = (fabs(W[1]) + fast_speed(G, W[0], W[4], b2, W[5])) / dx +
-         (fabs(W[2]) + fast_speed(G, W[0], W[4], b2, W[6])) / dy +
-         (fabs(W[3]) + fast_speed(G, W[0], W[4], b2, W[7])) / dz;
+    sp = (fabs(W[1]) + fast_speed(G, W[0], W[4], b2, W[5])) * geo.ih[0] +
+         (fabs(W[2]) + fast_speed(G, W[0], W[4], b2, W[6])) * geo.ih[1] +
+         (fabs(W[3]) + fast_speed(G, W[0], W[4], b2, W[7])) * geo.ih[2];
     if (!courant_ok(sp, W[0], W[4])) { err |= ERR_NONPHYS; sp = TC(0); }
   }
 #pragma unroll

@@ -163,16 +163,19 @@ struct Gas<double> : GasConst<double> {
   }
 };
 
-// Fast magnetosonic speed along a direction with normal field bn.
+// Square of the fast magnetosonic speed along a direction with normal field bn; ir =
+// 1/rho.
+template <class T>
+__device__ __forceinline__ T fast_speed2(const Gas<T>& G, T ir, T p, T b2, T bn) {
+  const T a2 = G.g * p * ir;
+  const T s = a2 + b2 * ir;
+  T disc = s * s - T(4) * a2 * (bn * bn * ir);
+  disc = negv(disc) ? T(0) : disc;
+  return T(0.5) * (s + sqrtv(disc));
+}
 template <class T>
 __device__ __forceinline__ T fast_speed(const Gas<T>& G, T rho, T p, T b2, T bn) {
-  T a2 = G.g * p / rho;
-  T bb = b2 / rho;
-  T bn2 = bn * bn / rho;
-  T s = a2 + bb;
-  T disc = s * s - T(4) * a2 * bn2;
-  disc = disc < T(0) ? T(0) : disc;
-  return rsqrtv(T(0.5) * (s + rsqrtv(disc)));
+  return sqrtv(fast_speed2(G, rcpv(rho), p, b2, bn));
 }
 
 // ----------------------------------------------------------------------------
@@ -271,8 +274,6 @@ __device__ __forceinline__ T exact_pstar(const Gas<T>& G, T rL, T uL, T pL, T cL
 //     rarefaction-star choice is a select; only the transonic rarefaction fan,
 //     which is rare, is a branch.
 // ----------------------------------------------------------------------------
-__device__ __forceinline__ float rcpf(float x) { return __fdividef(1.0f, x); }
-__device__ __forceinline__ float sqrtf_pos(float x) { return x * rsqrtf(x); }  // x > 0
 
 // The first guess and Newton iteration above: p* and the last linearisation, taken at
 // p0 (f_K, f_K' there).
@@ -296,23 +297,23 @@ __device__ __forceinline__ Star32 star_f32(const GasConst<float>& G, float rL, f
   if (!(pmax <= 2.0f * pmin && pmin <= pv && pv <= pmax)) {
     if (pv < pmin) {  // two rarefactions
       const float num = fmaxf(cL + cR - 0.5f * G.gm1 * du, 0.0f);
-      const float den = cL * exp2f(-G.z * __log2f(pL)) + cR * exp2f(-G.z * __log2f(pR));
-      p = exp2f(G.inv_z * __log2f(num * rcpf(den)));
+      const float den = cL * ex2v(-G.z * lg2v(pL)) + cR * ex2v(-G.z * lg2v(pR));
+      p = ex2v(G.inv_z * lg2v(num * rcpv(den)));
     } else {  // two shocks
-      const float gL = rsqrtf((BL + pv) * AiL), gR = rsqrtf((BR + pv) * AiR);
-      p = (gL * pL + gR * pR - du) * rcpf(gL + gR);
+      const float gL = rsqrtp((BL + pv) * AiL), gR = rsqrtp((BR + pv) * AiR);
+      p = (gL * pL + gR * pR - du) * rcpv(gL + gR);
     }
   }
   const float pfloor = 1e-10f * pmin;
   if (!(p > pfloor)) p = pfloor;
   Star32 S = {p, p, 0.0f, 0.0f, 1.0f, 1.0f, false};
   for (int it = 0; it < Prec<float>::newton_max; ++it) {
-    const float rp = rcpf(p);
+    const float rp = rcpv(p);
     {
       const float dp = p - pL;
-      const float q = rsqrtf((p + BL) * AiL);
+      const float q = rsqrtp((p + BL) * AiL);
       const float fs = dp * q, dfs = q * (1.0f - 0.5f * dp * q * q * AiL);
-      const float qr = exp2f(G.z * __log2f(p * ipL));
+      const float qr = ex2v(G.z * lg2v(p * ipL));
       const float fr = CL * (qr - 1.0f), dfr = qr * DL * rp;
       const bool sh = p > pL;
       S.fL = sh ? fs : fr;
@@ -320,15 +321,15 @@ __device__ __forceinline__ Star32 star_f32(const GasConst<float>& G, float rL, f
     }
     {
       const float dp = p - pR;
-      const float q = rsqrtf((p + BR) * AiR);
+      const float q = rsqrtp((p + BR) * AiR);
       const float fs = dp * q, dfs = q * (1.0f - 0.5f * dp * q * q * AiR);
-      const float qr = exp2f(G.z * __log2f(p * ipR));
+      const float qr = ex2v(G.z * lg2v(p * ipR));
       const float fr = CR * (qr - 1.0f), dfr = qr * DR * rp;
       const bool sh = p > pR;
       S.fR = sh ? fs : fr;
       S.dfR = sh ? dfs : dfr;
     }
-    float pn = p - (S.fL + S.fR + du) * rcpf(S.dfL + S.dfR);
+    float pn = p - (S.fL + S.fR + du) * rcpv(S.dfL + S.dfR);
     if (!(pn > pfloor)) pn = pfloor;
     S.p0 = p;
     const bool done = 2.0f * fabsf(pn - p) < accept * (pn + p);
@@ -348,9 +349,9 @@ __device__ __forceinline__ void exact_flux_f32(const Gas<float>& G, float rL, fl
     for (int q = 0; q < 3 + NT; ++q) F[q] = 0.0f;
     return;
   }
-  const float ipL = rcpf(pL), ipR = rcpf(pR);
-  const float aL = G.g * pL * rcpf(rL), aR = G.g * pR * rcpf(rR);
-  const float cL = sqrtf_pos(aL), cR = sqrtf_pos(aR);
+  const float ipL = rcpv(pL), ipR = rcpv(pR);
+  const float aL = G.g * pL * rcpv(rL), aR = G.g * pR * rcpv(rR);
+  const float cL = sqrtv(aL), cR = sqrtv(aR);
   const float du = uR - uL;
   if (G.two_gm1 * cL + G.two_gm1 * cR <= du) err |= ERR_VACUUM;
   const Star32 S = star_f32(G, rL, pL, ipL, cL, rR, pR, ipR, cR, du);
@@ -368,11 +369,11 @@ __device__ __forceinline__ void exact_flux_f32(const Gas<float>& G, float rL, fl
   const float w = sg * (left ? uL : uR), ws = sg * us;
   const float pr = p * ipK;
   const bool shock = p > pK;
-  const float Ssh = w - cK * sqrtf_pos(G.shk1 * pr + G.z);         // shock speed
-  const float rsh = rK * (pr + G.g6) * rcpf(G.g6 * pr + 1.0f);      // behind the shock
-  const float lpr = __log2f(pr);
-  const float cm = cK * exp2f(G.z * lpr);                           // sound speed behind the fan
-  const float rrf = rK * exp2f(G.inv_g * lpr);                      // isentropic star density
+  const float Ssh = w - cK * sqrtv(G.shk1 * pr + G.z);         // shock speed
+  const float rsh = rK * (pr + G.g6) * rcpv(G.g6 * pr + 1.0f);      // behind the shock
+  const float lpr = lg2v(pr);
+  const float cm = cK * ex2v(G.z * lpr);                           // sound speed behind the fan
+  const float rrf = rK * ex2v(G.inv_g * lpr);                      // isentropic star density
   const bool unpert = shock ? Ssh >= 0.0f : w - cK >= 0.0f;
   const bool fan = !shock && !unpert && !(ws - cm < 0.0f);
   float rho = unpert ? rK : (shock ? rsh : rrf);
@@ -380,10 +381,10 @@ __device__ __forceinline__ void exact_flux_f32(const Gas<float>& G, float rL, fl
   float pp = unpert ? pK : p;
   if (fan) {
     const float c = G.two_gp1 * (cK + 0.5f * G.gm1 * w);
-    const float lc = __log2f(c * rcpf(cK));
+    const float lc = lg2v(c * rcpv(cK));
     u = c;
-    rho = rK * exp2f(G.two_gm1 * lc);
-    pp = pK * exp2f(G.inv_z * lc);
+    rho = rK * ex2v(G.two_gm1 * lc);
+    pp = pK * ex2v(G.inv_z * lc);
   }
   u *= sg;
   float vt[NT > 0 ? NT : 1];
@@ -418,9 +419,9 @@ __device__ __forceinline__ void exact_flux_f32(const Gas<float>& G, float rL, fl
 // evaluations, a re-evaluation and the sampling).
 // ----------------------------------------------------------------------------
 // Pressure function of one side at p: f, f' and, for p <= pK, w = (p/pK)^z (0 where the
-// side is a shock at p).
+// side is a shock at p); x = p/pK.
 __device__ __forceinline__ void side_f64(const Gas<double>& G, double p, double ip, double rK,
-                                         double pK, double ipK, double cK, double& f, double& df,
+                                         double pK, double x, double cK, double& f, double& df,
                                          double& w) {
   if (gt_pos(p, pK)) {
     const double Ai = (0.5 * G.gp1) * rK, dp = p - pK;  // 1 / A_K
@@ -429,18 +430,18 @@ __device__ __forceinline__ void side_f64(const Gas<double>& G, double p, double 
     df = fma(-0.5 * f, q * q * Ai, q);
     w = 0.0;
   } else {
-    const double wm1 = pow_m1(p * ipK, G.z, w);
+    const double wm1 = pow_m1(x, G.z, w);
     f = (G.two_gm1 * cK) * wm1;
     df = (cK * G.inv_g) * (w * ip);
   }
 }
 
-// f''/f' of one side at p, times p (FP32).
-__device__ __forceinline__ float curvature_f32(const GasConst<float>& G, float p, float pK) {
-  const float B = G.g6 * pK;
-  const float sh = -0.25f * p * (4.0f * B + 3.0f * p + pK) *
-                   rcpf((p + B) * (0.5f * (p + pK) + B));
-  return p > pK ? sh : -G.shk1;
+// p f''/f' of one side at x = p/pK (FP32).
+__device__ __forceinline__ float curvature_f32(const GasConst<float>& G, float x) {
+  const float B = G.g6;
+  const float sh = -0.25f * x * (4.0f * B + 3.0f * x + 1.0f) *
+                   rcpv((x + B) * (0.5f * (x + 1.0f) + B));
+  return x > 1.0f ? sh : -G.shk1;
 }
 
 struct Star64 {
@@ -454,8 +455,8 @@ __device__ __forceinline__ Star64 star_f64(const Gas<double>& G, double rL, doub
                                            double du, unsigned& err) {
   const GasConst<float>& H = G.lo;
   const float pLf = Cvt<float>::to_tc(pL), pRf = Cvt<float>::to_tc(pR);
-  const Star32 S = star_f32(H, Cvt<float>::to_tc(rL), pLf, rcpf(pLf), Cvt<float>::to_tc(cL),
-                            Cvt<float>::to_tc(rR), pRf, rcpf(pRf), Cvt<float>::to_tc(cR),
+  const Star32 S = star_f32(H, Cvt<float>::to_tc(rL), pLf, rcpv(pLf), Cvt<float>::to_tc(cL),
+                            Cvt<float>::to_tc(rR), pRf, rcpv(pRf), Cvt<float>::to_tc(cR),
                             Cvt<float>::to_tc(du));
   const double pfloor = 1e-10 * (gt_pos(pR, pL) ? pL : pR);
   double p = Cvt<double>::to_tc(Cvt<float>::to_f64(S.p));
@@ -466,14 +467,17 @@ __device__ __forceinline__ Star64 star_f64(const Gas<double>& G, double rL, doub
   for (int it = 0; it < Prec<double>::newton_max; ++it) {
     const double ip = rcpv(p);
     double fL, dfL, fR, dfR;
-    side_f64(G, p, ip, rL, pL, ipL, cL, fL, dfL, R.wL);
-    side_f64(G, p, ip, rR, pR, ipR, cR, fR, dfR, R.wR);
+    const double xL = p * ipL, xR = p * ipR;
+    side_f64(G, p, ip, rL, pL, xL, cL, fL, dfL, R.wL);
+    side_f64(G, p, ip, rR, pR, xR, cR, fR, dfR, R.wR);
     // relative Newton step, then Halley's correction 1 / (1 + step H), H = p f''/(2 f')
-    double x = -(fL + fR + du) * rcpv(dfL + dfR) * ip;
-    const float xf = Cvt<float>::to_tc(x), pf = Cvt<float>::to_tc(p);
-    const float dLf = Cvt<float>::to_tc(dfL), dRf = Cvt<float>::to_tc(dfR);
-    const float kL = dLf * curvature_f32(H, pf, pLf), kR = dRf * curvature_f32(H, pf, pRf);
-    float c = xf * 0.5f * (kL + kR) * rcpf(dLf + dRf);
+    const double dS = dfL + dfR, idS = rcpv(dS);
+    double x = -(fL + fR + du) * idS * ip;
+    const float xf = Cvt<float>::to_tc(x);
+    const float tL = Cvt<float>::to_tc(dfL * idS), tR = 1.0f - tL;  // shares of f'
+    const float kL = tL * curvature_f32(H, Cvt<float>::to_tc(xL));
+    const float kR = tR * curvature_f32(H, Cvt<float>::to_tc(xR));
+    float c = xf * 0.5f * (kL + kR);
     if (!(fabsf(c) < 0.05f)) c = 0.0f;
     x = fma(-x, Cvt<float>::to_f64(c), x);
     double pn = fma(p, x, p);
@@ -482,7 +486,7 @@ __device__ __forceinline__ Star64 star_f64(const Gas<double>& G, double rL, doub
     R.step = x;
     const double d = pn - p;
     // second order of f_R - f_L: p f'' d x / 2
-    R.uj = fma(d, fma(0.5 * Cvt<float>::to_f64(kR - kL), x, dfR - dfL), fR - fL);
+    R.uj = fma(d, fma(dS * Cvt<float>::to_f64(0.5f * (kR - kL)), x, dfR - dfL), fR - fL);
     p = pn;
     if (fabsf(xf) < 2e-6f) { conv = true; break; }
   }
@@ -527,7 +531,7 @@ __device__ __forceinline__ void exact_flux_f64(const Gas<double>& G, double rL, 
   double q = 1.0;  // (p/pK)^z at p*
   if (shock) {
     const float cf = Cvt<float>::to_tc(cK);
-    const float s = Cvt<float>::to_tc(w) - cf * sqrtf_pos(G.lo.shk1 * Cvt<float>::to_tc(x) + G.lo.z);
+    const float s = Cvt<float>::to_tc(w) - cf * sqrtv(G.lo.shk1 * Cvt<float>::to_tc(x) + G.lo.z);
     unpert = s >= 0.0f;
     if (!(fabsf(s) > 1e-4f * cf)) unpert = w - cK * sqrt64(fma(G.shk1, x, G.z)) >= 0.0;
   } else {
@@ -579,229 +583,159 @@ __device__ __forceinline__ void exact_flux(const Gas<T>& G, T rL, T uL, T pL, co
 }
 
 // ----------------------------------------------------------------------------
-// HLLD solver, planar MHD (one transverse velocity v and field bt; out-of-plane
-// components are zero).  bn is the common normal field.  Output in the face
-// frame: F[0] mass, F[1] normal momentum, F[2] transverse momentum, F[3] energy,
-// F[4] flux of the transverse field (the normal-field flux is zero).
+// HLLD solver with NT transverse components (1: planar MHD, 2: 3D MHD): per side
+// (rho, u, p) with u normal, v[] and bt[] the transverse velocity and field; bn the
+// common normal field.  Output in the face frame: F[0] mass, F[1] normal momentum,
+// F[2 ..] transverse momenta, F[2+NT] energy, F[3+NT ..] transverse field fluxes (the
+// normal-field flux is zero).
+//
+// The flux is that of one state, evaluated once: the outer state of side K, or its
+// single- or double-star state with the normal velocity SM and the total pressure of
+// the star region (K the side of the contact that x/t = 0 lies on).  By the solver's
+// own jump relations this equals F_K + S_K (U*_K - U_K) + S*_K (U**_K - U*_K), without
+// forming the four vectors of both sides.  On a degenerate side, where the transverse
+// star state is set equal to the outer one, the field flux of that sum differs by
+// bt (u_K - SM), which is added.
 // ----------------------------------------------------------------------------
-template <class T>
-__device__ __forceinline__ void hlld_flux(const Gas<T>& G, T rL, T uL, T vL, T pL, T btL, T rR,
-                                          T uR, T vR, T pR, T btR, T bn, T* F, unsigned& err) {
-  if (!(rL > T(0) && pL > T(0) && rR > T(0) && pR > T(0))) {
+template <class T, int NT>
+__device__ __forceinline__ void hlld_core(const Gas<T>& G, T rL, T uL, const T* vL, T pL,
+                                          const T* btL, T rR, T uR, const T* vR, T pR,
+                                          const T* btR, T bn, T* F, unsigned& err) {
+  if (!(posv(rL) && posv(pL) && posv(rR) && posv(pR))) {
     err |= ERR_NONPHYS;
-    for (int q = 0; q < 5; ++q) F[q] = T(0);
+    for (int q = 0; q < 3 + 2 * NT; ++q) F[q] = T(0);
     return;
   }
   const T bn2 = bn * bn;
-  const T b2L = bn2 + btL * btL, b2R = bn2 + btR * btR;
-  const T EL = pL * G.inv_gm1 + T(0.5) * rL * (uL * uL + vL * vL) + T(0.5) * b2L;
-  const T ER = pR * G.inv_gm1 + T(0.5) * rR * (uR * uR + vR * vR) + T(0.5) * b2R;
+  T b2L = bn2, b2R = bn2;
+#pragma unroll
+  for (int a = 0; a < NT; ++a) {
+    b2L += btL[a] * btL[a];
+    b2R += btR[a] * btR[a];
+  }
   const T pTL = pL + T(0.5) * b2L, pTR = pR + T(0.5) * b2R;
-  const T cfL = fast_speed(G, rL, pL, b2L, bn), cfR = fast_speed(G, rR, pR, b2R, bn);
-  const T cmax = cfL > cfR ? cfL : cfR;
-  const T SL = (uL < uR ? uL : uR) - cmax;
-  const T SR = (uL < uR ? uR : uL) + cmax;
-  // physical fluxes and conserved vectors of both sides
-  T FL[5], FR[5], UL[5], UR[5];
-  {
-    T vB = uL * bn + vL * btL;
-    FL[0] = rL * uL; FL[1] = rL * uL * uL + pTL - bn2; FL[2] = rL * uL * vL - bn * btL;
-    FL[3] = (EL + pTL) * uL - bn * vB; FL[4] = btL * uL - vL * bn;
-    UL[0] = rL; UL[1] = rL * uL; UL[2] = rL * vL; UL[3] = EL; UL[4] = btL;
-    vB = uR * bn + vR * btR;
-    FR[0] = rR * uR; FR[1] = rR * uR * uR + pTR - bn2; FR[2] = rR * uR * vR - bn * btR;
-    FR[3] = (ER + pTR) * uR - bn * vB; FR[4] = btR * uR - vR * bn;
-    UR[0] = rR; UR[1] = rR * uR; UR[2] = rR * vR; UR[3] = ER; UR[4] = btR;
-  }
-  if (SL > T(0)) {
-    for (int q = 0; q < 5; ++q) F[q] = FL[q];
-    return;
-  }
-  if (SR < T(0)) {
-    for (int q = 0; q < 5; ++q) F[q] = FR[q];
-    return;
-  }
+  const T c2L = fast_speed2(G, rcpv(rL), pL, b2L, bn), c2R = fast_speed2(G, rcpv(rR), pR, b2R, bn);
+  const T cmax = sqrtv(gt_pos(c2L, c2R) ? c2L : c2R);
+  const bool lt = uL < uR;
+  const T SL = (lt ? uL : uR) - cmax, SR = (lt ? uR : uL) + cmax;
   const T dL = SL - uL, dR = SR - uR;
-  const T den = dR * rR - dL * rL;
-  const T SM = (dR * rR * uR - dL * rL * uL - pTR + pTL) / den;
-  const T pTs = (dR * rR * pTL - dL * rL * pTR + rL * rR * dR * dL * (uR - uL)) / den;
-  // single-star states
-  T rsL, vsL, btsL, EsL, rsR, vsR, btsR, EsR;
+  const T mL = rL * dL, mR = rR * dR;  // mass fluxes through the fast waves
+  const T iden = rcpv(mR - mL);
+  const T SM = (mR * uR - mL * uL - pTR + pTL) * iden;
+  const T pTs = (mR * pTL - mL * pTR + mL * mR * (uR - uL)) * iden;
+  // single-star transverse states of both sides
+  T vsL[NT], bsL[NT], vsR[NT], bsR[NT];
+  const T eL = SL - SM, eR = SR - SM;
+  const T iL = rcpv(eL), iR = rcpv(eR);
+  const T rsL = mL * iL, rsR = mR * iR;
+  bool degL, degR;
   {
-    T dd = rL * dL * (SL - SM) - bn2;
-    rsL = rL * dL / (SL - SM);
-    if (fabs(dd) < Prec<T>::hlld_degenerate * (rL * dL * dL + bn2)) {
-      vsL = vL; btsL = btL;
-    } else {
-      T tv = bn * (SM - uL) / dd;
-      T tb = (rL * dL * dL - bn2) / dd;
-      vsL = vL - btL * tv;
-      btsL = btL * tb;
+    const T mm = mL * dL, dd = mL * eL - bn2;
+    degL = fabs(dd) < Prec<T>::hlld_degenerate * (mm + bn2);
+    // (m d - bn^2) / dd = 1 + m (SM - u) / dd, without the cancellation
+    const T k = (SM - uL) * rcpv(dd);
+    const T tv = bn * k, tb = mL * k + T(1);
+#pragma unroll
+    for (int a = 0; a < NT; ++a) {
+      vsL[a] = degL ? vL[a] : vL[a] - btL[a] * tv;
+      bsL[a] = degL ? btL[a] : btL[a] * tb;
     }
-    T vB = uL * bn + vL * btL, vBs = SM * bn + vsL * btsL;
-    EsL = (dL * EL - pTL * uL + pTs * SM + bn * (vB - vBs)) / (SL - SM);
-    dd = rR * dR * (SR - SM) - bn2;
-    rsR = rR * dR / (SR - SM);
-    if (fabs(dd) < Prec<T>::hlld_degenerate * (rR * dR * dR + bn2)) {
-      vsR = vR; btsR = btR;
-    } else {
-      T tv = bn * (SM - uR) / dd;
-      T tb = (rR * dR * dR - bn2) / dd;
-      vsR = vR - btR * tv;
-      btsR = btR * tb;
+  }
+  {
+    const T mm = mR * dR, dd = mR * eR - bn2;
+    degR = fabs(dd) < Prec<T>::hlld_degenerate * (mm + bn2);
+    // (m d - bn^2) / dd = 1 + m (SM - u) / dd, without the cancellation
+    const T k = (SM - uR) * rcpv(dd);
+    const T tv = bn * k, tb = mR * k + T(1);
+#pragma unroll
+    for (int a = 0; a < NT; ++a) {
+      vsR[a] = degR ? vR[a] : vR[a] - btR[a] * tv;
+      bsR[a] = degR ? btR[a] : btR[a] * tb;
     }
-    vB = uR * bn + vR * btR;
-    vBs = SM * bn + vsR * btsR;
-    EsR = (dR * ER - pTR * uR + pTs * SM + bn * (vB - vBs)) / (SR - SM);
   }
-  T UsL[5] = {rsL, rsL * SM, rsL * vsL, EsL, btsL};
-  T UsR[5] = {rsR, rsR * SM, rsR * vsR, EsR, btsR};
-  const T sqL = rsqrtv(rsL), sqR = rsqrtv(rsR);
-  const T SsL = SM - fabs(bn) / sqL, SsR = SM + fabs(bn) / sqR;
-  if (SsL >= T(0)) {
-    for (int q = 0; q < 5; ++q) F[q] = FL[q] + SL * (UsL[q] - UL[q]);
-    return;
+  const T yL = rsqrtp(rsL), yR = rsqrtp(rsR);
+  const T sqL = rsL * yL, sqR = rsR * yR;
+  const T abn = fabs(bn);
+  // the side and the region
+  const bool left = !negv(SM);
+  const bool outer = left ? !negv(SL) : negv(SR);
+  const bool single = left ? !negv(SM - abn * yL) : !posv(SM + abn * yR);
+  const T rK = left ? rL : rR, uK = left ? uL : uR, pTK = left ? pTL : pTR;
+  const T pK = left ? pL : pR, b2K = left ? b2L : b2R;
+  T vK[NT], bK[NT], v[NT], b[NT];
+#pragma unroll
+  for (int a = 0; a < NT; ++a) {
+    vK[a] = left ? vL[a] : vR[a];
+    bK[a] = left ? btL[a] : btR[a];
+    v[a] = left ? vsL[a] : vsR[a];
+    b[a] = left ? bsL[a] : bsR[a];
   }
-  if (SsR <= T(0)) {
-    for (int q = 0; q < 5; ++q) F[q] = FR[q] + SR * (UsR[q] - UR[q]);
-    return;
+  T v2 = uK * uK, vB = uK * bn;
+#pragma unroll
+  for (int a = 0; a < NT; ++a) {
+    v2 += vK[a] * vK[a];
+    vB += vK[a] * bK[a];
   }
-  // double-star states between the Alfven waves
-  const T sg = bn > T(0) ? T(1) : (bn < T(0) ? T(-1) : T(0));
-  const T inv = T(1) / (sqL + sqR);
-  const T vss = (sqL * vsL + sqR * vsR + (btsR - btsL) * sg) * inv;
-  const T btss = (sqL * btsR + sqR * btsL + sqL * sqR * (vsR - vsL) * sg) * inv;
-  const T vBss = SM * bn + vss * btss;
-  if (SM >= T(0)) {
-    T vBsL = SM * bn + vsL * btsL;
-    T E2 = EsL - sqL * (vBsL - vBss) * sg;
-    T U2[5] = {rsL, rsL * SM, rsL * vss, E2, btss};
-    for (int q = 0; q < 5; ++q)
-      F[q] = FL[q] + SL * (UsL[q] - UL[q]) + SsL * (U2[q] - UsL[q]);
+  const T EK = pK * G.inv_gm1 + T(0.5) * (rK * v2 + b2K);
+  T r, u, E, pT, extra[NT], vBf;
+  if (outer) {
+    r = rK; u = uK; E = EK; pT = pTK; vBf = vB;
+#pragma unroll
+    for (int a = 0; a < NT; ++a) { v[a] = vK[a]; b[a] = bK[a]; extra[a] = T(0); }
   } else {
-    T vBsR = SM * bn + vsR * btsR;
-    T E2 = EsR + sqR * (vBsR - vBss) * sg;
-    T U2[5] = {rsR, rsR * SM, rsR * vss, E2, btss};
-    for (int q = 0; q < 5; ++q)
-      F[q] = FR[q] + SR * (UsR[q] - UR[q]) + SsR * (U2[q] - UsR[q]);
+    r = left ? rsL : rsR;
+    u = SM;
+    pT = pTs;
+    T vBs = SM * bn;
+#pragma unroll
+    for (int a = 0; a < NT; ++a) vBs += v[a] * b[a];
+    const T dK = left ? dL : dR, iK = left ? iL : iR;
+    E = (dK * EK - pTK * uK + pTs * SM + bn * (vB - vBs)) * iK;
+    const bool deg = left ? degL : degR;
+#pragma unroll
+    for (int a = 0; a < NT; ++a) extra[a] = deg ? b[a] * (uK - SM) : T(0);
+    vBf = vBs;
+    if (!single) {  // between the Alfven waves
+      const T sg = bn > T(0) ? T(1) : (bn < T(0) ? T(-1) : T(0));
+      const T inv = rcpv(sqL + sqR), sqLR = sqL * sqR;
+      T vBss = SM * bn;
+#pragma unroll
+      for (int a = 0; a < NT; ++a) {
+        v[a] = (sqL * vsL[a] + sqR * vsR[a] + (bsR[a] - bsL[a]) * sg) * inv;
+        b[a] = (sqL * bsR[a] + sqR * bsL[a] + sqLR * (vsR[a] - vsL[a]) * sg) * inv;
+        vBss += v[a] * b[a];
+      }
+      E += (left ? -sqL : sqR) * (vBs - vBss) * sg;
+      vBf = vBss;
+    }
+  }
+  const T m = r * u;
+  F[0] = m;
+  F[1] = m * u + pT - bn2;
+  F[2 + NT] = (E + pT) * u - bn * vBf;
+#pragma unroll
+  for (int a = 0; a < NT; ++a) {
+    F[2 + a] = m * v[a] - bn * b[a];
+    F[3 + NT + a] = b[a] * u - v[a] * bn + extra[a];
   }
 }
 
-// ----------------------------------------------------------------------------
-// HLLD solver with two transverse components (3D MHD): per side (rho, u, v, w, p,
-// bv, bw) with u normal and (v, w), (bv, bw) the transverse velocity and field;
-// bn the common normal field.  Output in the face frame: F[0] mass, F[1] normal
-// momentum, F[2], F[3] transverse momenta, F[4] energy, F[5], F[6] transverse
-// field fluxes (the normal-field flux is zero).  Same wave-speed estimates and
-// degeneracy switch as hlld_flux.
-// ----------------------------------------------------------------------------
+// Planar MHD: F[0] mass, F[1] normal and F[2] transverse momentum, F[3] energy, F[4]
+// transverse field.
+template <class T>
+__device__ __forceinline__ void hlld_flux(const Gas<T>& G, T rL, T uL, T vL, T pL, T btL, T rR,
+                                          T uR, T vR, T pR, T btR, T bn, T* F, unsigned& err) {
+  hlld_core<T, 1>(G, rL, uL, &vL, pL, &btL, rR, uR, &vR, pR, &btR, bn, F, err);
+}
+
+// 3D MHD: F[0] mass, F[1] normal, F[2], F[3] transverse momenta, F[4] energy, F[5],
+// F[6] transverse field.
 template <class T>
 __device__ __forceinline__ void hlld_flux3(const Gas<T>& G, T rL, T uL, T vL, T wL, T pL, T bvL,
                                            T bwL, T rR, T uR, T vR, T wR, T pR, T bvR, T bwR,
                                            T bn, T* F, unsigned& err) {
-  if (!(rL > T(0) && pL > T(0) && rR > T(0) && pR > T(0))) {
-    err |= ERR_NONPHYS;
-    for (int q = 0; q < 7; ++q) F[q] = T(0);
-    return;
-  }
-  const T bn2 = bn * bn;
-  const T b2L = bn2 + bvL * bvL + bwL * bwL, b2R = bn2 + bvR * bvR + bwR * bwR;
-  const T EL = pL * G.inv_gm1 + T(0.5) * rL * (uL * uL + vL * vL + wL * wL) + T(0.5) * b2L;
-  const T ER = pR * G.inv_gm1 + T(0.5) * rR * (uR * uR + vR * vR + wR * wR) + T(0.5) * b2R;
-  const T pTL = pL + T(0.5) * b2L, pTR = pR + T(0.5) * b2R;
-  const T cfL = fast_speed(G, rL, pL, b2L, bn), cfR = fast_speed(G, rR, pR, b2R, bn);
-  const T cmax = cfL > cfR ? cfL : cfR;
-  const T SL = (uL < uR ? uL : uR) - cmax;
-  const T SR = (uL < uR ? uR : uL) + cmax;
-  T FL[7], FR[7], UL[7], UR[7];
-  {
-    T vB = uL * bn + vL * bvL + wL * bwL;
-    FL[0] = rL * uL; FL[1] = rL * uL * uL + pTL - bn2; FL[2] = rL * uL * vL - bn * bvL;
-    FL[3] = rL * uL * wL - bn * bwL; FL[4] = (EL + pTL) * uL - bn * vB;
-    FL[5] = bvL * uL - vL * bn; FL[6] = bwL * uL - wL * bn;
-    UL[0] = rL; UL[1] = rL * uL; UL[2] = rL * vL; UL[3] = rL * wL; UL[4] = EL;
-    UL[5] = bvL; UL[6] = bwL;
-    vB = uR * bn + vR * bvR + wR * bwR;
-    FR[0] = rR * uR; FR[1] = rR * uR * uR + pTR - bn2; FR[2] = rR * uR * vR - bn * bvR;
-    FR[3] = rR * uR * wR - bn * bwR; FR[4] = (ER + pTR) * uR - bn * vB;
-    FR[5] = bvR * uR - vR * bn; FR[6] = bwR * uR - wR * bn;
-    UR[0] = rR; UR[1] = rR * uR; UR[2] = rR * vR; UR[3] = rR * wR; UR[4] = ER;
-    UR[5] = bvR; UR[6] = bwR;
-  }
-  if (SL > T(0)) {
-    for (int q = 0; q < 7; ++q) F[q] = FL[q];
-    return;
-  }
-  if (SR < T(0)) {
-    for (int q = 0; q < 7; ++q) F[q] = FR[q];
-    return;
-  }
-  const T dL = SL - uL, dR = SR - uR;
-  const T den = dR * rR - dL * rL;
-  const T SM = (dR * rR * uR - dL * rL * uL - pTR + pTL) / den;
-  const T pTs = (dR * rR * pTL - dL * rL * pTR + rL * rR * dR * dL * (uR - uL)) / den;
-  // single-star states
-  T rsL, vsL, wsL, bvsL, bwsL, EsL, rsR, vsR, wsR, bvsR, bwsR, EsR;
-  {
-    T dd = rL * dL * (SL - SM) - bn2;
-    rsL = rL * dL / (SL - SM);
-    if (fabs(dd) < Prec<T>::hlld_degenerate * (rL * dL * dL + bn2)) {
-      vsL = vL; wsL = wL; bvsL = bvL; bwsL = bwL;
-    } else {
-      T tv = bn * (SM - uL) / dd;
-      T tb = (rL * dL * dL - bn2) / dd;
-      vsL = vL - bvL * tv; wsL = wL - bwL * tv;
-      bvsL = bvL * tb; bwsL = bwL * tb;
-    }
-    T vB = uL * bn + vL * bvL + wL * bwL, vBs = SM * bn + vsL * bvsL + wsL * bwsL;
-    EsL = (dL * EL - pTL * uL + pTs * SM + bn * (vB - vBs)) / (SL - SM);
-    dd = rR * dR * (SR - SM) - bn2;
-    rsR = rR * dR / (SR - SM);
-    if (fabs(dd) < Prec<T>::hlld_degenerate * (rR * dR * dR + bn2)) {
-      vsR = vR; wsR = wR; bvsR = bvR; bwsR = bwR;
-    } else {
-      T tv = bn * (SM - uR) / dd;
-      T tb = (rR * dR * dR - bn2) / dd;
-      vsR = vR - bvR * tv; wsR = wR - bwR * tv;
-      bvsR = bvR * tb; bwsR = bwR * tb;
-    }
-    vB = uR * bn + vR * bvR + wR * bwR;
-    vBs = SM * bn + vsR * bvsR + wsR * bwsR;
-    EsR = (dR * ER - pTR * uR + pTs * SM + bn * (vB - vBs)) / (SR - SM);
-  }
-  T UsL[7] = {rsL, rsL * SM, rsL * vsL, rsL * wsL, EsL, bvsL, bwsL};
-  T UsR[7] = {rsR, rsR * SM, rsR * vsR, rsR * wsR, EsR, bvsR, bwsR};
-  const T sqL = rsqrtv(rsL), sqR = rsqrtv(rsR);
-  const T SsL = SM - fabs(bn) / sqL, SsR = SM + fabs(bn) / sqR;
-  if (SsL >= T(0)) {
-    for (int q = 0; q < 7; ++q) F[q] = FL[q] + SL * (UsL[q] - UL[q]);
-    return;
-  }
-  if (SsR <= T(0)) {
-    for (int q = 0; q < 7; ++q) F[q] = FR[q] + SR * (UsR[q] - UR[q]);
-    return;
-  }
-  // double-star states between the Alfven waves
-  const T sg = bn > T(0) ? T(1) : (bn < T(0) ? T(-1) : T(0));
-  const T inv = T(1) / (sqL + sqR);
-  const T vss = (sqL * vsL + sqR * vsR + (bvsR - bvsL) * sg) * inv;
-  const T wss = (sqL * wsL + sqR * wsR + (bwsR - bwsL) * sg) * inv;
-  const T bvss = (sqL * bvsR + sqR * bvsL + sqL * sqR * (vsR - vsL) * sg) * inv;
-  const T bwss = (sqL * bwsR + sqR * bwsL + sqL * sqR * (wsR - wsL) * sg) * inv;
-  const T vBss = SM * bn + vss * bvss + wss * bwss;
-  if (SM >= T(0)) {
-    T vBsL = SM * bn + vsL * bvsL + wsL * bwsL;
-    T E2 = EsL - sqL * (vBsL - vBss) * sg;
-    T U2[7] = {rsL, rsL * SM, rsL * vss, rsL * wss, E2, bvss, bwss};
-    for (int q = 0; q < 7; ++q)
-      F[q] = FL[q] + SL * (UsL[q] - UL[q]) + SsL * (U2[q] - UsL[q]);
-  } else {
-    T vBsR = SM * bn + vsR * bvsR + wsR * bwsR;
-    T E2 = EsR + sqR * (vBsR - vBss) * sg;
-    T U2[7] = {rsR, rsR * SM, rsR * vss, rsR * wss, E2, bvss, bwss};
-    for (int q = 0; q < 7; ++q)
-      F[q] = FR[q] + SR * (UsR[q] - UR[q]) + SsR * (U2[q] - UsR[q]);
-  }
+  const T vl[2] = {vL, wL}, bl[2] = {bvL, bwL}, vr[2] = {vR, wR}, br[2] = {bvR, bwR};
+  hlld_core<T, 2>(G, rL, uL, vl, pL, bl, rR, uR, vr, pR, br, bn, F, err);
 }
 
 // ----------------------------------------------------------------------------
@@ -815,17 +749,16 @@ __device__ __forceinline__ void hlld_flux3(const Gas<T>& G, T rL, T uL, T vL, T 
 template <class T, int DIM>
 __device__ __forceinline__ T limiter_alpha(T phi, T phimax, T phimin, const T* grad,
                                            const T* half_h) {
-  T amax = T(0);
+  T amax = fabs(grad[0] * half_h[0]);
 #pragma unroll
-  for (int d = 0; d < DIM; ++d) {
-    T a = fabs(grad[d] * half_h[d]);
-    amax = a > amax ? a : amax;
+  for (int d = 1; d < DIM; ++d) {
+    const T a = fabs(grad[d] * half_h[d]);
+    amax = gt_pos(a, amax) ? a : amax;
   }
-  if (!(amax > T(0))) return T(1);
-  T up = phimax - phi, dn = phi - phimin;
-  T m = up < dn ? up : dn;
-  T psi = m / amax;
-  return psi < T(1) ? psi : T(1);
+  const T up = phimax - phi, dn = phi - phimin;  // both >= 0
+  const T m = gt_pos(dn, up) ? up : dn;
+  // psi = m / amax < 1
+  return gt_pos(amax, m) && !gt_pos(T(Tiny<T>::v), amax) ? m * rcpv(amax) : T(1);
 }
 
 }  // namespace dgk

@@ -97,13 +97,13 @@ struct TileScalars {
 template <int EQ, class TC>
 __device__ __forceinline__ void prims2d(const Gas<TC>& G, const TC* c, TC* W, unsigned& err) {
   TC rho = c[0];
-  TC inv = TC(1) / rho;
+  TC inv = rcpv(rho);
   TC vx = c[1] * inv, vy = c[2] * inv;
   TC kin = TC(0.5) * (c[1] * vx + c[2] * vy);
   TC mag = TC(0);
   if (EQ == 1) mag = TC(0.5) * (c[4] * c[4] + c[5] * c[5]);
   TC p = G.gm1 * (c[3] - kin - mag);
-  if (!(rho > TC(0) && p > TC(0))) err |= ERR_NONPHYS;
+  if (!(posv(rho) && posv(p))) err |= ERR_NONPHYS;
   W[0] = rho; W[1] = vx; W[2] = vy; W[3] = p;
   if (EQ == 1) { W[4] = c[4]; W[5] = c[5]; }
 }
@@ -118,17 +118,14 @@ __device__ __forceinline__ void limit_cell2d(const Gas<TC>& G, const TC* hh, con
   TC hi[NP], lo[NP];
 #pragma unroll
   for (int q = 0; q < NP; ++q) {
-    TC a = W[q], b = W[q];
+    Extremes<TC> ex(W[q]);
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      a = Wn[k][q] > a ? Wn[k][q] : a;
-      b = Wn[k][q] < b ? Wn[k][q] : b;
-    }
-    hi[q] = a;
-    lo[q] = b;
+    for (int k = 0; k < 4; k += 2) ex.add(Wn[k][q], Wn[k + 1][q]);
+    hi[q] = ex.max();
+    lo[q] = ex.min();
   }
   const TC rho = W[0], vx = W[1], vy = W[2];
-  const TC inv = TC(1) / rho;
+  const TC inv = rcpv(rho);
   TC gr[2], gvx[2], gvy[2], gp[2], gbx[2], gby[2];
   if (EQ == 1) {
     gbx[0] = s[10]; gbx[1] = s[8];   // dBx/dx = a3, dBx/dy = a1
@@ -175,12 +172,12 @@ __device__ __forceinline__ void limit_cell2d(const Gas<TC>& G, const TC* hh, con
 template <int EQ, class TC>
 __device__ __forceinline__ void phys_flux2d(const Gas<TC>& G, const TC* c, TC* Fx, TC* Fy,
                                             unsigned& err) {
-  TC rho = c[0], inv = TC(1) / rho;
+  TC rho = c[0], inv = rcpv(rho);
   TC vx = c[1] * inv, vy = c[2] * inv;
   TC bx = TC(0), by = TC(0), b2h = TC(0);
   if (EQ == 1) { bx = c[4]; by = c[5]; b2h = TC(0.5) * (bx * bx + by * by); }
   TC p = G.gm1 * (c[3] - TC(0.5) * (c[1] * vx + c[2] * vy) - b2h);
-  if (!(rho > TC(0) && p > TC(0))) err |= ERR_NONPHYS;
+  if (!(posv(rho) && posv(p))) err |= ERR_NONPHYS;
   TC pT = p + b2h;
   TC e = c[3] + pT;
   Fx[0] = c[1];
@@ -216,7 +213,7 @@ template <int EQ, class TC>
 __device__ __forceinline__ void face_flux2d(const Gas<TC>& G, int dir, const TC* cl,
                                             const TC* cr, TC* F, unsigned& err) {
   TC rl = cl[0], rr = cr[0];
-  TC il = TC(1) / rl, ir = TC(1) / rr;
+  TC il = rcpv(rl), ir = rcpv(rr);
   TC vxl = cl[1] * il, vyl = cl[2] * il, vxr = cr[1] * ir, vyr = cr[2] * ir;
   TC magl = TC(0), magr = TC(0);
   if (EQ == 1) {
@@ -353,9 +350,8 @@ __device__ __forceinline__ void stage2d_prefetch_base(const Stage2DArgs<TS>& A,
 // word.
 template <int EQ, class TC, class TS, int NT>
 __device__ __forceinline__ void courant_commit2d(const Stage2DArgs<TS>& A, const Gas<TC>& G,
-                                                 bool owner, const double* o0, TC dx, TC dy,
-                                                 double dt, unsigned nblk, unsigned err,
-                                                 TileScalars<NT>& S) {
+                                                 bool owner, const double* o0, double dt, unsigned nblk,
+                                                 unsigned err, TileScalars<NT>& S) {
   constexpr int NV = Tr2<EQ>::NV, NP = Tr2<EQ>::NP;
   const int tid = threadIdx.x;
   // Courant signal speed of the new state, reduced over the grid (in TC; the
@@ -368,13 +364,13 @@ __device__ __forceinline__ void courant_commit2d(const Stage2DArgs<TS>& A, const
     prims2d<EQ, TC>(G, c, W, err);
     TC cx, cy;
     if (EQ == 0) {
-      cx = cy = sqrt(G.g * W[3] / W[0]);
+      cx = cy = sqrtv(G.g * W[3] * rcpv(W[0]));
     } else {
       TC b2 = W[4] * W[4] + W[5] * W[5];
       cx = fast_speed(G, W[0], W[3], b2, W[4]);
       cy = fast_speed(G, W[0], W[3], b2, W[5]);
     }
-    sp = (fabs(W[1]) + cx) / dx + (fabs(W[2]) + cy) / dy;
+    sp = (fabs(W[1]) + cx) * A.geo.ix + (fabs(W[2]) + cy) * A.geo.iy;
     if (!courant_ok(sp, W[0], W[3])) { err |= ERR_NONPHYS; sp = TC(0); }
   }
 #pragma unroll
@@ -458,8 +454,8 @@ __device__ __forceinline__ void stage2d_compute(const Stage2DArgs<TS>& A, int i0
   __syncthreads();
   if (ph) ph->mark(1);
 
-  const TC dx = Cvt<TC>::to_tc(A.dx), dy = Cvt<TC>::to_tc(A.dy);
-  TC hh[2] = {TC(0.5) * dx, TC(0.5) * dy};
+  const Geo2D<TS>& geo = A.geo;
+  const TC hh[2] = {geo.hx, geo.hy};
 
   // ---- limiter on the tile and its 1-cell ring, in place
   if (A.limiter) {
@@ -487,7 +483,7 @@ __device__ __forceinline__ void stage2d_compute(const Stage2DArgs<TS>& A, int i0
   if (ph) ph->mark(2);
 
   // ---- faces: Riemann fluxes at the Gauss points, each face once
-  const TC ox = dx * TC(0.28867513459481288225), oy = dy * TC(0.28867513459481288225);
+  const TC ox = geo.ox, oy = geo.oy;
   for (int e = tid; e < 2 * (NFX + NFY); e += NT) {
     const bool xf = e < 2 * NFX;
     const int ee = xf ? e : e - 2 * NFX;
@@ -565,9 +561,8 @@ __device__ __forceinline__ void stage2d_compute(const Stage2DArgs<TS>& A, int i0
     b0 = s_fy[(q * NFY + fym + TX) * 2]; b1 = s_fy[(q * NFY + fym + TX) * 2 + 1];
     Sym[q] = a0 + a1; Dym[q] = a1 - a0; Syp[q] = b0 + b1; Dyp[q] = b1 - b0;
   }
-  const TC inv2dx = TC(0.5) / dx, inv2dy = TC(0.5) / dy;
-  const TC c3x = TC(3) / (dx * dx), c3y = TC(3) / (dy * dy);
-  const TC r3 = TC(1.7320508075688772935) / (dx * dy);
+  const TC inv2dx = geo.i2x, inv2dy = geo.i2y;
+  const TC c3x = geo.c3x, c3y = geo.c3y, r3 = geo.r3;
   TC rc0[NV], rs[NS];
 #pragma unroll
   for (int v = 0; v < 4; ++v) {
@@ -580,8 +575,7 @@ __device__ __forceinline__ void stage2d_compute(const Stage2DArgs<TS>& A, int i0
     rc0[5] = -(Sxp[4] - Sxm[4]) * inv2dx;
     rs[8] = c3y * (sFy[4] - (Syp[4] + Sym[4]));
     rs[9] = c3x * (sFx[4] - (Sxp[4] + Sxm[4]));
-    const TC ca3 = TC(1.7320508075688772935) / (dx * dx + dy * dy);
-    rs[10] = ca3 * ((dy / dx) * (Dxp[4] - Dxm[4]) - (dx / dy) * (Dyp[4] - Dym[4]));
+    rs[10] = geo.ax * (Dxp[4] - Dxm[4]) - geo.ay * (Dyp[4] - Dym[4]);
   }
 
   double o0[NV];
@@ -640,7 +634,7 @@ __device__ __forceinline__ void stage2d_compute(const Stage2DArgs<TS>& A, int i0
 
   if (ph) ph->mark(4);
   if (STAGE == 2) {
-    courant_commit2d<EQ, TC, TS, NT>(A, G, owner, o0, dx, dy, dt, nblk, err, S);
+    courant_commit2d<EQ, TC, TS, NT>(A, G, owner, o0, dt, nblk, err, S);
   } else {
     if (err) atomicOr(&S.err, err);
     __syncthreads();

@@ -52,10 +52,10 @@ __host__ __device__ constexpr size_t stage3d_smem_bytes() {
 
 template <class TC>
 __device__ __forceinline__ void prims3d(const Gas<TC>& G, const TC* c, TC* W, unsigned& err) {
-  TC rho = c[0], inv = TC(1) / rho;
+  TC rho = c[0], inv = rcpv(rho);
   TC vx = c[1] * inv, vy = c[2] * inv, vz = c[3] * inv;
   TC p = G.gm1 * (c[4] - TC(0.5) * (c[1] * vx + c[2] * vy + c[3] * vz));
-  if (!(rho > TC(0) && p > TC(0))) err |= ERR_NONPHYS;
+  if (!(posv(rho) && posv(p))) err |= ERR_NONPHYS;
   W[0] = rho; W[1] = vx; W[2] = vy; W[3] = vz; W[4] = p;
 }
 
@@ -67,16 +67,13 @@ __device__ __forceinline__ void limit_cell3d(const Gas<TC>& G, const TC* hh, con
   TC hi[5], lo[5];
 #pragma unroll
   for (int q = 0; q < 5; ++q) {
-    TC a = W[q], b = W[q];
+    Extremes<TC> ex(W[q]);
 #pragma unroll
-    for (int k = 0; k < 6; ++k) {
-      a = Wn[k][q] > a ? Wn[k][q] : a;
-      b = Wn[k][q] < b ? Wn[k][q] : b;
-    }
-    hi[q] = a;
-    lo[q] = b;
+    for (int k = 0; k < 6; k += 2) ex.add(Wn[k][q], Wn[k + 1][q]);
+    hi[q] = ex.max();
+    lo[q] = ex.min();
   }
-  const TC rho = W[0], inv = TC(1) / rho;
+  const TC rho = W[0], inv = rcpv(rho);
   const TC v[3] = {W[1], W[2], W[3]};
   const TC v2h = TC(0.5) * (v[0] * v[0] + v[1] * v[1] + v[2] * v[2]);
   TC gr[3], gv[3][3], gp[3];
@@ -155,10 +152,10 @@ __device__ __forceinline__ void rec_put(TC* rec, const TC* v) {
 template <class TC>
 __device__ __forceinline__ void phys_flux3d(const Gas<TC>& G, const TC* c, int d, TC* F,
                                             unsigned& err) {
-  TC rho = c[0], inv = TC(1) / rho;
+  TC rho = c[0], inv = rcpv(rho);
   TC v[3] = {c[1] * inv, c[2] * inv, c[3] * inv};
   TC p = G.gm1 * (c[4] - TC(0.5) * (c[1] * v[0] + c[2] * v[1] + c[3] * v[2]));
-  if (!(rho > TC(0) && p > TC(0))) err |= ERR_NONPHYS;
+  if (!(posv(rho) && posv(p))) err |= ERR_NONPHYS;
   TC vd = v[d];
   F[0] = c[1 + d];
   F[1] = c[1] * vd;
@@ -175,7 +172,7 @@ __device__ __forceinline__ void phys_flux3d(const Gas<TC>& G, const TC* c, int d
 template <class TC>
 __device__ __forceinline__ void face_flux3d(const Gas<TC>& G, int d, const TC* cl, const TC* cr,
                                             TC* F, unsigned& err) {
-  TC il = TC(1) / cl[0], ir = TC(1) / cr[0];
+  TC il = rcpv(cl[0]), ir = rcpv(cr[0]);
   TC lx = cl[1] * il, ly = cl[2] * il, lz = cl[3] * il;
   TC rx = cr[1] * ir, ry = cr[2] * ir, rz = cr[3] * ir;
   TC pl = G.gm1 * (cl[4] - TC(0.5) * (cl[1] * lx + cl[2] * ly + cl[3] * lz));
@@ -197,13 +194,10 @@ __device__ __forceinline__ void face_flux3d(const Gas<TC>& G, int d, const TC* c
 // variables; s_f holds [var][face][gauss point] with the 2x2 points in the order
 // (a, b) = (--, -+, +-, ++) of the transverse axes (e1, e2).
 template <int D, class TC, int NV = 5>
-__device__ __forceinline__ void gather3d(const TC* s_f, int FMAX, int fm, int fp, const TC* hd,
-                                         TC* rc0, TC* rs) {
+__device__ __forceinline__ void gather3d(const TC* s_f, int FMAX, int fm, int fp,
+                                         const Geo3D<TC>& geo, TC* rc0, TC* rs) {
   constexpr int E1 = D == 0 ? 1 : 0, E2 = D == 2 ? 1 : 2;
-  const TC c0f = TC(0.25) / hd[D];
-  const TC csf = TC(1.5) / (hd[D] * hd[D]);
-  const TC ce1 = TC(0.86602540378443864676) / (hd[E1] * hd[D]);
-  const TC ce2 = TC(0.86602540378443864676) / (hd[E2] * hd[D]);
+  const TC c0f = geo.c0[D], csf = geo.cs[D], ce1 = geo.ce[D][E1], ce2 = geo.ce[D][E2];
 #pragma unroll
   for (int v = 0; v < NV; ++v) {
     const TC* m = s_f + (v * FMAX + fm) * 4;
@@ -389,10 +383,9 @@ __global__ void __launch_bounds__(TX * TY * TZ, (Stage3dMinBlocks<TX * TY * TZ, 
   __syncthreads();
   ph.mark(0);
 
-  const TC dx = Cvt<TC>::to_tc(A.dx), dy = Cvt<TC>::to_tc(A.dy), dz = Cvt<TC>::to_tc(A.dz);
-  const TC hh[3] = {TC(0.5) * dx, TC(0.5) * dy, TC(0.5) * dz};
-  const TC oo[3] = {dx * TC(0.28867513459481288225), dy * TC(0.28867513459481288225),
-                    dz * TC(0.28867513459481288225)};
+  const Geo3D<TS>& geo = A.geo;
+  const TC hh[3] = {geo.hh[0], geo.hh[1], geo.hh[2]};
+  const TC oo[3] = {geo.oo[0], geo.oo[1], geo.oo[2]};
 
   // ---- limiter on the tile and its face slabs (the cells the faces read)
   if (A.limiter) {
@@ -458,16 +451,14 @@ __global__ void __launch_bounds__(TX * TY * TZ, (Stage3dMinBlocks<TX * TY * TZ, 
         for (int v = 0; v < 5; ++v) sF[d][v] += F[v];
       }
     }
-    const TC hd[3] = {dx, dy, dz};
 #pragma unroll
     for (int v = 0; v < 5; ++v)
 #pragma unroll
-      for (int d = 0; d < 3; ++d) rs[3 * v + d] = TC(1.5) / (hd[d] * hd[d]) * sF[d][v];
+      for (int d = 0; d < 3; ++d) rs[3 * v + d] = geo.cs[d] * sF[d][v];
   }
 
   ph.mark(2);
   // ---- faces, one orientation at a time (rolled loop: one copy of the solver)
-  const TC hd[3] = {dx, dy, dz};
 #pragma unroll 1
   for (int d = 0; d < 3; ++d) {
     const int FX = TX + (d == 0), FY = TY + (d == 1), FZ = TZ + (d == 2);
@@ -507,9 +498,9 @@ __global__ void __launch_bounds__(TX * TY * TZ, (Stage3dMinBlocks<TX * TY * TZ, 
     {
       const int fm = (lz * FY + ly) * FX + lx;
       const int fp = fm + (d == 0 ? 1 : (d == 1 ? FX : FX * FY));
-      if (d == 0) gather3d<0, TC>(s_f, FMAX, fm, fp, hd, rc0, rs);
-      else if (d == 1) gather3d<1, TC>(s_f, FMAX, fm, fp, hd, rc0, rs);
-      else gather3d<2, TC>(s_f, FMAX, fm, fp, hd, rc0, rs);
+      if (d == 0) gather3d<0, TC>(s_f, FMAX, fm, fp, geo, rc0, rs);
+      else if (d == 1) gather3d<1, TC>(s_f, FMAX, fm, fp, geo, rc0, rs);
+      else gather3d<2, TC>(s_f, FMAX, fm, fp, geo, rc0, rs);
     }
     __syncthreads();
     ph.mark(4 + 2 * d);
@@ -590,8 +581,9 @@ __global__ void __launch_bounds__(TX * TY * TZ, (Stage3dMinBlocks<TX * TY * TZ, 
 #pragma unroll
       for (int v = 0; v < 5; ++v) c[v] = Cvt<TC>::to_tc(o0[v]);
       prims3d<TC>(G, c, W, err);
-      TC cs = sqrt(G.g * W[4] / W[0]);
-      sp = (fabs(W[1]) + cs) / dx + (fabs(W[2]) + cs) / dy + (fabs(W[3]) + cs) / dz;
+      TC cs = sqrtv(G.g * W[4] * rcpv(W[0]));
+      sp = (fabs(W[1]) + cs) * geo.ih[0] + (fabs(W[2]) + cs) * geo.ih[1] +
+           (fabs(W[3]) + cs) * geo.ih[2];
       if (!courant_ok(sp, W[0], W[4])) { err |= ERR_NONPHYS; sp = TC(0); }
     }
 #pragma unroll

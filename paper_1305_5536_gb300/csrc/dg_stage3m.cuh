@@ -50,11 +50,11 @@ __host__ __device__ constexpr size_t stage3m_smem_bytes() {
 // Centroid primitives (rho, vx, vy, vz, p, Bx, By, Bz) from averages.
 template <class TC>
 __device__ __forceinline__ void prims3m(const Gas<TC>& G, const TC* c, TC* W, unsigned& err) {
-  TC rho = c[0], inv = TC(1) / rho;
+  TC rho = c[0], inv = rcpv(rho);
   TC vx = c[1] * inv, vy = c[2] * inv, vz = c[3] * inv;
   TC mag = TC(0.5) * (c[5] * c[5] + c[6] * c[6] + c[7] * c[7]);
   TC p = G.gm1 * (c[4] - TC(0.5) * (c[1] * vx + c[2] * vy + c[3] * vz) - mag);
-  if (!(rho > TC(0) && p > TC(0))) err |= ERR_NONPHYS;
+  if (!(posv(rho) && posv(p))) err |= ERR_NONPHYS;
   W[0] = rho; W[1] = vx; W[2] = vy; W[3] = vz; W[4] = p;
   W[5] = c[5]; W[6] = c[6]; W[7] = c[7];
 }
@@ -75,16 +75,13 @@ __device__ __forceinline__ void limit_cell3m(const Gas<TC>& G, const TC* hh, con
   TC hi[8], lo[8];
 #pragma unroll
   for (int q = 0; q < 8; ++q) {
-    TC a = W[q], b = W[q];
+    Extremes<TC> ex(W[q]);
 #pragma unroll
-    for (int k = 0; k < 6; ++k) {
-      a = Wn[k][q] > a ? Wn[k][q] : a;
-      b = Wn[k][q] < b ? Wn[k][q] : b;
-    }
-    hi[q] = a;
-    lo[q] = b;
+    for (int k = 0; k < 6; k += 2) ex.add(Wn[k][q], Wn[k + 1][q]);
+    hi[q] = ex.max();
+    lo[q] = ex.min();
   }
-  const TC rho = W[0], inv = TC(1) / rho;
+  const TC rho = W[0], inv = rcpv(rho);
   const TC v[3] = {W[1], W[2], W[3]};
   const TC v2h = TC(0.5) * (v[0] * v[0] + v[1] * v[1] + v[2] * v[2]);
   TC gB[3][3];
@@ -147,16 +144,13 @@ __device__ __forceinline__ void weno_cell3m(const Gas<TC>& G, const TC* hh, cons
   TC hi[8], lo[8];
 #pragma unroll
   for (int q = 0; q < 8; ++q) {
-    TC a = W[q], b = W[q];
+    Extremes<TC> ex(W[q]);
 #pragma unroll
-    for (int k = 0; k < 6; ++k) {
-      a = Wn[k][q] > a ? Wn[k][q] : a;
-      b = Wn[k][q] < b ? Wn[k][q] : b;
-    }
-    hi[q] = a;
-    lo[q] = b;
+    for (int k = 0; k < 6; k += 2) ex.add(Wn[k][q], Wn[k + 1][q]);
+    hi[q] = ex.max();
+    lo[q] = ex.min();
   }
-  const TC rho = W[0], inv = TC(1) / rho;
+  const TC rho = W[0], inv = rcpv(rho);
   const TC v[3] = {W[1], W[2], W[3]};
   const TC v2h = TC(0.5) * (v[0] * v[0] + v[1] * v[1] + v[2] * v[2]);
   TC gB[3][3];
@@ -194,7 +188,7 @@ __device__ __forceinline__ void weno_cell3m(const Gas<TC>& G, const TC* hh, cons
   const TC hx2 = hh[0] * hh[0], hy2 = hh[1] * hh[1], hz2 = hh[2] * hh[2];
   const TC P = hx2 * Gs[0][0] - hy2 * Gs[1][1], Q = hx2 * Gs[0][0] - hz2 * Gs[2][2];
   const TC Am = hx2 + hy2, Bm = hx2 + hz2;
-  const TC idet = TC(1) / (Am * Bm - hx2 * hx2);
+  const TC idet = rcpv(Am * Bm - hx2 * hx2);
   TC st[23];  // the projected stencil field in slots 15..22
   st[15] = Gs[0][1]; st[16] = Gs[0][2]; st[17] = Gs[1][0];
   st[18] = Gs[1][2]; st[19] = Gs[2][0]; st[20] = Gs[2][1];
@@ -209,9 +203,9 @@ __device__ __forceinline__ void weno_cell3m(const Gas<TC>& G, const TC* hh, cons
     for (int k = 0; k < 6; ++k) nb[k] = Wn[k][5 + i];
     os += weno_osc<TC, 3>(W[5 + i], nb, sB[i], hh);
   }
-  const TC wd = TC(1) / sqrt(TC(kWenoEps) + od);
-  const TC ws = TC(1) / sqrt(TC(kWenoEps) + os);
-  const TC iw = TC(1) / (wd + ws);
+  const TC wd = rsqrtp(TC(kWenoEps) + od);
+  const TC ws = rsqrtp(TC(kWenoEps) + os);
+  const TC iw = rcpv(wd + ws);
 #pragma unroll
   for (int k = 15; k < 23; ++k) s[k] = (wd * s[k] + ws * st[k]) * iw;
   field_grad3m<TC>(s, gB);  // the limited field's gradients
@@ -255,12 +249,12 @@ __device__ __forceinline__ void eval3m(const TC* c0, const TC* s, TC x, TC y, TC
 template <class TC>
 __device__ __forceinline__ void phys_flux3m(const Gas<TC>& G, const TC* c, int d, TC* F,
                                             unsigned& err) {
-  const TC rho = c[0], inv = TC(1) / rho;
+  const TC rho = c[0], inv = rcpv(rho);
   const TC v[3] = {c[1] * inv, c[2] * inv, c[3] * inv};
   const TC B[3] = {c[5], c[6], c[7]};
   const TC b2h = TC(0.5) * (B[0] * B[0] + B[1] * B[1] + B[2] * B[2]);
   const TC p = G.gm1 * (c[4] - TC(0.5) * (c[1] * v[0] + c[2] * v[1] + c[3] * v[2]) - b2h);
-  if (!(rho > TC(0) && p > TC(0))) err |= ERR_NONPHYS;
+  if (!(posv(rho) && posv(p))) err |= ERR_NONPHYS;
   const TC pT = p + b2h;
   const TC vd = d == 0 ? v[0] : (d == 1 ? v[1] : v[2]);
   const TC Bd = d == 0 ? B[0] : (d == 1 ? B[1] : B[2]);
@@ -314,17 +308,14 @@ __device__ __forceinline__ void face_flux3m(const Gas<TC>& G, int d, const TC* c
 
 // Field part of the right-hand side from the Taylor-like gathers r[3*(5+i)+d].
 template <class TC>
-__device__ __forceinline__ void field_rhs3m(const TC* rs24, const TC* hd, TC* ra) {
+__device__ __forceinline__ void field_rhs3m(const TC* rs24, const Geo3D<TC>& geo, TC* ra) {
   const TC rxx = rs24[15], rxy = rs24[16], rxz = rs24[17];
   const TC ryx = rs24[18], ryy = rs24[19], ryz = rs24[20];
   const TC rzx = rs24[21], rzy = rs24[22], rzz = rs24[23];
   ra[0] = rxy; ra[1] = rxz; ra[2] = ryx; ra[3] = ryz; ra[4] = rzx; ra[5] = rzy;
-  const TC hx2 = hd[0] * hd[0], hy2 = hd[1] * hd[1], hz2 = hd[2] * hd[2];
-  const TC P = hx2 * rxx - hy2 * ryy, Q = hx2 * rxx - hz2 * rzz;
-  const TC A = hx2 + hy2, Bm = hx2 + hz2;
-  const TC det = A * Bm - hx2 * hx2;
-  ra[6] = (Bm * P - hx2 * Q) / det;
-  ra[7] = (A * Q - hx2 * P) / det;
+  const TC P = geo.h2[0] * rxx - geo.h2[1] * ryy, Q = geo.h2[0] * rxx - geo.h2[2] * rzz;
+  ra[6] = geo.f[0] * P + geo.f[1] * Q;
+  ra[7] = geo.f[2] * P + geo.f[3] * Q;
 }
 
 // FP32: two resident 256-thread CTAs per SM (128 registers a thread); FP64 keeps
@@ -402,11 +393,9 @@ __global__ void __launch_bounds__(TX * TY * TZ, (Stage3mMinBlocks<TX * TY * TZ, 
   cp_async_wait_all();
   __syncthreads();
 
-  const TC dx = Cvt<TC>::to_tc(A.dx), dy = Cvt<TC>::to_tc(A.dy), dz = Cvt<TC>::to_tc(A.dz);
-  const TC hh[3] = {TC(0.5) * dx, TC(0.5) * dy, TC(0.5) * dz};
-  const TC oo[3] = {dx * TC(0.28867513459481288225), dy * TC(0.28867513459481288225),
-                    dz * TC(0.28867513459481288225)};
-  const TC hd[3] = {dx, dy, dz};
+  const Geo3D<TS>& geo = A.geo;
+  const TC hh[3] = {geo.hh[0], geo.hh[1], geo.hh[2]};
+  const TC oo[3] = {geo.oo[0], geo.oo[1], geo.oo[2]};
 
   // ---- limiter on the tile and its face slabs (the cells the faces read)
   if (A.limiter) {
@@ -458,7 +447,7 @@ __global__ void __launch_bounds__(TX * TY * TZ, (Stage3mMinBlocks<TX * TY * TZ, 
       for (int d = 0; d < 3; ++d) {
         TC F[8];
         phys_flux3m<TC>(G, c, d, F, err);
-        const TC w = TC(1.5) / (hd[d] * hd[d]);
+        const TC w = geo.cs[d];
 #pragma unroll
         for (int v = 0; v < 8; ++v) rs[3 * v + d] += w * F[v];
       }
@@ -503,14 +492,14 @@ __global__ void __launch_bounds__(TX * TY * TZ, (Stage3mMinBlocks<TX * TY * TZ, 
       const int fp = fm + (d == 0 ? 1 : (d == 1 ? FX : FX * FY));
       // gather3d for the 5 Taylor variables and the 3 field components
       if (d == 0) {
-        gather3d<0, TC>(s_f, FMAX, fm, fp, hd, rc0, rs);
-        gather3d<0, TC, 3>(s_f + 5 * FMAX * 4, FMAX, fm, fp, hd, rc0 + 5, rs + 15);
+        gather3d<0, TC>(s_f, FMAX, fm, fp, geo, rc0, rs);
+        gather3d<0, TC, 3>(s_f + 5 * FMAX * 4, FMAX, fm, fp, geo, rc0 + 5, rs + 15);
       } else if (d == 1) {
-        gather3d<1, TC>(s_f, FMAX, fm, fp, hd, rc0, rs);
-        gather3d<1, TC, 3>(s_f + 5 * FMAX * 4, FMAX, fm, fp, hd, rc0 + 5, rs + 15);
+        gather3d<1, TC>(s_f, FMAX, fm, fp, geo, rc0, rs);
+        gather3d<1, TC, 3>(s_f + 5 * FMAX * 4, FMAX, fm, fp, geo, rc0 + 5, rs + 15);
       } else {
-        gather3d<2, TC>(s_f, FMAX, fm, fp, hd, rc0, rs);
-        gather3d<2, TC, 3>(s_f + 5 * FMAX * 4, FMAX, fm, fp, hd, rc0 + 5, rs + 15);
+        gather3d<2, TC>(s_f, FMAX, fm, fp, geo, rc0, rs);
+        gather3d<2, TC, 3>(s_f + 5 * FMAX * 4, FMAX, fm, fp, geo, rc0 + 5, rs + 15);
       }
     }
     __syncthreads();
@@ -518,7 +507,7 @@ __global__ void __launch_bounds__(TX * TY * TZ, (Stage3mMinBlocks<TX * TY * TZ, 
   TC rsl[23];
 #pragma unroll
   for (int k = 0; k < 15; ++k) rsl[k] = rs[k];
-  field_rhs3m<TC>(rs, hd, rsl + 15);
+  field_rhs3m<TC>(rs, geo, rsl + 15);
 
   // ---- Runge-Kutta combination
   const int gi = i0 + lx, gj = j0 + ly, gk = k0 + lz;
@@ -588,9 +577,9 @@ __global__ void __launch_bounds__(TX * TY * TZ, (Stage3mMinBlocks<TX * TY * TZ, 
       for (int v = 0; v < 8; ++v) c[v] = Cvt<TC>::to_tc(o0[v]);
       prims3m<TC>(G, c, W, err);
       const TC b2 = W[5] * W[5] + W[6] * W[6] + W[7] * W[7];
-      sp = (fabs(W[1]) + fast_speed(G, W[0], W[4], b2, W[5])) / dx +
-           (fabs(W[2]) + fast_speed(G, W[0], W[4], b2, W[6])) / dy +
-           (fabs(W[3]) + fast_speed(G, W[0], W[4], b2, W[7])) / dz;
+      sp = (fabs(W[1]) + fast_speed(G, W[0], W[4], b2, W[5])) * geo.ih[0] +
+           (fabs(W[2]) + fast_speed(G, W[0], W[4], b2, W[6])) * geo.ih[1] +
+           (fabs(W[3]) + fast_speed(G, W[0], W[4], b2, W[7])) * geo.ih[2];
       if (!courant_ok(sp, W[0], W[4])) { err |= ERR_NONPHYS; sp = TC(0); }
     }
 #pragma unroll

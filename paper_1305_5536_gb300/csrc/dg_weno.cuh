@@ -42,7 +42,7 @@ template <class TC, int DIM>
 __device__ __forceinline__ void weno_stencil(TC phi, TC hi, TC lo, const TC* nb, const TC* hh,
                                              TC* gs) {
 #pragma unroll
-  for (int d = 0; d < DIM; ++d) gs[d] = (nb[2 * d + 1] - nb[2 * d]) * (TC(0.25) / hh[d]);
+  for (int d = 0; d < DIM; ++d) gs[d] = (nb[2 * d + 1] - nb[2 * d]) * (TC(0.25) * rcpv(hh[d]));
   const TC a = limiter_alpha<TC, DIM>(phi, hi, lo, gs, hh);
 #pragma unroll
   for (int d = 0; d < DIM; ++d) gs[d] *= a;
@@ -54,9 +54,9 @@ __device__ __forceinline__ void weno_blend(TC phi, TC hi, TC lo, const TC* nb, c
                                            TC* g) {
   TC gs[DIM];
   weno_stencil<TC, DIM>(phi, hi, lo, nb, hh, gs);
-  const TC wd = TC(1) / sqrt(TC(kWenoEps) + weno_osc<TC, DIM>(phi, nb, g, hh));
-  const TC ws = TC(1) / sqrt(TC(kWenoEps) + weno_osc<TC, DIM>(phi, nb, gs, hh));
-  const TC inv = TC(1) / (wd + ws);
+  const TC wd = rsqrtp(TC(kWenoEps) + weno_osc<TC, DIM>(phi, nb, g, hh));
+  const TC ws = rsqrtp(TC(kWenoEps) + weno_osc<TC, DIM>(phi, nb, gs, hh));
+  const TC inv = rcpv(wd + ws);
 #pragma unroll
   for (int d = 0; d < DIM; ++d) g[d] = (wd * g[d] + ws * gs[d]) * inv;
 }
@@ -72,17 +72,14 @@ __device__ __forceinline__ void weno_cell2d(const Gas<TC>& G, const TC* hh, cons
   TC hi[NP], lo[NP];
 #pragma unroll
   for (int q = 0; q < NP; ++q) {
-    TC a = W[q], b = W[q];
+    Extremes<TC> ex(W[q]);
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      a = Wn[k][q] > a ? Wn[k][q] : a;
-      b = Wn[k][q] < b ? Wn[k][q] : b;
-    }
-    hi[q] = a;
-    lo[q] = b;
+    for (int k = 0; k < 4; k += 2) ex.add(Wn[k][q], Wn[k + 1][q]);
+    hi[q] = ex.max();
+    lo[q] = ex.min();
   }
   const TC rho = W[0], vx = W[1], vy = W[2];
-  const TC inv = TC(1) / rho;
+  const TC inv = rcpv(rho);
   const TC v2h = TC(0.5) * (vx * vx + vy * vy);
   TC a1 = TC(0), a2 = TC(0), a3 = TC(0);
   if (EQ == 1) { a1 = s[8]; a2 = s[9]; a3 = s[10]; }
@@ -109,14 +106,14 @@ __device__ __forceinline__ void weno_cell2d(const Gas<TC>& G, const TC* hh, cons
     weno_stencil<TC, 2>(W[4], hi[4], lo[4], nbx, hh, gx);
     weno_stencil<TC, 2>(W[5], hi[5], lo[5], nby, hh, gy);
     const TC h02 = hh[0] * hh[0], h12 = hh[1] * hh[1];
-    const TC st1 = gx[1], st2 = gy[0], st3 = (gx[0] * h02 - gy[1] * h12) / (h02 + h12);
+    const TC st1 = gx[1], st2 = gy[0], st3 = (gx[0] * h02 - gy[1] * h12) * rcpv(h02 + h12);
     const TC dbx[2] = {a3, a1}, dby[2] = {a2, -a3};
     const TC sbx[2] = {st3, st1}, sby[2] = {st2, -st3};
-    const TC wd = TC(1) / sqrt(TC(kWenoEps) + weno_osc<TC, 2>(W[4], nbx, dbx, hh) +
+    const TC wd = rsqrtp(TC(kWenoEps) + weno_osc<TC, 2>(W[4], nbx, dbx, hh) +
                                weno_osc<TC, 2>(W[5], nby, dby, hh));
-    const TC ws = TC(1) / sqrt(TC(kWenoEps) + weno_osc<TC, 2>(W[4], nbx, sbx, hh) +
+    const TC ws = rsqrtp(TC(kWenoEps) + weno_osc<TC, 2>(W[4], nbx, sbx, hh) +
                                weno_osc<TC, 2>(W[5], nby, sby, hh));
-    const TC iw = TC(1) / (wd + ws);
+    const TC iw = rcpv(wd + ws);
     a1 = (wd * a1 + ws * st1) * iw;
     a2 = (wd * a2 + ws * st2) * iw;
     a3 = (wd * a3 + ws * st3) * iw;
@@ -151,7 +148,7 @@ __device__ __forceinline__ void weno_cell2d(const Gas<TC>& G, const TC* hh, cons
 template <class TC>
 __device__ __forceinline__ void weno_cell3d(const Gas<TC>& G, const TC* hh, const TC* W,
                                             const TC (*Wn)[5], TC* s, TC* gout) {
-  const TC rho = W[0], inv = TC(1) / rho;
+  const TC rho = W[0], inv = rcpv(rho);
   const TC v[3] = {W[1], W[2], W[3]};
   const TC v2h = TC(0.5) * (v[0] * v[0] + v[1] * v[1] + v[2] * v[2]);
   TC g[5][3];
@@ -168,15 +165,13 @@ __device__ __forceinline__ void weno_cell3d(const Gas<TC>& G, const TC* hh, cons
   }
 #pragma unroll
   for (int q = 0; q < 5; ++q) {
-    TC hi = W[q], lo = W[q];
+    Extremes<TC> ex(W[q]);
     TC nb[6];
 #pragma unroll
-    for (int k = 0; k < 6; ++k) {
-      nb[k] = Wn[k][q];
-      hi = nb[k] > hi ? nb[k] : hi;
-      lo = nb[k] < lo ? nb[k] : lo;
-    }
-    weno_blend<TC, 3>(W[q], hi, lo, nb, hh, g[q]);
+    for (int k = 0; k < 6; ++k) nb[k] = Wn[k][q];
+#pragma unroll
+    for (int k = 0; k < 6; k += 2) ex.add(nb[k], nb[k + 1]);
+    weno_blend<TC, 3>(W[q], ex.max(), ex.min(), nb, hh, g[q]);
   }
 #pragma unroll
   for (int d = 0; d < 3; ++d) {

@@ -13,7 +13,7 @@ CSRC = os.path.join(PKG, "csrc")
 ROOT = os.path.dirname(PKG)
 OBJ = os.path.join(PKG, "_build")
 LIB = os.path.join(PKG, "libdg.so")
-SOURCES = ["dg_capi.cu", "dg_misc.cu", "dg_k2d.cu", "dg_k3d.cu", "dg_k3m.cu", "dg_kmh.cu", "dg_kmh3d.cu",
+SOURCES = ["dg_capi.cu", "dg_misc.cu", "dg_load.cu", "dg_k2d.cu", "dg_k3d.cu", "dg_k3m.cu", "dg_kmh.cu", "dg_kmh3d.cu",
            "dg_kmh3m.cu", "dg_adjoint.cu",
            "dg_noalloc.cu", "dg_batch.cu", "dg_peak.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]

@@ -59,6 +59,11 @@ struct dg_ctx {
   Ctl* ctl = nullptr;       // device, one per problem
   Ctl* ctl_host = nullptr;  // pinned mirror for readback
   double* scratch = nullptr;  // device, one interchange plane (host transfers, totals)
+  double* stage = nullptr;    // device, all interchange planes (pageable host transfers of
+                              // states up to kStageElems; allocated by the first one)
+  LoadProb* ltab = nullptr;   // device, work list of the state load and save launches
+  LoadAcc* lacc = nullptr;    // device, one per problem
+  int lblocks = 0;
   size_t scratch_elems = 0;
   double* totals_dev = nullptr;
   int variant = -1;  // tile shape (-1: not tuned yet)
@@ -199,6 +204,25 @@ dg_status alloc_ctx(dg_ctx* c) {
   CK(c, cudaMemset(c->ctl, 0, c->probs.size() * sizeof(Ctl)));
   CK(c, cudaMallocHost(&c->ctl_host, c->probs.size() * sizeof(Ctl)));
   CK(c, cudaMalloc(&c->totals_dev, 16 * sizeof(double)));
+  std::vector<LoadProb> tab;
+  for (auto& p : c->probs) {
+    LoadProb l;
+    l.ncell = p.ncell;
+    l.c0_off = (long)p.c0_off;
+    l.sl_off = (long)p.sl_off;
+    l.plane_off = (long)p.plane_off;
+    l.ih[0] = 1.0 / p.dx;
+    l.ih[1] = 1.0 / p.dy;
+    l.ih[2] = 1.0 / p.dz;
+    l.blk0 = c->lblocks;
+    l.nblk = load_blocks(p.ncell);
+    c->lblocks += l.nblk;
+    tab.push_back(l);
+  }
+  CK(c, cudaMalloc(&c->ltab, tab.size() * sizeof(LoadProb)));
+  CK(c, cudaMemcpy(c->ltab, tab.data(), tab.size() * sizeof(LoadProb), cudaMemcpyHostToDevice));
+  CK(c, cudaMalloc(&c->lacc, tab.size() * sizeof(LoadAcc)));
+  CK(c, cudaMemset(c->lacc, 0, tab.size() * sizeof(LoadAcc)));
   return DG_OK;
 }
 
@@ -403,9 +427,8 @@ dg_status read_ctl(dg_ctx* c) {
   return DG_OK;
 }
 
-dg_status check_err(dg_ctx* c) {
-  dg_status s = read_ctl(c);
-  if (s != DG_OK) return s;
+// The error words of the host mirror of the control blocks.
+dg_status check_host_ctl(dg_ctx* c) {
   for (size_t p = 0; p < c->probs.size(); ++p) {
     unsigned e = c->ctl_host[p].err;
     if (e & ERR_TIMEOUT) {
@@ -429,24 +452,33 @@ dg_status check_err(dg_ctx* c) {
   return DG_OK;
 }
 
-// Initial Courant speed of the current state of every problem.
-template <class TS>
-dg_status init_cfl_t(dg_ctx* c) {
-  for (size_t ip = 0; ip < c->probs.size(); ++ip) {
-    const Prob& p = c->probs[ip];
-    CK(c, launch_cfl<TS>(c->eq, c->dim, sbuf<TS>(c, c->cur, p), p.nx, p.ny, p.nz, p.dx, p.dy, p.dz,
-                         c->gamma, c->ctl + ip, c->stream));
-  }
-  return DG_OK;
+dg_status check_err(dg_ctx* c) {
+  dg_status s = read_ctl(c);
+  return s != DG_OK ? s : check_host_ctl(c);
 }
 
-dg_status reset_ctl_and_cfl(dg_ctx* c) {
-  CK(c, launch_ctl_reset(c->ctl, (int)c->probs.size(), c->stream));
+// The state of every problem from the device-readable interchange planes src (null: it
+// is in place already), with its Courant speed and fresh control blocks, mirrored on
+// the host once the stream has run.
+template <class TS>
+dg_status load_state_t(dg_ctx* c, const double* src) {
   if (c->bar) CK(c, cudaMemsetAsync(c->bar, 0, 2 * sizeof(unsigned), c->stream));
-  dg_status s = c->fp32 ? init_cfl_t<float>(c) : init_cfl_t<double>(c);
-  if (s != DG_OK) return s;
-  CK(c, launch_ctl_commit(c->ctl, (int)c->probs.size(), c->cfl, c->stream));
+  LoadArgs<TS> a;
+  a.src = src;
+  a.c0 = c->c0[c->cur];
+  a.sl = reinterpret_cast<TS*>(c->sl[c->cur]);
+  a.tab = c->ltab;
+  a.nprob = (int)c->probs.size();
+  a.gas.set(c->gamma);
+  a.cfl = c->cfl;
+  a.acc = c->lacc;
+  a.ctl = c->ctl;
+  a.host = c->ctl_host;
+  CK(c, launch_state_load<TS>(c->eq, c->dim, c->lblocks, a, c->stream));
   return DG_OK;
+}
+dg_status reset_ctl_and_cfl(dg_ctx* c) {
+  return c->fp32 ? load_state_t<float>(c, nullptr) : load_state_t<double>(c, nullptr);
 }
 
 // ---------------------------------------------------------------------------
@@ -578,32 +610,42 @@ static void* mapped_view(const void* host) {
   return a.type == cudaMemoryTypeHost ? a.devicePointer : nullptr;
 }
 
+// Pageable host memory up to this many elements (64 MB) crosses in one copy through a
+// device buffer kept by the context; larger states plane by plane through `scratch`.
+constexpr size_t kStageElems = size_t(8) << 20;
+static double* stage_buffer(dg_ctx* c) {
+  const size_t n = (size_t)c->nplanes * c->ncell_total;
+  if (n > kStageElems) return nullptr;
+  if (!c->stage && cudaMalloc(&c->stage, n * sizeof(double)) != cudaSuccess) {
+    cudaGetLastError();
+    c->stage = nullptr;
+  }
+  return c->stage;
+}
+
 template <class TS>
 static dg_status set_state_t(dg_ctx* c, const double* src, int on_device) {
   if (!on_device) {
     if (const double* view = static_cast<const double*>(mapped_view(src))) {
       src = view;
       on_device = 1;
+    } else if (double* st = stage_buffer(c)) {
+      CK(c, cudaMemcpyAsync(st, src, (size_t)c->nplanes * c->ncell_total * sizeof(double),
+                            cudaMemcpyHostToDevice, c->stream));
+      src = st;
+      on_device = 1;
     }
   }
+  if (on_device) return load_state_t<TS>(c, src);
   for (const Prob& p : c->probs) {
     StateBuf<TS> dst = sbuf<TS>(c, c->cur, p);
-    if (on_device) {
-      CK(c, launch_state_in<TS>(src + p.plane_off, dst, c->pmap, p.ncell, c->stream));
-      continue;
-    }
     for (int k = 0; k < c->nplanes; ++k) {
-      const double* plane = src + p.plane_off + (size_t)k * p.ncell;
-      const double* dsrc = plane;
-      if (!on_device) {
-        CK(c, cudaMemcpyAsync(c->scratch, plane, p.ncell * sizeof(double), cudaMemcpyHostToDevice,
-                              c->stream));
-        dsrc = c->scratch;
-      }
-      CK(c, launch_plane_in<TS>(dsrc, dst, c->pmap.kind[k], c->pmap.idx[k], p.ncell, c->stream));
+      CK(c, cudaMemcpyAsync(c->scratch, src + p.plane_off + (size_t)k * p.ncell,
+                            p.ncell * sizeof(double), cudaMemcpyHostToDevice, c->stream));
+      CK(c, launch_plane_in<TS>(c->scratch, dst, c->pmap.kind[k], c->pmap.idx[k], p.ncell, c->stream));
     }
   }
-  return DG_OK;
+  return load_state_t<TS>(c, nullptr);
 }
 
 template <class TS>
@@ -614,19 +656,23 @@ static dg_status get_state_t(dg_ctx* c, double* dst, int on_device) {
       on_device = 1;
     }
   }
-  for (const Prob& p : c->probs) {
-    StateBuf<TS> src = sbuf<TS>(c, c->cur, p);
-    if (on_device) {
-      CK(c, launch_state_out<TS>(src, dst + p.plane_off, c->pmap, p.ncell, c->stream));
-      continue;
-    }
-    for (int k = 0; k < c->nplanes; ++k) {
-      double* plane = dst + p.plane_off + (size_t)k * p.ncell;
-      double* ddst = on_device ? plane : c->scratch;
-      CK(c, launch_plane_out<TS>(src, ddst, c->pmap.kind[k], c->pmap.idx[k], p.ncell, c->stream));
-      if (!on_device)
-        CK(c, cudaMemcpyAsync(plane, c->scratch, p.ncell * sizeof(double), cudaMemcpyDeviceToHost,
-                              c->stream));
+  double* st = on_device ? dst : stage_buffer(c);
+  if (st) {
+    CK(c, launch_state_save<TS>(c->eq, c->dim, c->lblocks, c->ltab, (int)c->probs.size(),
+                                c->c0[c->cur], reinterpret_cast<const TS*>(c->sl[c->cur]), st,
+                                c->stream));
+    if (st != dst)
+      CK(c, cudaMemcpyAsync(dst, st, (size_t)c->nplanes * c->ncell_total * sizeof(double),
+                            cudaMemcpyDeviceToHost, c->stream));
+  } else {
+    for (const Prob& p : c->probs) {
+      StateBuf<TS> src = sbuf<TS>(c, c->cur, p);
+      for (int k = 0; k < c->nplanes; ++k) {
+        CK(c, launch_plane_out<TS>(src, c->scratch, c->pmap.kind[k], c->pmap.idx[k], p.ncell,
+                                   c->stream));
+        CK(c, cudaMemcpyAsync(dst + p.plane_off + (size_t)k * p.ncell, c->scratch,
+                              p.ncell * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
+      }
     }
   }
   CK(c, cudaStreamSynchronize(c->stream));
@@ -779,6 +825,9 @@ void dg_destroy(dg_ctx* c) {
     cudaFree(c->sl[b]);
   }
   cudaFree(c->scratch);
+  cudaFree(c->stage);
+  cudaFree(c->ltab);
+  cudaFree(c->lacc);
   cudaFree(c->ctl);
   cudaFree(c->totals_dev);
   for (int v = 0; v < 3; ++v) cudaFree(c->btab[v]);
@@ -797,11 +846,10 @@ dg_status dg_set_state(dg_ctx* c, const double* coeffs, int on_device) {
   dg_status s = c->fp32 ? set_state_t<float>(c, coeffs, on_device)
                         : set_state_t<double>(c, coeffs, on_device);
   if (s != DG_OK) return s;
-  s = reset_ctl_and_cfl(c);
-  if (s != DG_OK) return s;
   adjoint_reset(c->adj);
   c->state_set = true;
-  s = check_err(c);
+  CK(c, cudaStreamSynchronize(c->stream));  // the launch has filled ctl_host
+  s = check_host_ctl(c);
   if (s != DG_OK) return s;
   return autotune(c);
 }

@@ -72,13 +72,39 @@ template <class TS>
 cudaError_t launch_plane_out(StateBuf<TS> src, double* dst, int kind, int idx, long ncell,
                              cudaStream_t st);
 
-// Courant signal speed of a state: max over cells of sum_d (|v_d| + c_d)/dx_d into
-// ctl->vmax_next (atomic max); then commit moves it to vmax_cur.
+// A whole context's state in (layout, Courant speed, reset and commit of the control
+// blocks and their host copy) or out, one launch for all problems (dg_load.cu).
+struct LoadProb {
+  long ncell;
+  long c0_off, sl_off;  // element offsets inside the state arrays
+  long plane_off;       // offset in the concatenated interchange array
+  double ih[3];         // 1 / cell size
+  int blk0, nblk;       // this problem's blocks of the launch
+};
+// Accumulators of one problem: zero between launches.
+struct LoadAcc {
+  unsigned long long vmax;
+  unsigned err, ticket;
+};
 template <class TS>
-cudaError_t launch_cfl(int eq, int dim, StateBuf<TS> s, int nx, int ny, int nz, double dx,
-                       double dy, double dz, double gamma, Ctl* ctl, cudaStream_t st);
-cudaError_t launch_ctl_reset(Ctl* ctl, int nprob, cudaStream_t st);
-cudaError_t launch_ctl_commit(Ctl* ctl, int nprob, double cfl, cudaStream_t st);
+struct LoadArgs {
+  const double* src;  // interchange planes, or null: the state is already in place
+  double* c0;
+  TS* sl;
+  const LoadProb* tab;
+  int nprob;
+  GasPair gas;
+  double cfl;
+  LoadAcc* acc;
+  Ctl* ctl;
+  Ctl* host;  // page-locked mirror of ctl
+};
+int load_blocks(long ncell);
+template <class TS>
+cudaError_t launch_state_load(int eq, int dim, int blocks, const LoadArgs<TS>& A, cudaStream_t st);
+template <class TS>
+cudaError_t launch_state_save(int eq, int dim, int blocks, const LoadProb* tab, int nprob,
+                              const double* c0, const TS* sl, double* dst, cudaStream_t st);
 
 // Neumaier-compensated FP64 sums of the average planes: out[v] = sum_cells c0[v].
 cudaError_t launch_totals(const double* c0, int nv, long ncell, double* partial, double* out,

@@ -113,115 +113,6 @@ template cudaError_t launch_plane_out<float>(StateBuf<float>, double*, int, int,
                                              cudaStream_t);
 
 // ---------------------------------------------------------------------------
-// Courant signal speed of a state (used when a state is set; during stepping
-// the same reduction is fused into stage 2).  Arithmetic in TC = TS, as in the
-// fused reduction of the stage kernels.
-// ---------------------------------------------------------------------------
-template <class TS>
-__global__ void cfl_kernel(int eq, int dim, StateBuf<TS> s, int nx, int ny, int nz, double dx,
-                           double dy, double dz, double gamma, Ctl* ctl) {
-  using TC = TS;
-  Gas<TC> G;
-  G.set(gamma);
-  const long ncell = (long)nx * ny * nz;
-  double m = 0.0;
-  unsigned err = 0;
-  for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < ncell;
-       i += (long)gridDim.x * blockDim.x) {
-    TC rho = (TC)s.c0[i];
-    TC inv = TC(1) / rho;
-    TC vx = (TC)s.c0[ncell + i] * inv, vy = (TC)s.c0[2 * ncell + i] * inv, vz = TC(0);
-    TC kin = TC(0.5) * ((TC)s.c0[ncell + i] * vx + (TC)s.c0[2 * ncell + i] * vy);
-    int ie = 3;
-    if (dim == 3) {
-      vz = (TC)s.c0[3 * ncell + i] * inv;
-      kin = TC(0.5) * ((TC)s.c0[ncell + i] * vx + (TC)s.c0[2 * ncell + i] * vy +
-                       (TC)s.c0[3 * ncell + i] * vz);
-      ie = 4;
-    }
-    TC bx = TC(0), by = TC(0), bz = TC(0), mag = TC(0);
-    if (eq == 1) {
-      const int ib = ie + 1;  // the field averages follow the energy
-      bx = (TC)s.c0[ib * ncell + i];
-      by = (TC)s.c0[(ib + 1) * ncell + i];
-      if (dim == 3) bz = (TC)s.c0[(ib + 2) * ncell + i];
-      mag = TC(0.5) * (bx * bx + by * by + bz * bz);
-    }
-    TC p = G.gm1 * ((TC)s.c0[ie * ncell + i] - kin - mag);
-    // a non-finite density or pressure is as non-physical as a negative one (an
-    // infinite density would give a zero signal speed)
-    if (!(rho > TC(0) && p > TC(0) && rho < TC(INFINITY) && p < TC(INFINITY))) {
-      err |= ERR_NONPHYS;
-      continue;
-    }
-    TC sp;
-    if (eq == 1) {
-      TC b2 = bx * bx + by * by + bz * bz;
-      sp = (fabs(vx) + fast_speed(G, rho, p, b2, bx)) / (TC)dx +
-           (fabs(vy) + fast_speed(G, rho, p, b2, by)) / (TC)dy;
-      if (dim == 3) sp += (fabs(vz) + fast_speed(G, rho, p, b2, bz)) / (TC)dz;
-    } else {
-      TC c = sqrt(G.g * p / rho);
-      sp = (fabs(vx) + c) / (TC)dx + (fabs(vy) + c) / (TC)dy;
-      if (dim == 3) sp += (fabs(vz) + c) / (TC)dz;
-    }
-    m = (double)sp > m ? (double)sp : m;
-  }
-  for (int o = 16; o > 0; o >>= 1) {
-    double t = __shfl_xor_sync(0xffffffffu, m, o);
-    m = t > m ? t : m;
-  }
-  if ((threadIdx.x & 31) == 0) atomicMax(&ctl->vmax_next, (unsigned long long)__double_as_longlong(m));
-  if (err) atomicOr(&ctl->err, err);
-}
-
-template <class TS>
-cudaError_t launch_cfl(int eq, int dim, StateBuf<TS> s, int nx, int ny, int nz, double dx,
-                       double dy, double dz, double gamma, Ctl* ctl, cudaStream_t st) {
-  long n = (long)nx * ny * nz;
-  cfl_kernel<TS><<<grid_for(n, 256), 256, 0, st>>>(eq, dim, s, nx, ny, nz, dx, dy, dz, gamma, ctl);
-  return cudaGetLastError();
-}
-template cudaError_t launch_cfl<double>(int, int, StateBuf<double>, int, int, int, double, double,
-                                        double, double, Ctl*, cudaStream_t);
-template cudaError_t launch_cfl<float>(int, int, StateBuf<float>, int, int, int, double, double,
-                                       double, double, Ctl*, cudaStream_t);
-
-__global__ void ctl_reset_kernel(Ctl* ctl, int nprob) {
-  int p = blockIdx.x * blockDim.x + threadIdx.x;
-  if (p < nprob) {
-    ctl[p].vmax_cur = 0.0;
-    ctl[p].dt_cur = 0.0;
-    ctl[p].vmax_next = 0ull;
-    ctl[p].t = 0.0;
-    ctl[p].dt_last = 0.0;
-    ctl[p].step = 0;
-    ctl[p].ticket = 0u;
-    ctl[p].err = 0u;
-    ctl[p].err_step = -1;
-  }
-}
-__global__ void ctl_commit_kernel(Ctl* ctl, int nprob, double cfl) {
-  int p = blockIdx.x * blockDim.x + threadIdx.x;
-  if (p < nprob) {
-    double vm = __longlong_as_double((long long)ctl[p].vmax_next);
-    ctl[p].vmax_cur = vm;
-    ctl[p].dt_cur = cfl / vm;
-    ctl[p].vmax_next = 0ull;
-    if (!(vm > 0.0)) ctl[p].err |= ERR_NONPHYS;
-    if (ctl[p].err && ctl[p].err_step < 0) ctl[p].err_step = ctl[p].step;
-  }
-}
-cudaError_t launch_ctl_reset(Ctl* ctl, int nprob, cudaStream_t st) {
-  ctl_reset_kernel<<<(nprob + 127) / 128, 128, 0, st>>>(ctl, nprob);
-  return cudaGetLastError();
-}
-cudaError_t launch_ctl_commit(Ctl* ctl, int nprob, double cfl, cudaStream_t st) {
-  ctl_commit_kernel<<<(nprob + 127) / 128, 128, 0, st>>>(ctl, nprob, cfl);
-  return cudaGetLastError();
-}
-
-// ---------------------------------------------------------------------------
 // Neumaier-compensated totals: per block (sum, compensation) pairs, then one
 // block combines the partials in a fixed order (deterministic).
 // ---------------------------------------------------------------------------

@@ -620,41 +620,42 @@ __device__ __forceinline__ void hlld_core(const Gas<T>& G, T rL, T uL, const T* 
   const T SL = (lt ? uL : uR) - cmax, SR = (lt ? uR : uL) + cmax;
   const T dL = SL - uL, dR = SR - uR;
   const T mL = rL * dL, mR = rR * dR;  // mass fluxes through the fast waves
-  const T iden = rcpv(mR - mL);
-  const T SM = (mR * uR - mL * uL - pTR + pTL) * iden;
-  const T pTs = (mR * pTL - mL * pTR + mL * mR * (uR - uL)) * iden;
+  // contact speed and total pressure of the star region, as corrections of the left
+  // state (small jumps lose nothing to cancellation): jK = SM - uK
+  const T du = uR - uL;
+  const T jL = (mR * du - (pTR - pTL)) * rcpv(mR - mL), jR = jL - du;
+  const T SM = uL + jL;
+  const T pTs = pTL + mL * jL;
   // single-star transverse states of both sides
   T vsL[NT], bsL[NT], vsR[NT], bsR[NT];
-  const T eL = SL - SM, eR = SR - SM;
+  const T eL = dL - jL, eR = dR - jR;  // S - SM
   const T iL = rcpv(eL), iR = rcpv(eR);
   const T rsL = mL * iL, rsR = mR * iR;
   bool degL, degR;
   {
-    const T mm = mL * dL, dd = mL * eL - bn2;
-    degL = fabs(dd) < Prec<T>::hlld_degenerate * (mm + bn2);
-    // (m d - bn^2) / dd = 1 + m (SM - u) / dd, without the cancellation
-    const T k = (SM - uL) * rcpv(dd);
-    const T tv = bn * k, tb = mL * k + T(1);
+    const T dd = mL * eL - bn2;
+    degL = fabs(dd) < Prec<T>::hlld_degenerate * (mL * dL + bn2);
+    const T k = jL * rcpv(dd);
+    const T tv = bn * k, tb = mL * k;  // tb + 1 = (m d - bn^2) / dd
 #pragma unroll
     for (int a = 0; a < NT; ++a) {
       vsL[a] = degL ? vL[a] : vL[a] - btL[a] * tv;
-      bsL[a] = degL ? btL[a] : btL[a] * tb;
+      bsL[a] = degL ? btL[a] : btL[a] + btL[a] * tb;
     }
   }
   {
-    const T mm = mR * dR, dd = mR * eR - bn2;
-    degR = fabs(dd) < Prec<T>::hlld_degenerate * (mm + bn2);
-    // (m d - bn^2) / dd = 1 + m (SM - u) / dd, without the cancellation
-    const T k = (SM - uR) * rcpv(dd);
-    const T tv = bn * k, tb = mR * k + T(1);
+    const T dd = mR * eR - bn2;
+    degR = fabs(dd) < Prec<T>::hlld_degenerate * (mR * dR + bn2);
+    const T k = jR * rcpv(dd);
+    const T tv = bn * k, tb = mR * k;
 #pragma unroll
     for (int a = 0; a < NT; ++a) {
       vsR[a] = degR ? vR[a] : vR[a] - btR[a] * tv;
-      bsR[a] = degR ? btR[a] : btR[a] * tb;
+      bsR[a] = degR ? btR[a] : btR[a] + btR[a] * tb;
     }
   }
   const T yL = rsqrtp(rsL), yR = rsqrtp(rsR);
-  const T sqL = rsL * yL, sqR = rsR * yR;
+  const T sqL = rsL * yL, sqR = rsR * yR;  // sqrt(rho*)
   const T abn = fabs(bn);
   // the side and the region
   const bool left = !negv(SM);
@@ -689,20 +690,22 @@ __device__ __forceinline__ void hlld_core(const Gas<T>& G, T rL, T uL, const T* 
     T vBs = SM * bn;
 #pragma unroll
     for (int a = 0; a < NT; ++a) vBs += v[a] * b[a];
-    const T dK = left ? dL : dR, iK = left ? iL : iR;
+    const T dK = left ? dL : dR, iK = left ? iL : iR, jK = left ? jL : jR;
     E = (dK * EK - pTK * uK + pTs * SM + bn * (vB - vBs)) * iK;
     const bool deg = left ? degL : degR;
 #pragma unroll
-    for (int a = 0; a < NT; ++a) extra[a] = deg ? b[a] * (uK - SM) : T(0);
+    for (int a = 0; a < NT; ++a) extra[a] = deg ? -b[a] * jK : T(0);
     vBf = vBs;
     if (!single) {  // between the Alfven waves
       const T sg = bn > T(0) ? T(1) : (bn < T(0) ? T(-1) : T(0));
-      const T inv = rcpv(sqL + sqR), sqLR = sqL * sqR;
+      const T inv = rcpv(sqL + sqR);
       T vBss = SM * bn;
 #pragma unroll
       for (int a = 0; a < NT; ++a) {
-        v[a] = (sqL * vsL[a] + sqR * vsR[a] + (bsR[a] - bsL[a]) * sg) * inv;
-        b[a] = (sqL * bsR[a] + sqR * bsL[a] + sqLR * (vsR[a] - vsL[a]) * sg) * inv;
+        // v** - v*_L, and b** - b*_L = sqrt(rho*_L) sign(bn) (v** - v*_L)
+        const T q = (sqR * (vsR[a] - vsL[a]) + (bsR[a] - bsL[a]) * sg) * inv;
+        v[a] = vsL[a] + q;
+        b[a] = bsL[a] + sqL * sg * q;
         vBss += v[a] * b[a];
       }
       E += (left ? -sqL : sqR) * (vBs - vBss) * sg;

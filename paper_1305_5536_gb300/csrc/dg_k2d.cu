@@ -12,30 +12,30 @@
 
 namespace dgk {
 
-template <int EQ, class TC, class TS, int TX, int TY, bool WENO>
+template <int EQ, class TC, class TS, int TX, int TY, bool WENO, int NT>
 static cudaError_t launch2d_w(int stage, const Stage2DArgs<TS>& a, cudaStream_t st) {
-  constexpr size_t smem = stage2d_smem_bytes<EQ, TX, TY, TC>();
+  constexpr size_t smem = stage2d_smem_bytes<EQ, TX, TY, TC, NT>();
   static_assert(smem <= 227 * 1024, "tile too large for shared memory");
   static bool attr_set = false;
   if (!attr_set) {
-    cudaError_t e1 = cudaFuncSetAttribute(stage2d_kernel<EQ, TC, TS, TX, TY, 1, WENO>,
+    cudaError_t e1 = cudaFuncSetAttribute(stage2d_kernel<EQ, TC, TS, TX, TY, 1, WENO, NT>,
                                           cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    cudaError_t e2 = cudaFuncSetAttribute(stage2d_kernel<EQ, TC, TS, TX, TY, 2, WENO>,
+    cudaError_t e2 = cudaFuncSetAttribute(stage2d_kernel<EQ, TC, TS, TX, TY, 2, WENO, NT>,
                                           cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e1 != cudaSuccess) return e1;
     if (e2 != cudaSuccess) return e2;
     attr_set = true;
   }
   dim3 grid((a.nx + TX - 1) / TX, (a.ny + TY - 1) / TY);
-  if (stage == 1) return launch_pdl(stage2d_kernel<EQ, TC, TS, TX, TY, 1, WENO>, grid, TX * TY, smem, st, a);
-  return launch_pdl(stage2d_kernel<EQ, TC, TS, TX, TY, 2, WENO>, grid, TX * TY, smem, st, a);
+  if (stage == 1) return launch_pdl(stage2d_kernel<EQ, TC, TS, TX, TY, 1, WENO, NT>, grid, NT, smem, st, a);
+  return launch_pdl(stage2d_kernel<EQ, TC, TS, TX, TY, 2, WENO, NT>, grid, NT, smem, st, a);
 }
 
 // The WENO-type limiter only in the instantiation that needs it.
-template <int EQ, class TC, class TS, int TX, int TY>
+template <int EQ, class TC, class TS, int TX, int TY, int NT = TX * TY>
 static cudaError_t launch2d(int stage, const Stage2DArgs<TS>& a, cudaStream_t st) {
-  if (a.limiter == 2) return launch2d_w<EQ, TC, TS, TX, TY, true>(stage, a, st);
-  return launch2d_w<EQ, TC, TS, TX, TY, false>(stage, a, st);
+  if (a.limiter == 2) return launch2d_w<EQ, TC, TS, TX, TY, true, NT>(stage, a, st);
+  return launch2d_w<EQ, TC, TS, TX, TY, false, NT>(stage, a, st);
 }
 
 // ---------------------------------------------------------------------------
@@ -131,12 +131,16 @@ static cudaError_t launch2d_tma(int stage, const Stage2DArgs<TS>& a, cudaStream_
 
 // Tile shapes per precision (variant 0 is the default before tuning); variants 3
 // and 4 are the persistent TMA kernels (grids whose rows are 16-byte aligned).
-int stage2d_variants(int, int) { return 5; }
+// FP64 variants 5 and 6 are small tiles with four threads per cell: a grid of a few
+// thousand cells then covers every SM, and the four FP64 pipes of each share a tile's
+// faces and volume points (one warp keeps one pipe busy for 64 cycles an instruction).
+int stage2d_variants(int, int fp32) { return fp32 ? 5 : 7; }
 
 const char* stage2d_variant_name(int, int fp32, int v) {
-  static const char* n64[] = {"16x8", "8x8", "32x4", "tma16x8", "tma32x4"};
+  static const char* n64[] = {"16x8", "8x8", "32x4", "tma16x8", "tma32x4", "8x4 (4 threads a cell)",
+                              "8x8 (4 threads a cell)"};
   static const char* n32[] = {"16x16", "32x8", "16x8", "tma16x8", "tma16x16"};
-  if (v < 0 || v > 4) return "?";
+  if (v < 0 || v > (fp32 ? 4 : 6)) return "?";
   return fp32 ? n32[v] : n64[v];
 }
 
@@ -148,6 +152,8 @@ cudaError_t launch_stage2d(int eq, int variant, int stage, const Stage2DArgs<dou
       case 2: return launch2d<0, double, double, 32, 4>(stage, a, st);
       case 3: return launch2d_tma<0, double, double, 16, 8>(stage, a, st);
       case 4: return launch2d_tma<0, double, double, 32, 4>(stage, a, st);
+      case 5: return launch2d<0, double, double, 8, 4, 128>(stage, a, st);
+      case 6: return launch2d<0, double, double, 8, 8, 256>(stage, a, st);
       default: return launch2d<0, double, double, 16, 8>(stage, a, st);
     }
   }
@@ -156,6 +162,8 @@ cudaError_t launch_stage2d(int eq, int variant, int stage, const Stage2DArgs<dou
     case 2: return launch2d<1, double, double, 32, 4>(stage, a, st);
     case 3: return launch2d_tma<1, double, double, 16, 8>(stage, a, st);
     case 4: return launch2d_tma<1, double, double, 32, 4>(stage, a, st);
+    case 5: return launch2d<1, double, double, 8, 4, 128>(stage, a, st);
+    case 6: return launch2d<1, double, double, 8, 8, 256>(stage, a, st);
     default: return launch2d<1, double, double, 16, 8>(stage, a, st);
   }
 }

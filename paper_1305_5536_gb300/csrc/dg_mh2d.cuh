@@ -52,10 +52,11 @@ struct MhTile2D {
   static_assert(NV == NP, "the primitives replace the averages in place");
 };
 
-template <int EQ, int TX, int TY, int NGF, class TC>
+template <int EQ, int TX, int TY, int NGF, class TC, int NT = TX * TY>
 __host__ __device__ constexpr size_t mh2d_smem_bytes() {
   using T = Tile2D<EQ, TX, TY>;
-  return size_t(MhTile2D<EQ, TX, TY, NGF>::ELEMS) * sizeof(TC) + sizeof(int) * (T::R2X + T::R2Y);
+  return size_t(MhTile2D<EQ, TX, TY, NGF>::ELEMS) * sizeof(TC) + sizeof(int) * (T::R2X + T::R2Y) +
+         (NT == 4 * T::NT ? size_t(2 * T::NF) * T::NT * sizeof(TC) : 0);
 }
 
 template <class TC>
@@ -239,17 +240,17 @@ __device__ __forceinline__ void face_flux_prim2d(const Gas<TC>& G, int dir, cons
   else { F[1] = Ff[2]; F[2] = Ff[1]; }
 }
 
-template <int EQ, class TC, class TS, int TX, int TY, int NGF, bool WENO>
+template <int EQ, class TC, class TS, int TX, int TY, int NGF, bool WENO, int NT>
 __device__ __forceinline__ void mh2d_compute(const Stage2DArgs<TS>& A, int i0, int j0,
                                              unsigned nblk, const MhMem2D<TC>& MM,
-                                             TileScalars<TX * TY>& S) {
+                                             TileScalars<NT>& S) {
   using Tr = Tr2<EQ>;
   constexpr int NV = Tr::NV, NS = Tr::NS, NP = Tr::NP, NF = Tr::NF;
   constexpr int R2X = TX + 4, R2Y = TY + 4, R2 = R2X * R2Y;
   constexpr int R1X = TX + 2, R1Y = TY + 2, R1 = R1X * R1Y;
   constexpr int NFX = (TX + 1) * TY, NFY = TX * (TY + 1);
-  constexpr int NT = TX * TY;
-  static_assert(NT % 32 == 0, "tile must be whole warps");
+  constexpr int NC = TX * TY;  // cells; NT threads
+  static_assert(NC % 32 == 0 && NT % 32 == 0 && NT >= NC, "tile must be whole warps");
   static_assert(NGF == 1 || NGF == 2, "face rule: 1 or 2 points");
   (void)R2Y;
   (void)R1Y;
@@ -307,7 +308,7 @@ __device__ __forceinline__ void mh2d_compute(const Stage2DArgs<TS>& A, int i0, i
     if ((unsigned)(rx - 1) < (unsigned)TX && (unsigned)(ry - 1) < (unsigned)TY) {
       const int t = (ry - 1) * TX + rx - 1;
 #pragma unroll
-      for (int k = 0; k < NS; ++k) s_ls[k * NT + t] = s[k];
+      for (int k = 0; k < NS; ++k) s_ls[k * NC + t] = s[k];
     }
 #pragma unroll
     for (int q = 0; q < NP; ++q) s_wp[q * R1 + r1] = W[q] + hdt * Wt[q];
@@ -348,25 +349,54 @@ __device__ __forceinline__ void mh2d_compute(const Stage2DArgs<TS>& A, int i0, i
       for (int q = 0; q < NF; ++q) s_fy[(q * NFY + f) * NGF + gp] = F[q];
     }
   }
+  // ---- four threads per cell: one volume Gauss point each (as in dg_stage2d.cuh)
+  constexpr bool SPLIT = NT == 4 * NC;
+  TC* s_vol = reinterpret_cast<TC*>(MM.m.gy + R2Y);
+  static_assert(!SPLIT || (R2X + R2Y) % 2 == 0, "FP64 sums behind the offset tables");
+  if constexpr (SPLIT) {
+    const int cell = tid >> 2, qp = tid & 3, cy = cell / TX, cx = cell - cy * TX;
+    const int q1 = (cy + 1) * R1X + cx + 1;
+    TC W[NP], Fx[NF], Fy[NF];
+    mh_eval2d<EQ, TC>(s_wp + q1, s_g + q1, R1, (qp & 1) ? ox : -ox, (qp & 2) ? oy : -oy, W);
+    prim_flux2d<EQ, TC>(G, W, Fx, Fy, err);
+#pragma unroll
+    for (int q = 0; q < NF; ++q) {
+#pragma unroll
+      for (int o = 1; o < 4; o <<= 1) {
+        Fx[q] += __shfl_xor_sync(0xffffffffu, Fx[q], o);
+        Fy[q] += __shfl_xor_sync(0xffffffffu, Fy[q], o);
+      }
+      if (qp == 0) s_vol[q * NC + cell] = Fx[q];
+      if (qp == 1) s_vol[(NF + q) * NC + cell] = Fy[q];
+    }
+  }
   __syncthreads();
 
   // ---- 4. per cell: volume integral, face moments, mass matrix, update
-  const int lx = tid % TX, ly = tid / TX;
+  const bool mine = NT == NC || tid < NC;
+  const int lx = tid % TX, ly = mine ? tid / TX : 0;
   const int gi = i0 + lx, gj = j0 + ly;
-  const bool owner = gi < nx && gj < ny;
+  const bool owner = mine && gi < nx && gj < ny;
+  double o0[NV];
+  if (mine) {
   const int r1 = (ly + 1) * R1X + lx + 1;
   const size_t gc = (size_t)s_gy[ly + 2] + s_gx[lx + 2];
 
   TC sFx[NF], sFy[NF];
 #pragma unroll
   for (int q = 0; q < NF; ++q) { sFx[q] = TC(0); sFy[q] = TC(0); }
+  if constexpr (SPLIT) {
 #pragma unroll
-  for (int qp = 0; qp < 4; ++qp) {
-    TC W[NP], Fx[NF], Fy[NF];
-    mh_eval2d<EQ, TC>(s_wp + r1, s_g + r1, R1, (qp & 1) ? ox : -ox, (qp & 2) ? oy : -oy, W);
-    prim_flux2d<EQ, TC>(G, W, Fx, Fy, err);
+    for (int q = 0; q < NF; ++q) { sFx[q] = s_vol[q * NC + tid]; sFy[q] = s_vol[(NF + q) * NC + tid]; }
+  } else {
 #pragma unroll
-    for (int q = 0; q < NF; ++q) { sFx[q] += Fx[q]; sFy[q] += Fy[q]; }
+    for (int qp = 0; qp < 4; ++qp) {
+      TC W[NP], Fx[NF], Fy[NF];
+      mh_eval2d<EQ, TC>(s_wp + r1, s_g + r1, R1, (qp & 1) ? ox : -ox, (qp & 2) ? oy : -oy, W);
+      prim_flux2d<EQ, TC>(G, W, Fx, Fy, err);
+#pragma unroll
+      for (int q = 0; q < NF; ++q) { sFx[q] += Fx[q]; sFy[q] += Fy[q]; }
+    }
   }
 
   const int fxm = ly * (TX + 1) + lx, fym = ly * TX + lx;
@@ -404,18 +434,18 @@ __device__ __forceinline__ void mh2d_compute(const Stage2DArgs<TS>& A, int i0, i
   }
 
   // U^{n+1} = U^n + dt L, U^n the limited step input
-  double o0[NV];
   TC os[NS];
 #pragma unroll
   for (int v = 0; v < NV; ++v) o0[v] = fma(dt, Cvt<TC>::to_f64(rc0[v]), A.in.c0[v * ncell + gc]);
 #pragma unroll
-  for (int k = 0; k < NS; ++k) os[k] = s_ls[k * NT + tid] + dtc * rs[k];
+  for (int k = 0; k < NS; ++k) os[k] = s_ls[k * NC + tid] + dtc * rs[k];
   if (owner) {
 #pragma unroll
     for (int v = 0; v < NV; ++v) A.out.c0[v * ncell + gc] = o0[v];
 #pragma unroll
     for (int k = 0; k < NS; ++k) A.out.sl[k * ncell + gc] = (TS)os[k];
   }
+  }  // mine
   courant_commit2d<EQ, TC, TS, NT>(A, G, owner, o0, dt, nblk, err, S);
 }
 
@@ -427,20 +457,20 @@ struct MhMinBlocks {
   static constexpr int v = sizeof(TC) == 4 ? 65536 / (R * NT) : 1;
 };
 
-template <int EQ, class TC, class TS, int TX, int TY, int NGF, bool WENO>
-__global__ void __launch_bounds__(TX * TY, (MhMinBlocks<EQ, TX * TY, NGF, WENO, TC>::v))
+template <int EQ, class TC, class TS, int TX, int TY, int NGF, bool WENO, int NT = TX * TY>
+__global__ void __launch_bounds__(NT, (MhMinBlocks<EQ, NT, NGF, WENO, TC>::v))
     mh2d_kernel(const Stage2DArgs<TS> A) {
   griddep_launch_dependents();  // programmatic dependent launch: see griddep_wait()
   griddep_wait();
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  __shared__ TileScalars<TX * TY> S;
+  __shared__ TileScalars<NT> S;
   const MhMem2D<TC> M = mh2d_mem<EQ, TX, TY, NGF, TC>(smem_raw);
   const int i0 = blockIdx.x * TX, j0 = blockIdx.y * TY;
-  stage2d_setup<EQ, TC, TS, TX, TY>(A, i0, j0, M.m, S);
+  stage2d_setup<EQ, TC, TS, TX, TY, NT>(A, i0, j0, M.m, S);
   __syncthreads();
-  stage2d_load<EQ, TC, TS, TX, TY>(A, M.m);
+  stage2d_load<EQ, TC, TS, TX, TY, NT>(A, M.m);
   __syncthreads();
-  mh2d_compute<EQ, TC, TS, TX, TY, NGF, WENO>(A, i0, j0, gridDim.x * gridDim.y, M, S);
+  mh2d_compute<EQ, TC, TS, TX, TY, NGF, WENO, NT>(A, i0, j0, gridDim.x * gridDim.y, M, S);
 }
 
 }  // namespace dgk

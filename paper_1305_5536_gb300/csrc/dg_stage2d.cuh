@@ -58,10 +58,12 @@ struct Tile2D {
   static constexpr int ELEMS = NV * R2 + NS * R1 + WSZ;
 };
 
-template <int EQ, int TX, int TY, class TC>
+// NT = 4 TX TY (four threads per cell): also the volume sums [2 NF][TX TY].
+template <int EQ, int TX, int TY, class TC, int NT = TX * TY>
 __host__ __device__ constexpr size_t stage2d_smem_bytes() {
   using T = Tile2D<EQ, TX, TY>;
-  return size_t(T::ELEMS) * sizeof(TC) + sizeof(int) * (T::R2X + T::R2Y);
+  return size_t(T::ELEMS) * sizeof(TC) + sizeof(int) * (T::R2X + T::R2Y) +
+         (NT == 4 * T::NT ? size_t(2 * T::NF) * T::NT * sizeof(TC) : 0);
 }
 
 template <class TC>
@@ -244,10 +246,11 @@ __device__ __forceinline__ void face_flux2d(const Gas<TC>& G, int dir, const TC*
 
 // Start of a tile: the time step, the error word, and the wrapped global row and
 // column offsets of the halo-2 region.  The caller synchronises afterwards.
-template <int EQ, class TC, class TS, int TX, int TY>
+template <int EQ, class TC, class TS, int TX, int TY, int NT = TX * TY>
 __device__ __forceinline__ void stage2d_setup(const Stage2DArgs<TS>& A, int i0, int j0,
-                                              const TileMem<TC>& M, TileScalars<TX * TY>& S) {
+                                              const TileMem<TC>& M, TileScalars<NT>& S) {
   using T = Tile2D<EQ, TX, TY>;
+  static_assert(T::R2X + T::R2Y <= NT, "one thread per row and column offset");
   const int tid = threadIdx.x;
   if (tid == 0) {
     S.err = 0;
@@ -268,10 +271,23 @@ __device__ __forceinline__ void stage2d_setup(const Stage2DArgs<TS>& A, int i0, 
 // plain copies go through cp.async, and the FP64 averages of the FP32 path are
 // loaded into registers in chunks of 8 passes and converted after each chunk.
 // The caller synchronises.
-template <int EQ, class TC, class TS, int TX, int TY>
+template <int EQ, class TC, class TS, int TX, int TY, int NT = TX * TY>
 __device__ __forceinline__ void stage2d_load(const Stage2DArgs<TS>& A, const TileMem<TC>& M) {
   using T = Tile2D<EQ, TX, TY>;
   static_assert(sizeof(TS) == sizeof(TC), "derivative coefficients are staged as stored");
+  if constexpr (NT > T::NT) {  // several threads per cell (FP64): element by element
+    static_assert(sizeof(TC) == 8, "small tiles with several threads per cell are FP64");
+    for (int e = threadIdx.x; e < T::NS * T::R1; e += NT) {
+      const int v = e / T::R1, r = e - v * T::R1, ry = r / T::R1X, rx = r - ry * T::R1X;
+      cp_async_elem<8>(&M.sl[e], A.in.sl + (size_t)v * A.ncell + M.gy[ry + 1] + M.gx[rx + 1]);
+    }
+    for (int e = threadIdx.x; e < T::NV * T::R2; e += NT) {
+      const int v = e / T::R2, r = e - v * T::R2, ry = r / T::R2X, rx = r - ry * T::R2X;
+      cp_async_elem<8>(&M.c0[e], A.in.c0 + (size_t)v * A.ncell + M.gy[ry] + M.gx[rx]);
+    }
+    cp_async_wait_all();
+    return;
+  } else {
   constexpr int C1 = T::NT / T::R1X, C0 = T::NT / T::R2X;
   static_assert(C1 >= 1 && C1 <= T::R1Y && C0 >= 1 && C0 <= T::R2Y,
                 "a pass of rows advances by at most one variable");
@@ -325,6 +341,7 @@ __device__ __forceinline__ void stage2d_load(const Stage2DArgs<TS>& A, const Til
     }
   }
   cp_async_wait_all();
+  }
 }
 
 // Stage 2 reads the step's input state U^n of its own cell only at the end (the
@@ -334,6 +351,7 @@ __device__ __forceinline__ void stage2d_prefetch_base(const Stage2DArgs<TS>& A,
                                                       const TileMem<TC>& M) {
   using T = Tile2D<EQ, TX, TY>;
   const size_t ncell = (size_t)A.ncell;
+  if (threadIdx.x >= T::NT) return;
   const int lx = threadIdx.x % TX, ly = threadIdx.x / TX;
   const size_t gc = (size_t)M.gy[ly + 2] + M.gx[lx + 2];
   const TS* sl = A.limiter && A.lim_sl ? A.lim_sl : A.base.sl;
@@ -414,18 +432,18 @@ __device__ __forceinline__ void courant_commit2d(const Stage2DArgs<TS>& A, const
 // or 1: its code raises the registers and stack of the common path).
 // `ph` (profiling build): phases 1 primitives, 2 limiter, 3 faces, 4 per-cell
 // right-hand side and combination, 5 Courant reduction and commit.
-template <int EQ, class TC, class TS, int TX, int TY, int STAGE, bool WENO = true>
+template <int EQ, class TC, class TS, int TX, int TY, int STAGE, bool WENO = true, int NT = TX * TY>
 __device__ __forceinline__ void stage2d_compute(const Stage2DArgs<TS>& A, int i0, int j0,
                                                 unsigned nblk, const TileMem<TC>& M,
-                                                TileScalars<TX * TY>& S,
+                                                TileScalars<NT>& S,
                                                 PhaseStamp* ph = nullptr) {
   using Tr = Tr2<EQ>;
   constexpr int NV = Tr::NV, NS = Tr::NS, NP = Tr::NP, NF = Tr::NF;
   constexpr int R2X = TX + 4, R2Y = TY + 4, R2 = R2X * R2Y;
   constexpr int R1X = TX + 2, R1Y = TY + 2, R1 = R1X * R1Y;
   constexpr int NFX = (TX + 1) * TY, NFY = TX * (TY + 1);
-  constexpr int NT = TX * TY;
-  static_assert(NT % 32 == 0, "tile must be whole warps");
+  constexpr int NC = TX * TY;  // cells; NT threads
+  static_assert(NC % 32 == 0 && NT % 32 == 0 && NT >= NC, "tile must be whole warps");
   (void)R2Y;
   (void)R1Y;
   TC* s_c0 = M.c0;
@@ -521,17 +539,45 @@ __device__ __forceinline__ void stage2d_compute(const Stage2DArgs<TS>& A, int i0
       for (int q = 0; q < NF; ++q) s_fy[(q * NFY + f) * 2 + g] = F[q];
     }
   }
+  // ---- four threads per cell: one volume Gauss point each, summed over the four lanes
+  constexpr bool SPLIT = NT == 4 * NC;
+  TC* s_vol = reinterpret_cast<TC*>(M.gy + R2Y);
+  static_assert(!SPLIT || (R2X + R2Y) % 2 == 0, "FP64 sums behind the offset tables");
+  if constexpr (SPLIT) {
+    const int cell = tid >> 2, qp = tid & 3, cy = cell / TX, cx = cell - cy * TX;
+    const int q2 = (cy + 2) * R2X + cx + 2, q1 = (cy + 1) * R1X + cx + 1;
+    TC a0[NV], s[NS], c[NV], Fx[NF], Fy[NF];
+#pragma unroll
+    for (int v = 0; v < NV; ++v) a0[v] = s_c0[v * R2 + q2];
+#pragma unroll
+    for (int k = 0; k < NS; ++k) s[k] = s_sl[k * R1 + q1];
+    eval2d<EQ, TC>(a0, s, (qp & 1) ? ox : -ox, (qp & 2) ? oy : -oy, c);
+    phys_flux2d<EQ, TC>(G, c, Fx, Fy, err);
+#pragma unroll
+    for (int q = 0; q < NF; ++q) {
+#pragma unroll
+      for (int o = 1; o < 4; o <<= 1) {
+        Fx[q] += __shfl_xor_sync(0xffffffffu, Fx[q], o);
+        Fy[q] += __shfl_xor_sync(0xffffffffu, Fy[q], o);
+      }
+      if (qp == 0) s_vol[q * NC + cell] = Fx[q];
+      if (qp == 1) s_vol[(NF + q) * NC + cell] = Fy[q];
+    }
+  }
   __syncthreads();
   if (ph) ph->mark(3);
 
   // ---- per cell: volume integral, face moments, mass matrix, RK combination
-  const int lx = tid % TX, ly = tid / TX;
+  const bool mine = NT == NC || tid < NC;
+  const int lx = tid % TX, ly = mine ? tid / TX : 0;
   const int gi = i0 + lx, gj = j0 + ly;
-  const bool owner = gi < nx && gj < ny;
+  const bool owner = mine && gi < nx && gj < ny;
+  double o0[NV];
+  if (mine) {
   const int r2 = (ly + 2) * R2X + lx + 2, r1 = (ly + 1) * R1X + lx + 1;
   const size_t gc = (size_t)s_gy[ly + 2] + s_gx[lx + 2];
+  const TC dtc = Cvt<TC>::to_tc(S.dt);
   const double dt = S.dt;
-  const TC dtc = Cvt<TC>::to_tc(dt);
   TC c0[NV], s[NS];
 #pragma unroll
   for (int v = 0; v < NV; ++v) c0[v] = s_c0[v * R2 + r2];
@@ -541,13 +587,18 @@ __device__ __forceinline__ void stage2d_compute(const Stage2DArgs<TS>& A, int i0
   TC sFx[NF], sFy[NF];
 #pragma unroll
   for (int q = 0; q < NF; ++q) { sFx[q] = TC(0); sFy[q] = TC(0); }
+  if constexpr (SPLIT) {
 #pragma unroll
-  for (int qp = 0; qp < 4; ++qp) {
-    TC c[NV], Fx[NF], Fy[NF];
-    eval2d<EQ, TC>(c0, s, (qp & 1) ? ox : -ox, (qp & 2) ? oy : -oy, c);
-    phys_flux2d<EQ, TC>(G, c, Fx, Fy, err);
+    for (int q = 0; q < NF; ++q) { sFx[q] = s_vol[q * NC + tid]; sFy[q] = s_vol[(NF + q) * NC + tid]; }
+  } else {
 #pragma unroll
-    for (int q = 0; q < NF; ++q) { sFx[q] += Fx[q]; sFy[q] += Fy[q]; }
+    for (int qp = 0; qp < 4; ++qp) {
+      TC c[NV], Fx[NF], Fy[NF];
+      eval2d<EQ, TC>(c0, s, (qp & 1) ? ox : -ox, (qp & 2) ? oy : -oy, c);
+      phys_flux2d<EQ, TC>(G, c, Fx, Fy, err);
+#pragma unroll
+      for (int q = 0; q < NF; ++q) { sFx[q] += Fx[q]; sFy[q] += Fy[q]; }
+    }
   }
 
   const int fxm = ly * (TX + 1) + lx, fym = ly * TX + lx;
@@ -578,7 +629,6 @@ __device__ __forceinline__ void stage2d_compute(const Stage2DArgs<TS>& A, int i0
     rs[10] = geo.ax * (Dxp[4] - Dxm[4]) - geo.ay * (Dyp[4] - Dym[4]);
   }
 
-  double o0[NV];
   TC os[NS];
   if (STAGE == 1) {
     // V^1 = U^n + dt L(U^n), U^n = limited V^n
@@ -632,9 +682,10 @@ __device__ __forceinline__ void stage2d_compute(const Stage2DArgs<TS>& A, int i0
     for (int k = 0; k < NS; ++k) A.out.sl[k * ncell + gc] = (TS)os[k];
   }
 
+  }  // mine
   if (ph) ph->mark(4);
   if (STAGE == 2) {
-    courant_commit2d<EQ, TC, TS, NT>(A, G, owner, o0, dt, nblk, err, S);
+    courant_commit2d<EQ, TC, TS, NT>(A, G, owner, o0, S.dt, nblk, err, S);
   } else {
     if (err) atomicOr(&S.err, err);
     __syncthreads();
@@ -646,21 +697,22 @@ __device__ __forceinline__ void stage2d_compute(const Stage2DArgs<TS>& A, int i0
 
 
 // One tile of one stage (classic staging): the CTA owns cells [i0, i0+TX) x
-// [j0, j0+TY) of the problem described by A.
-template <int EQ, class TC, class TS, int TX, int TY, int STAGE, bool WENO = true>
+// [j0, j0+TY) of the problem described by A; NT threads (TX TY, or 4 TX TY for small
+// FP64 tiles).
+template <int EQ, class TC, class TS, int TX, int TY, int STAGE, bool WENO = true, int NT = TX * TY>
 __device__ __forceinline__ void stage2d_tile(const Stage2DArgs<TS>& A, int i0, int j0,
                                              unsigned nblk, unsigned char* smem_raw) {
-  __shared__ TileScalars<TX * TY> S;
+  __shared__ TileScalars<NT> S;
   PhaseStamp ph;  // phase 0: set-up and staging (profiling build)
   ph.begin(A.phase, STAGE);
   const TileMem<TC> M = tile_mem<EQ, TX, TY, TC>(smem_raw);
-  stage2d_setup<EQ, TC, TS, TX, TY>(A, i0, j0, M, S);
+  stage2d_setup<EQ, TC, TS, TX, TY, NT>(A, i0, j0, M, S);
   __syncthreads();
   if (STAGE == 2) stage2d_prefetch_base<EQ, TC, TS, TX, TY>(A, M);
-  stage2d_load<EQ, TC, TS, TX, TY>(A, M);
+  stage2d_load<EQ, TC, TS, TX, TY, NT>(A, M);
   __syncthreads();
   ph.mark(0);
-  stage2d_compute<EQ, TC, TS, TX, TY, STAGE, WENO>(A, i0, j0, nblk, M, S, &ph);
+  stage2d_compute<EQ, TC, TS, TX, TY, STAGE, WENO, NT>(A, i0, j0, nblk, M, S, &ph);
 }
 
 // FP32: as many resident CTAs as 72 registers a thread allow for 128-thread
@@ -674,16 +726,16 @@ struct StageMinBlocks {
   static constexpr int v = sizeof(TC) == 4 && 65536 / (R * NT) > 0 ? 65536 / (R * NT) : 1;
 };
 
-template <int EQ, class TC, class TS, int TX, int TY, int STAGE, bool WENO>
-__global__ void __launch_bounds__(TX * TY, (StageMinBlocks<TX * TY, TC>::v))
+template <int EQ, class TC, class TS, int TX, int TY, int STAGE, bool WENO, int NT = TX * TY>
+__global__ void __launch_bounds__(NT, (StageMinBlocks<NT, TC>::v))
     stage2d_kernel(const Stage2DArgs<TS> A) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   // launched as a programmatic dependent of the previous stage: everything of the
   // tile reads that stage's output, so wait for it before anything else
   griddep_launch_dependents();
   griddep_wait();
-  stage2d_tile<EQ, TC, TS, TX, TY, STAGE, WENO>(A, blockIdx.x * TX, blockIdx.y * TY,
-                                          gridDim.x * gridDim.y, smem_raw);
+  stage2d_tile<EQ, TC, TS, TX, TY, STAGE, WENO, NT>(A, blockIdx.x * TX, blockIdx.y * TY,
+                                                gridDim.x * gridDim.y, smem_raw);
 }
 
 }  // namespace dgk

@@ -35,8 +35,10 @@ namespace {
 
 // tile of the transposed right-hand-side kernel (static shared memory < 48 KB)
 template <class TC> struct VjpTile;
-template <> struct VjpTile<double> { static constexpr int X = 8, Y = 8; };
-template <> struct VjpTile<float> { static constexpr int X = 16, Y = 8; };
+// and its threads: two per cell, since a tile has 4.4 face points per cell and only a
+// few CTAs fit an SM
+template <> struct VjpTile<double> { static constexpr int X = 8, Y = 8, NT = 128; };
+template <> struct VjpTile<float> { static constexpr int X = 16, Y = 8, NT = 256; };
 
 // ---------------------------------------------------------------------------
 // U = Lambda(V): the limited state as its own array (internal layout)
@@ -82,6 +84,11 @@ struct VjpArgs {
   int nx, ny;
   long ncell;
   double dx, dy, gamma;
+  GasPair gas;
+  Geo2D<double> geo64;
+  Geo2D<float> geo32;
+  __device__ __forceinline__ const Geo2D<double>& geo(double) const { return geo64; }
+  __device__ __forceinline__ const Geo2D<float>& geo(float) const { return geo32; }
   const double* y;
   const double* x1;
   double a1;
@@ -93,8 +100,8 @@ struct VjpArgs {
 };
 
 template <class TC, class TS>
-__global__ void __launch_bounds__(VjpTile<TC>::X * VjpTile<TC>::Y) rhs_vjp2d_kernel(StateBuf<TS> U, VjpArgs A) {
-  constexpr int AX = VjpTile<TC>::X, AY = VjpTile<TC>::Y, ANT = AX * AY;
+__global__ void __launch_bounds__(VjpTile<TC>::NT) rhs_vjp2d_kernel(StateBuf<TS> U, VjpArgs A) {
+  constexpr int AX = VjpTile<TC>::X, AY = VjpTile<TC>::Y, ANT = VjpTile<TC>::NT;
   constexpr int R1X = AX + 2, R1Y = AY + 2, R1 = R1X * R1Y;
   constexpr int NFX = (AX + 1) * AY, NFY = AX * (AY + 1);
   __shared__ TC s_c0[4 * R1], s_sl[8 * R1], s_y[12 * R1];
@@ -104,8 +111,7 @@ __global__ void __launch_bounds__(VjpTile<TC>::X * VjpTile<TC>::Y) rhs_vjp2d_ker
   const int i0 = blockIdx.x * AX, j0 = blockIdx.y * AY;
   const int nx = A.nx, ny = A.ny;
   const size_t ncell = (size_t)A.ncell;
-  Gas<TC> G;
-  G.set(A.gamma);
+  const Gas<TC> G = gas_of<TC>(A.gas);
   unsigned err = 0;
   if (tid < R1X) s_gx[tid] = wrap_index(i0 - 1 + tid, nx);
   else if (tid < R1X + R1Y) s_gy[tid - R1X] = wrap_index(j0 - 1 + (tid - R1X), ny) * nx;
@@ -122,12 +128,9 @@ __global__ void __launch_bounds__(VjpTile<TC>::X * VjpTile<TC>::Y) rhs_vjp2d_ker
   }
   __syncthreads();
 
-  const TC dx = (TC)A.dx, dy = (TC)A.dy;
-  const TC hx = TC(0.5) * dx, hy = TC(0.5) * dy;
-  const TC ox = dx * TC(0.28867513459481288225), oy = dy * TC(0.28867513459481288225);
-  const TC c3x = TC(3) / (dx * dx), c3y = TC(3) / (dy * dy);
-  const TC r3 = TC(1.7320508075688772935) / (dx * dy);
-  const TC i2x = TC(0.5) / dx, i2y = TC(0.5) / dy;
+  const Geo2D<TC>& geo = A.geo(TC());
+  const TC hx = geo.hx, hy = geo.hy, ox = geo.ox, oy = geo.oy;
+  const TC c3x = geo.c3x, c3y = geo.c3y, r3 = geo.r3, i2x = geo.i2x, i2y = geo.i2y;
 
   // ---- faces: adjoint of every Gauss-point flux -> adjoints of both states
   for (int e = tid; e < 2 * (NFX + NFY); e += ANT) {
@@ -180,7 +183,7 @@ __global__ void __launch_bounds__(VjpTile<TC>::X * VjpTile<TC>::Y) rhs_vjp2d_ker
   // ---- per cell: gather faces and volume points
   const int lx = tid % AX, ly = tid / AX;
   const int gi = i0 + lx, gj = j0 + ly;
-  if (gi < nx && gj < ny) {
+  if (tid < AX * AY && gi < nx && gj < ny) {
     const int r = (ly + 1) * R1X + lx + 1;
     TC acc[12];
 #pragma unroll
@@ -230,8 +233,8 @@ __global__ void __launch_bounds__(VjpTile<TC>::X * VjpTile<TC>::Y) rhs_vjp2d_ker
     const size_t gc = (size_t)gj * nx + gi;
 #pragma unroll
     for (int p = 0; p < 12; ++p) {
-      double o = A.a1 * A.x1[p * ncell + gc] + A.beta * Cvt<TC>::to_f64(acc[p]);
-      if (A.x2) o += A.a2 * A.x2[p * ncell + gc];
+      double o = fma(A.beta, Cvt<TC>::to_f64(acc[p]), A.a1 * A.x1[p * ncell + gc]);
+      if (A.x2) o = fma(A.a2, A.x2[p * ncell + gc], o);
       A.out[p * ncell + gc] = o;
     }
   }
@@ -766,7 +769,9 @@ struct Work {
   double* c0[4];
   void* sl[4];
   double* lam[3];
-  double* segbuf;
+  // states of the segment being swept, in the internal layout: seg slots
+  char* segbuf;
+  size_t seg_stride, seg_sl;  // bytes from slot to slot and to a slot's coefficients
   double* lamrun[2];
   Ctl* ctl;
   unsigned* err;
@@ -777,6 +782,15 @@ StateBuf<TS> sb(const Work& w, int k) {
   StateBuf<TS> s;
   s.c0 = w.c0[k];
   s.sl = reinterpret_cast<TS*>(w.sl[k]);
+  return s;
+}
+
+template <class TS>
+StateBuf<TS> seg_state(const Work& w, long long i) {
+  StateBuf<TS> s;
+  char* b = w.segbuf + (size_t)i * w.seg_stride;
+  s.c0 = reinterpret_cast<double*>(b);
+  s.sl = reinterpret_cast<TS*>(b + w.seg_sl);
   return s;
 }
 
@@ -805,7 +819,9 @@ size_t carve_into(char* base, const AdjointCall& c, int seg, Work* w) {
   t.lamrun[1] = (double*)take(n * np * 8);
   t.ctl = (Ctl*)take(sizeof(Ctl));
   t.err = (unsigned*)take(sizeof(unsigned));
-  t.segbuf = (double*)take((size_t)seg * n * np * 8);
+  t.seg_sl = (n * nv * 8 + 255) / 256 * 256;
+  t.seg_stride = t.seg_sl + (n * ns * ts + 255) / 256 * 256;
+  t.segbuf = take((size_t)seg * t.seg_stride);
   if (w) *w = t;
   return off;
 }
@@ -861,11 +877,6 @@ cudaError_t to_internal(int eq, const double* src, StateBuf<TS> dst, long n, cud
 }
 
 template <class TS>
-cudaError_t to_interchange(int eq, StateBuf<TS> src, double* dst, long n, cudaStream_t st) {
-  return launch_state_out<TS>(src, dst, planes2d(eq), n, st);
-}
-
-template <class TS>
 Stage2DArgs<TS> stage_args(const AdjointCall& c, const Work& w, StateBuf<TS> in, StateBuf<TS> base,
                            StateBuf<TS> out, double dt) {
   Stage2DArgs<TS> a;
@@ -887,6 +898,9 @@ cudaError_t apply_rhs_vjp(const AdjointCall& c, const Work& w, StateBuf<TS> U, c
   VjpArgs A;
   A.nx = c.nx; A.ny = c.ny; A.ncell = (long)c.nx * c.ny;
   A.dx = c.dx; A.dy = c.dy; A.gamma = c.gamma;
+  A.gas.set(c.gamma);
+  A.geo64.set(c.dx, c.dy);
+  A.geo32.set(c.dx, c.dy);
   A.y = y; A.x1 = x1; A.a1 = a1; A.x2 = x2; A.a2 = a2; A.beta = beta; A.out = out;
   A.err = w.err;
   if (c.eq) {
@@ -897,19 +911,19 @@ cudaError_t apply_rhs_vjp(const AdjointCall& c, const Work& w, StateBuf<TS> U, c
   }
   constexpr int AX = VjpTile<TC>::X, AY = VjpTile<TC>::Y;
   dim3 grid((c.nx + AX - 1) / AX, (c.ny + AY - 1) / AY);
-  rhs_vjp2d_kernel<TC, TS><<<grid, AX * AY, 0, c.stream>>>(U, A);
+  rhs_vjp2d_kernel<TC, TS><<<grid, VjpTile<TC>::NT, 0, c.stream>>>(U, A);
   return cudaGetLastError();
 }
 
-// One reverse step given V^n (internal, buffer 0).  lam_next -> lam_prev.
+// One reverse step given V^n (internal layout).  lam_next -> lam_prev.
 template <class TC, class TS>
-cudaError_t reverse_step(const AdjointCall& c, const Work& w, const double* lam_next,
-                         double* lam_prev, double dt) {
+cudaError_t reverse_step(const AdjointCall& c, const Work& w, StateBuf<TS> Vn,
+                         const double* lam_next, double* lam_prev, double dt) {
   const long n = (long)c.nx * c.ny;
-  StateBuf<TS> Vn = sb<TS>(w, 0), Un = sb<TS>(w, 1), V1 = sb<TS>(w, 2), U1 = sb<TS>(w, 3);
+  StateBuf<TS> Un = sb<TS>(w, 1), V1 = sb<TS>(w, 2), U1 = sb<TS>(w, 3);
   cudaError_t e;
   // forward recompute of the stage states
-  e = launch_stage2d(c.eq, 0, 1, stage_args<TS>(c, w, Vn, Vn, V1, dt), c.stream);
+  e = launch_stage2d(c.eq, c.variant, 1, stage_args<TS>(c, w, Vn, Vn, V1, dt), c.stream);
   if (e != cudaSuccess) return e;
   if (c.limiter && c.eq) {
     limit2d_mhd_kernel<TC, TS><<<grid1d(n), 256, 0, c.stream>>>(Vn, Un, c.nx, c.ny, c.dx, c.dy, c.gamma);
@@ -991,7 +1005,7 @@ dg_status step_t(AdjointStore& S, const AdjointCall& c, const double* u_n, const
   if ((e = cudaMemsetAsync(w.err, 0, sizeof(unsigned), c.stream)) != cudaSuccess ||
       (e = cudaMemsetAsync(w.ctl, 0, sizeof(Ctl), c.stream)) != cudaSuccess ||
       (e = to_internal<TS>(c.eq, u_n, sb<TS>(w, 0), n, c.stream)) != cudaSuccess ||
-      (e = reverse_step<TC, TS>(c, w, lam_next, lam_prev, dt)) != cudaSuccess) {
+      (e = reverse_step<TC, TS>(c, w, sb<TS>(w, 0), lam_next, lam_prev, dt)) != cudaSuccess) {
     msg = std::string("adjoint step: ") + cudaGetErrorString(e);
     return DG_ECUDA;
   }
@@ -1029,34 +1043,26 @@ dg_status run_t(AdjointStore& S, const AdjointCall& c, int k, const double* lam_
   const long long nseg = (S.nrec + k - 1) / k;
   for (long long sgi = nseg - 1; sgi >= 0; --sgi) {
     const long long n0 = sgi * k, n1 = std::min<long long>(S.nrec, n0 + k);
-    // recompute V^{n0} .. V^{n1-1} from the checkpoint
+    // recompute V^{n0} .. V^{n1-1} from the checkpoint, each into its slot
     const double* ck = S.ckpt + (size_t)sgi * plane;
-    if ((e = cudaMemcpyAsync(w.segbuf, ck, plane * 8, cudaMemcpyDeviceToDevice, c.stream)) !=
-        cudaSuccess)
-      break;
-    if ((e = to_internal<TS>(c.eq, ck, sb<TS>(w, 0), n, c.stream)) != cudaSuccess) break;
-    int a = 0;  // buffers 0 and 1 take turns as the step's input and output
+    if ((e = to_internal<TS>(c.eq, ck, seg_state<TS>(w, 0), n, c.stream)) != cudaSuccess) break;
     for (long long m = n0; m + 1 < n1; ++m) {
       const double dt = dts[(size_t)m];
-      if ((e = launch_stage2d(c.eq, 0, 1, stage_args<TS>(c, w, sb<TS>(w, a), sb<TS>(w, a), sb<TS>(w, 2), dt),
+      const StateBuf<TS> in = seg_state<TS>(w, m - n0), out = seg_state<TS>(w, m + 1 - n0);
+      if ((e = launch_stage2d(c.eq, c.variant, 1, stage_args<TS>(c, w, in, in, sb<TS>(w, 2), dt),
                               c.stream)) != cudaSuccess)
         break;
-      if ((e = launch_stage2d(c.eq, 0, 2, stage_args<TS>(c, w, sb<TS>(w, 2), sb<TS>(w, a), sb<TS>(w, 1 - a), dt),
+      if ((e = launch_stage2d(c.eq, c.variant, 2, stage_args<TS>(c, w, sb<TS>(w, 2), in, out, dt),
                               c.stream)) != cudaSuccess)
         break;
-      if ((e = to_interchange<TS>(c.eq, sb<TS>(w, 1 - a), w.segbuf + (size_t)(m + 1 - n0) * plane, n,
-                                  c.stream)) != cudaSuccess)
-        break;
-      a = 1 - a;
     }
     if (e != cudaSuccess) break;
     // reverse through the segment
     for (long long m = n1 - 1; m >= n0; --m) {
-      if ((e = to_internal<TS>(c.eq, w.segbuf + (size_t)(m - n0) * plane, sb<TS>(w, 0), n, c.stream)) !=
-          cudaSuccess)
-        break;
       double* dst = (m == 0) ? lam_0 : w.lamrun[cur ^ 1];
-      if ((e = reverse_step<TC, TS>(c, w, w.lamrun[cur], dst, dts[(size_t)m])) != cudaSuccess) break;
+      if ((e = reverse_step<TC, TS>(c, w, seg_state<TS>(w, m - n0), w.lamrun[cur], dst,
+                                    dts[(size_t)m])) != cudaSuccess)
+        break;
       cur ^= 1;
     }
     if (e != cudaSuccess) break;

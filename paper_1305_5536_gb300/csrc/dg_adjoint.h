@@ -33,6 +33,7 @@ struct AdjointCall {
   int nx, ny;
   double dx, dy, gamma;
   int limiter, fp32;
+  int variant;  // tile shape of the forward stage kernels
   cudaStream_t stream;
 };
 

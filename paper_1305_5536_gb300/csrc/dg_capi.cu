@@ -725,6 +725,12 @@ dg_status build_batch(dg_ctx* c) {
   return DG_OK;
 }
 
+// Tile shape of the forward stages inside the adjoint: the tuned one, unless that is a
+// persistent TMA kernel, whose tensor maps are kept for the context's own buffers only.
+int adjoint_variant(const dg_ctx* c) {
+  return c->variant < 0 || c->variant == 3 || c->variant == 4 ? 0 : c->variant;
+}
+
 }  // namespace
 
 // ===========================================================================
@@ -1045,6 +1051,7 @@ dg_status dg_adjoint_step(dg_ctx* c, const double* lam_next, double* lam_prev, c
   call.dx = c->probs[0].dx; call.dy = c->probs[0].dy;
   call.gamma = c->gamma; call.limiter = c->limiter; call.fp32 = c->fp32;
   call.eq = c->eq;
+  call.variant = adjoint_variant(c);
   call.stream = c->stream;
   std::string msg;
   dg_status s = adjoint_step(c->adj, call, u_n, lam_next, lam_prev, dt, msg);
@@ -1123,6 +1130,7 @@ dg_status dg_adjoint(dg_ctx* c, const double* lam_N, double* lam_0) {
   call.nx = p.nx; call.ny = p.ny; call.dx = p.dx; call.dy = p.dy;
   call.gamma = c->gamma; call.limiter = c->limiter; call.fp32 = c->fp32;
   call.eq = c->eq;
+  call.variant = adjoint_variant(c);
   call.stream = c->stream;
   std::string msg;
   dg_status s = adjoint_run(c->adj, call, c->nplanes, c->ckpt_every, lam_N, lam_0, msg);

@@ -1,7 +1,6 @@
 // dg_dual.cuh -- forward-mode dual numbers for the device and the dual versions
 // of the 2D Euler building blocks used by the adjoint kernels: conserved ->
-// primitive conversion, physical fluxes, the exact Riemann flux and the min/max
-// limiter.  A Dn<T, N> carries a value and N tangents; branches are decided on
+// primitive conversion and the min/max limiter.  A Dn<T, N> carries a value and N tangents; branches are decided on
 // values (the derivative of the active branch).
 #pragma once
 
@@ -122,15 +121,6 @@ __device__ __forceinline__ Dn<T, N> dsqrt(const Dn<T, N>& a) {
   return r;
 }
 template <class T, int N>
-__device__ __forceinline__ Dn<T, N> dpow(const Dn<T, N>& a, T e) {
-  Dn<T, N> r;
-  r.v = rpow(a.v, e);
-  T k = a.v != T(0) ? e * r.v / a.v : T(0);
-#pragma unroll
-  for (int i = 0; i < N; ++i) r.d[i] = a.d[i] * k;
-  return r;
-}
-template <class T, int N>
 __device__ __forceinline__ Dn<T, N> dabs(const Dn<T, N>& a) { return a.v < T(0) ? -a : a; }
 
 // What the scalar device physics needs besides arithmetic, so that its templates
@@ -158,8 +148,6 @@ __device__ __forceinline__ Dn<T, N>& operator+=(Dn<T, N>& a, const Dn<T, N>& b) 
   return a;
 }
 template <class T, int N>
-__device__ __forceinline__ Dn<T, N> rsqrtv(const Dn<T, N>& a) { return dsqrt(a); }
-template <class T, int N>
 __device__ __forceinline__ Dn<T, N> sqrtv(const Dn<T, N>& a) { return dsqrt(a); }
 template <class T, int N>
 __device__ __forceinline__ Dn<T, N> rcpv(const Dn<T, N>& a) { return T(1) / a; }
@@ -177,7 +165,6 @@ struct Tiny<Dn<T, N>> {
 };
 template <class T, int N>
 struct Prec<Dn<T, N>> {
-  static constexpr T newton_tol = Prec<T>::newton_tol;
   static constexpr int newton_max = Prec<T>::newton_max;
   static constexpr T hlld_degenerate = Prec<T>::hlld_degenerate;
 };
@@ -191,124 +178,6 @@ __device__ __forceinline__ void dprims2d(const Gas<T>& G, const Dn<T, N>* c, Dn<
   W[1] = vx;
   W[2] = vy;
   W[3] = G.gm1 * (c[3] - T(0.5) * (c[1] * vx + c[2] * vy));
-}
-
-// Physical fluxes along x and y of conserved (rho, mx, my, E), dual.
-template <class T, int N>
-__device__ __forceinline__ void dphys_flux2d(const Gas<T>& G, const Dn<T, N>* c, Dn<T, N>* Fx,
-                                             Dn<T, N>* Fy) {
-  Dn<T, N> W[4];
-  dprims2d<T, N>(G, c, W);
-  Dn<T, N> e = c[3] + W[3];
-  Fx[0] = c[1]; Fx[1] = c[1] * W[1] + W[3]; Fx[2] = c[2] * W[1]; Fx[3] = e * W[1];
-  Fy[0] = c[2]; Fy[1] = c[1] * W[2]; Fy[2] = c[2] * W[2] + W[3]; Fy[3] = e * W[2];
-}
-
-template <class T, int N>
-__device__ __forceinline__ void dpressure_fn(const Gas<T>& G, const Dn<T, N>& p, const Dn<T, N>& rK,
-                                             const Dn<T, N>& pK, const Dn<T, N>& cK, Dn<T, N>& f,
-                                             Dn<T, N>& df) {
-  if (p.v > pK.v) {
-    Dn<T, N> A = G.two_gp1 / rK;
-    Dn<T, N> B = G.g6 * pK;
-    Dn<T, N> q = dsqrt(A / (p + B));
-    f = (p - pK) * q;
-    df = q * (T(1) - T(0.5) * (p - pK) / (B + p));
-  } else {
-    Dn<T, N> pr = p / pK;
-    f = (T(2) * G.inv_gm1) * cK * (dpow(pr, G.z) - T(1));
-    df = T(1) / (rK * cK) * dpow(pr, G.mzp);
-  }
-}
-
-// Exact-solver flux in the face frame (mass, normal momentum, transverse
-// momentum, energy) of dual primitive states; p* from the value solve, its
-// derivative from one Newton step taken in dual arithmetic at the root.
-template <class T, int N>
-__device__ void dexact_flux(const Gas<T>& G, const Dn<T, N>& rL, const Dn<T, N>& uL,
-                            const Dn<T, N>& pL, const Dn<T, N>& vL, const Dn<T, N>& rR,
-                            const Dn<T, N>& uR, const Dn<T, N>& pR, const Dn<T, N>& vR,
-                            Dn<T, N>* F, unsigned& err) {
-  typedef Dn<T, N> D;
-  if (!(rL.v > T(0) && pL.v > T(0) && rR.v > T(0) && pR.v > T(0))) {
-    err |= ERR_NONPHYS;
-    for (int q = 0; q < 4; ++q) F[q] = dconst<T, N>(T(0));
-    return;
-  }
-  D cL = dsqrt(G.g * pL / rL), cR = dsqrt(G.g * pR / rR);
-  const T pv = exact_pstar(G, rL.v, uL.v, pL.v, cL.v, rR.v, uR.v, pR.v, cR.v, err);
-  D p0 = dconst<T, N>(pv);
-  D fL, dfL, fR, dfR;
-  dpressure_fn(G, p0, rL, pL, cL, fL, dfL);
-  dpressure_fn(G, p0, rR, pR, cR, fR, dfR);
-  D p = p0 - (fL + fR + (uR - uL)) / (dfL + dfR);
-  p.v = pv;
-  dpressure_fn(G, p, rL, pL, cL, fL, dfL);
-  dpressure_fn(G, p, rR, pR, cR, fR, dfR);
-  D us = T(0.5) * (uL + uR) + T(0.5) * (fR - fL);
-  D rho, u, pp, vt;
-  if (T(0) <= us.v) {
-    vt = vL;
-    if (p.v > pL.v) {
-      D SL = uL - cL * dsqrt(G.shk1 * p / pL + G.z);
-      if (T(0) <= SL.v) { rho = rL; u = uL; pp = pL; }
-      else { rho = rL * ((p / pL + G.g6) / (G.g6 * p / pL + T(1))); u = us; pp = p; }
-    } else {
-      D SHL = uL - cL;
-      if (T(0) <= SHL.v) { rho = rL; u = uL; pp = pL; }
-      else {
-        D cmL = cL * dpow(p / pL, G.z);
-        if (T(0) > (us - cmL).v) { rho = rL * dpow(p / pL, G.inv_g); u = us; pp = p; }
-        else {
-          D c = G.two_gp1 * (cL + T(0.5) * G.gm1 * uL);
-          u = c;
-          rho = rL * dpow(c / cL, G.two_gm1);
-          pp = pL * dpow(c / cL, G.inv_z);
-        }
-      }
-    }
-  } else {
-    vt = vR;
-    if (p.v > pR.v) {
-      D SR = uR + cR * dsqrt(G.shk1 * p / pR + G.z);
-      if (T(0) >= SR.v) { rho = rR; u = uR; pp = pR; }
-      else { rho = rR * ((p / pR + G.g6) / (G.g6 * p / pR + T(1))); u = us; pp = p; }
-    } else {
-      D SHR = uR + cR;
-      if (T(0) >= SHR.v) { rho = rR; u = uR; pp = pR; }
-      else {
-        D cmR = cR * dpow(p / pR, G.z);
-        if (T(0) < (us + cmR).v) { rho = rR * dpow(p / pR, G.inv_g); u = us; pp = p; }
-        else {
-          D c = G.two_gp1 * (cR - T(0.5) * G.gm1 * uR);
-          u = -c;
-          rho = rR * dpow(c / cR, G.two_gm1);
-          pp = pR * dpow(c / cR, G.inv_z);
-        }
-      }
-    }
-  }
-  D E = pp * G.inv_gm1 + T(0.5) * rho * (u * u + vt * vt);
-  D mu = rho * u;
-  F[0] = mu;
-  F[1] = mu * u + pp;
-  F[2] = mu * vt;
-  F[3] = u * (E + pp);
-}
-
-// Lab-frame exact flux through a face along `dir` between dual conserved states.
-template <class T, int N>
-__device__ __forceinline__ void dface_flux2d(const Gas<T>& G, int dir, const Dn<T, N>* cl,
-                                             const Dn<T, N>* cr, Dn<T, N>* F, unsigned& err) {
-  Dn<T, N> Wl[4], Wr[4], Ff[4];
-  dprims2d<T, N>(G, cl, Wl);
-  dprims2d<T, N>(G, cr, Wr);
-  if (dir == 0) dexact_flux<T, N>(G, Wl[0], Wl[1], Wl[3], Wl[2], Wr[0], Wr[1], Wr[3], Wr[2], Ff, err);
-  else dexact_flux<T, N>(G, Wl[0], Wl[2], Wl[3], Wl[1], Wr[0], Wr[2], Wr[3], Wr[1], Ff, err);
-  F[0] = Ff[0];
-  F[3] = Ff[3];
-  if (dir == 0) { F[1] = Ff[1]; F[2] = Ff[2]; }
-  else { F[1] = Ff[2]; F[2] = Ff[1]; }
 }
 
 // Dual min/max limiter of one 2D Euler cell (Sec. 2.5): c0/s its averages and

@@ -32,12 +32,10 @@ enum : unsigned {
 
 template <class T> struct Prec;
 template <> struct Prec<double> {
-  static constexpr double newton_tol = 1e-12;
   static constexpr int newton_max = 50;
   static constexpr double hlld_degenerate = 1e-8;
 };
 template <> struct Prec<float> {
-  static constexpr float newton_tol = 1e-5f;
   static constexpr int newton_max = 20;
   static constexpr float hlld_degenerate = 1e-8f;
 };
@@ -47,8 +45,6 @@ template <> struct Prec<float> {
 // a few ulp for the exponents used here, ~10x fewer instructions than powf.
 __device__ __forceinline__ double rpow(double x, double e) { return pow(x, e); }
 __device__ __forceinline__ float rpow(float x, float e) { return __powf(x, e); }
-__device__ __forceinline__ double rsqrtv(double x) { return sqrt(x); }
-__device__ __forceinline__ float rsqrtv(float x) { return sqrtf(x); }
 
 // Conversions between the FP64 cell averages and the arithmetic type.  For the
 // FP32 path they are done with integer operations on the IEEE-754 bit patterns,
@@ -183,70 +179,28 @@ __device__ __forceinline__ T fast_speed(const Gas<T>& G, T rho, T p, T b2, T bn)
 // Output F[0] mass, F[1] normal momentum, F[2..1+NT] transverse momenta,
 // F[2+NT] energy -- all in the face frame.
 // ----------------------------------------------------------------------------
-template <class T>
-__device__ __forceinline__ void pressure_fn(const Gas<T>& G, T p, T rK, T pK, T cK, T& f,
-                                            T& df) {
-  if (p > pK) {
-    T A = G.two_gp1 / rK;
-    T B = G.g6 * pK;
-    T q = rsqrtv(A / (p + B));
-    f = (p - pK) * q;
-    df = q * (T(1) - T(0.5) * (p - pK) / (B + p));
-  } else {
-    // (p/pK)^(-(g+1)/(2g)) = (p/pK)^((g-1)/(2g)) / (p/pK): one power, not two
-    T pr = p / pK;
-    T q = rpow(pr, G.z);
-    f = T(2) * cK * G.inv_gm1 * (q - T(1));
-    df = q / (rK * cK * pr);
-  }
-}
-
 // Adaptive PVRS / two-rarefaction / two-shock first guess of the star-region pressure
-// (Toro's choice), at least the floor 1e-10 min(pL, pR).
-template <class T>
-__device__ __forceinline__ T exact_guess(const Gas<T>& G, T rL, T pL, T cL, T rR, T pR, T cR,
-                                         T du, T pfloor) {
-  T pv = T(0.5) * (pL + pR) - T(0.125) * du * (rL + rR) * (cL + cR);
-  pv = pv > T(0) ? pv : T(0);
-  const T pmin = pL < pR ? pL : pR, pmax = pL < pR ? pR : pL;
-  T p;
-  if (pmax / pmin <= T(2) && pmin <= pv && pv <= pmax) {
+// (Toro's choice) in FP64, for states outside the FP32 range; at least the floor 1e-10
+// min(pL, pR).
+__device__ __forceinline__ double exact_guess(const Gas<double>& G, double rL, double pL, double cL,
+                                              double rR, double pR, double cR, double du,
+                                              double pfloor) {
+  double pv = 0.5 * (pL + pR) - 0.125 * du * (rL + rR) * (cL + cR);
+  pv = pv > 0.0 ? pv : 0.0;
+  const double pmin = pL < pR ? pL : pR, pmax = pL < pR ? pR : pL;
+  double p;
+  if (pmax / pmin <= 2.0 && pmin <= pv && pv <= pmax) {
     p = pv;
   } else if (pv < pmin) {
-    T num = cL + cR - T(0.5) * G.gm1 * du;
-    T den = cL / rpow(pL, G.z) + cR / rpow(pR, G.z);
-    p = rpow((num > T(0) ? num : T(0)) / den, G.inv_z);
+    const double num = cL + cR - 0.5 * G.gm1 * du;
+    const double den = cL / rpow(pL, G.z) + cR / rpow(pR, G.z);
+    p = rpow((num > 0.0 ? num : 0.0) / den, G.inv_z);
   } else {
-    T gL = rsqrtv(G.two_gp1 / rL / (G.g6 * pL + pv));
-    T gR = rsqrtv(G.two_gp1 / rR / (G.g6 * pR + pv));
+    const double gL = sqrt(G.two_gp1 / rL / (G.g6 * pL + pv));
+    const double gR = sqrt(G.two_gp1 / rR / (G.g6 * pR + pv));
     p = (gL * pL + gR * pR - du) / (gL + gR);
   }
   return p > pfloor ? p : pfloor;
-}
-
-// Star-region pressure p* of the Riemann problem (rho, u, p)_L | (rho, u, p)_R:
-// root of f_L(p) + f_R(p) + (u_R - u_L) by Newton iteration from the adaptive
-// first guess.  cL, cR are the sound speeds.
-template <class T>
-__device__ __forceinline__ T exact_pstar(const Gas<T>& G, T rL, T uL, T pL, T cL, T rR, T uR, T pR,
-                                         T cR, unsigned& err) {
-  const T du = uR - uL;
-  if (G.two_gm1 * (cL + cR) <= du) err |= ERR_VACUUM;
-  const T pfloor = T(1e-10) * (pL < pR ? pL : pR);
-  T p = exact_guess<T>(G, rL, pL, cL, rR, pR, cR, du, pfloor);
-  bool conv = false;
-  for (int it = 0; it < Prec<T>::newton_max; ++it) {
-    T fL, dfL, fR, dfR;
-    pressure_fn(G, p, rL, pL, cL, fL, dfL);
-    pressure_fn(G, p, rR, pR, cR, fR, dfR);
-    T pn = p - (fL + fR + du) / (dfL + dfR);
-    if (!(pn > pfloor)) pn = pfloor;
-    T change = T(2) * fabs(pn - p) / (pn + p);
-    p = pn;
-    if (change < Prec<T>::newton_tol) { conv = true; break; }
-  }
-  if (!conv) err |= ERR_NEWTON;
-  return p;
 }
 
 // ----------------------------------------------------------------------------
@@ -461,7 +415,7 @@ __device__ __forceinline__ Star64 star_f64(const Gas<double>& G, double rL, doub
   const double pfloor = 1e-10 * (gt_pos(pR, pL) ? pL : pR);
   double p = Cvt<double>::to_tc(Cvt<float>::to_f64(S.p));
   if (!(S.conv && S.p > 1e-30f && S.p < 1e30f))
-    p = exact_guess<double>(G, rL, pL, cL, rR, pR, cR, du, pfloor);
+    p = exact_guess(G, rL, pL, cL, rR, pR, cR, du, pfloor);
   Star64 R;
   bool conv = false;
   for (int it = 0; it < Prec<double>::newton_max; ++it) {
@@ -492,15 +446,6 @@ __device__ __forceinline__ Star64 star_f64(const Gas<double>& G, double rL, doub
   }
   if (!conv) err |= ERR_NEWTON;
   return R;
-}
-
-template <>
-__device__ __forceinline__ double exact_pstar<double>(const Gas<double>& G, double rL, double uL,
-                                                      double pL, double cL, double rR, double uR,
-                                                      double pR, double cR, unsigned& err) {
-  const double du = uR - uL;
-  if (G.two_gm1 * (cL + cR) <= du) err |= ERR_VACUUM;
-  return star_f64(G, rL, pL, rcpv(pL), cL, rR, pR, rcpv(pR), cR, du, err).p;
 }
 
 template <int NT>

@@ -263,7 +263,7 @@ __device__ __forceinline__ void griddep_launch_dependents() {
 }
 
 // Launch of a stage kernel as a programmatic dependent of the kernel before it on
-// the stream (the kernel must begin with griddep_wait()).
+// the stream (the kernel must call griddep_wait() before it touches global memory).
 template <class... KArgs, class... Args>
 inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem,
                               cudaStream_t st, Args&&... args) {

@@ -461,13 +461,14 @@ template <int EQ, class TC, class TS, int TX, int TY, int NGF, bool WENO, int NT
 __global__ void __launch_bounds__(NT, (MhMinBlocks<EQ, NT, NGF, WENO, TC>::v))
     mh2d_kernel(const Stage2DArgs<TS> A) {
   griddep_launch_dependents();  // programmatic dependent launch: see griddep_wait()
-  griddep_wait();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ TileScalars<NT> S;
   const MhMem2D<TC> M = mh2d_mem<EQ, TX, TY, NGF, TC>(smem_raw);
   const int i0 = blockIdx.x * TX, j0 = blockIdx.y * TY;
   stage2d_setup<EQ, TC, TS, TX, TY, NT>(A, i0, j0, M.m, S);
   __syncthreads();
+  griddep_wait();
+  stage2d_take_dt(A, S);
   stage2d_load<EQ, TC, TS, TX, TY, NT>(A, M.m);
   __syncthreads();
   mh2d_compute<EQ, TC, TS, TX, TY, NGF, WENO, NT>(A, i0, j0, gridDim.x * gridDim.y, M, S);

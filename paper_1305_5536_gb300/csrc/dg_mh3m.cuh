@@ -156,7 +156,6 @@ __device__ __forceinline__ void prim_flux3m(const Gas<TC>& G, const TC* W, int d
 template <class TC, class TS, int TX, int TY, int TZ, int NGF, bool WENO>
 __global__ void __launch_bounds__(TX * TY * TZ) mh3m_kernel(const Stage3DArgs<TS> A) {
   griddep_launch_dependents();  // programmatic dependent launch: see griddep_wait()
-  griddep_wait();
   constexpr int R2X = TX + 4, R2Y = TY + 4, R2Z = TZ + 4, R2 = R2X * R2Y * R2Z;
   constexpr int R1X = TX + 2, R1Y = TY + 2, R1Z = TZ + 2, R1 = R1X * R1Y * R1Z;
   constexpr int NT = TX * TY * TZ;
@@ -185,20 +184,18 @@ __global__ void __launch_bounds__(TX * TY * TZ) mh3m_kernel(const Stage3DArgs<TS
   const size_t ncell = (size_t)A.ncell;
   const Gas<TC> G = gas_of<TC>(A.gas);
   unsigned err = 0;
-  if (tid == 0) {
-    s_err = 0;
-    double dt = A.dt_override > 0.0 ? A.dt_override : A.ctl->dt_cur;
-    if (!(dt > 0.0) || !(dt < 1e300)) err |= ERR_NONPHYS;
-    s_dt = dt;
-  }
+  if (tid == 0) s_err = 0;
   if (tid < R2X) s_gx[tid] = wrap_index(i0 - 2 + tid, nx);
   else if (tid < R2X + R2Y) s_gy[tid - R2X] = wrap_index(j0 - 2 + (tid - R2X), ny) * nx;
   else if (tid < R2X + R2Y + R2Z)
     s_gz[tid - R2X - R2Y] = wrap_index(k0 - 2 + (tid - R2X - R2Y), nz) * nx * ny;
   __syncthreads();
-  const double dt = s_dt;
-  const TC dtc = Cvt<TC>::to_tc(dt);
-  const TC hdt = TC(0.5) * dtc;
+  griddep_wait();  // the index tables need nothing from the kernel before
+  if (tid == 0) {
+    const double dt = A.dt_override > 0.0 ? A.dt_override : A.ctl->dt_cur;
+    if (!(dt > 0.0) || !(dt < 1e300)) err |= ERR_NONPHYS;
+    s_dt = dt;
+  }
 
   // ---- 1. primitives of the halo-2 box; coefficients of the halo-1 box
   stage3d_issue<8, 23, TX, TY, TZ>(A.in, ncell, s_gx, s_gy, s_gz, s_g);
@@ -215,6 +212,9 @@ __global__ void __launch_bounds__(TX * TY * TZ) mh3m_kernel(const Stage3DArgs<TS
   }
   cp_async_wait_all();
   __syncthreads();
+  const double dt = s_dt;
+  const TC dtc = Cvt<TC>::to_tc(dt);
+  const TC hdt = TC(0.5) * dtc;
 
   const Geo3D<TS>& geo = A.geo;
   const TC hh[3] = {geo.hh[0], geo.hh[1], geo.hh[2]};

@@ -244,22 +244,28 @@ __device__ __forceinline__ void face_flux2d(const Gas<TC>& G, int dir, const TC*
   else { F[1] = Ff[2]; F[2] = Ff[1]; }
 }
 
-// Start of a tile: the time step, the error word, and the wrapped global row and
-// column offsets of the halo-2 region.  The caller synchronises afterwards.
+// Start of a tile: the wrapped global row and column offsets of the halo-2 region and
+// the error word, which need nothing from the kernel before; the caller synchronises,
+// waits for that kernel and then takes the time step (stage2d_take_dt; visible after the
+// staging's barrier).
 template <int EQ, class TC, class TS, int TX, int TY, int NT = TX * TY>
 __device__ __forceinline__ void stage2d_setup(const Stage2DArgs<TS>& A, int i0, int j0,
                                               const TileMem<TC>& M, TileScalars<NT>& S) {
   using T = Tile2D<EQ, TX, TY>;
   static_assert(T::R2X + T::R2Y <= NT, "one thread per row and column offset");
   const int tid = threadIdx.x;
-  if (tid == 0) {
-    S.err = 0;
-    double dt = A.dt_override > 0.0 ? A.dt_override : A.ctl->dt_cur;
+  if (tid == 0) S.err = 0;
+  if (tid < T::R2X) M.gx[tid] = wrap_index(i0 - 2 + tid, A.nx);
+  else if (tid < T::R2X + T::R2Y) M.gy[tid - T::R2X] = wrap_index(j0 - 2 + (tid - T::R2X), A.ny) * A.nx;
+}
+
+template <class TS, int NT>
+__device__ __forceinline__ void stage2d_take_dt(const Stage2DArgs<TS>& A, TileScalars<NT>& S) {
+  if (threadIdx.x == 0) {
+    const double dt = A.dt_override > 0.0 ? A.dt_override : A.ctl->dt_cur;
     if (!(dt > 0.0) || !(dt < 1e300)) S.err |= ERR_NONPHYS;
     S.dt = dt;
   }
-  if (tid < T::R2X) M.gx[tid] = wrap_index(i0 - 2 + tid, A.nx);
-  else if (tid < T::R2X + T::R2Y) M.gy[tid - T::R2X] = wrap_index(j0 - 2 + (tid - T::R2X), A.ny) * A.nx;
 }
 
 // Stage the tile from global memory (periodic wrap): averages with halo 2,
@@ -708,6 +714,8 @@ __device__ __forceinline__ void stage2d_tile(const Stage2DArgs<TS>& A, int i0, i
   const TileMem<TC> M = tile_mem<EQ, TX, TY, TC>(smem_raw);
   stage2d_setup<EQ, TC, TS, TX, TY, NT>(A, i0, j0, M, S);
   __syncthreads();
+  griddep_wait();
+  stage2d_take_dt(A, S);
   if (STAGE == 2) stage2d_prefetch_base<EQ, TC, TS, TX, TY>(A, M);
   stage2d_load<EQ, TC, TS, TX, TY, NT>(A, M);
   __syncthreads();
@@ -730,10 +738,9 @@ template <int EQ, class TC, class TS, int TX, int TY, int STAGE, bool WENO, int 
 __global__ void __launch_bounds__(NT, (StageMinBlocks<NT, TC>::v))
     stage2d_kernel(const Stage2DArgs<TS> A) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  // launched as a programmatic dependent of the previous stage: everything of the
-  // tile reads that stage's output, so wait for it before anything else
+  // launched as a programmatic dependent of the previous stage: the tile waits for its
+  // output once its index tables are ready (stage2d_tile)
   griddep_launch_dependents();
-  griddep_wait();
   stage2d_tile<EQ, TC, TS, TX, TY, STAGE, WENO, NT>(A, blockIdx.x * TX, blockIdx.y * TY,
                                                 gridDim.x * gridDim.y, smem_raw);
 }

@@ -81,6 +81,7 @@ __global__ void __launch_bounds__(TX * TY)
     __syncthreads();  // the previous tile is done with shared memory
     stage2d_setup<EQ, TC, TS, TX, TY>(A, i0, j0, M, S);
     __syncthreads();
+    stage2d_take_dt(A, S);
     bool use_raw = false;
     if (pending) {
       const bool late = !mbar_wait_bounded(&bar, phase, spin_limit);

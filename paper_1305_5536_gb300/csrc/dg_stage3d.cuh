@@ -295,7 +295,6 @@ template <class TC, class TS, int TX, int TY, int TZ, int STAGE, bool WENO>
 __global__ void __launch_bounds__(TX * TY * TZ, (Stage3dMinBlocks<TX * TY * TZ, TC>::v))
     stage3d_kernel(const Stage3DArgs<TS> A) {
   griddep_launch_dependents();  // programmatic dependent launch: see griddep_wait()
-  griddep_wait();
   constexpr int R2X = TX + 4, R2Y = TY + 4, R2Z = TZ + 4, R2 = R2X * R2Y * R2Z;
   constexpr int R1X = TX + 2, R1Y = TY + 2, R1Z = TZ + 2, R1 = R1X * R1Y * R1Z;
   constexpr int NT = TX * TY * TZ;
@@ -325,17 +324,18 @@ __global__ void __launch_bounds__(TX * TY * TZ, (Stage3dMinBlocks<TX * TY * TZ, 
   // and store, 10 Courant reduction and commit
   PhaseStamp ph;
   ph.begin(A.phase, STAGE);
-  if (tid == 0) {
-    s_err = 0;
-    double dt = A.dt_override > 0.0 ? A.dt_override : A.ctl->dt_cur;
-    if (!(dt > 0.0) || !(dt < 1e300)) err |= ERR_NONPHYS;
-    s_dt = dt;
-  }
+  if (tid == 0) s_err = 0;
   if (tid < R2X) s_gx[tid] = wrap_index(i0 - 2 + tid, nx);
   else if (tid < R2X + R2Y) s_gy[tid - R2X] = wrap_index(j0 - 2 + (tid - R2X), ny) * nx;
   else if (tid < R2X + R2Y + R2Z)
     s_gz[tid - R2X - R2Y] = wrap_index(k0 - 2 + (tid - R2X - R2Y), nz) * nx * ny;
   __syncthreads();
+  griddep_wait();  // the index tables need nothing from the kernel before
+  if (tid == 0) {
+    const double dt = A.dt_override > 0.0 ? A.dt_override : A.ctl->dt_cur;
+    if (!(dt > 0.0) || !(dt < 1e300)) err |= ERR_NONPHYS;
+    s_dt = dt;
+  }
 
   // ---- primitives where the limiter reads them; averages of the halo-1 box
   if (STAGE == 2) stage3d_prefetch_base<5, 15, TX, TY>(A, ncell, s_gx, s_gy, s_gz);

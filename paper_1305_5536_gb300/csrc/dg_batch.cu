@@ -98,10 +98,17 @@ __device__ __forceinline__ void sweep(const BatchArgs<TS>& B, unsigned char* sme
   }
 }
 
+// FP32: 80 registers a thread (the tile code plus the work list's; at the stage kernels'
+// 64 it spills: 48 problems 638 against 630 us a step).
+template <int NT, class TC>
+struct BatchMinBlocks {
+  static constexpr int v = sizeof(TC) == 4 ? 65536 / (80 * NT) : 1;
+};
+
 // WENO = false compiles the WENO-type limiter out (launches with limiter 0 or 1),
 // as in the single-problem stage kernels: the tile code is then the same.
 template <int EQ, class TC, class TS, int TX, int TY, bool WENO>
-__global__ void __launch_bounds__(TX * TY, (StageMinBlocks<TX * TY, TC>::v))
+__global__ void __launch_bounds__(TX * TY, (BatchMinBlocks<TX * TY, TC>::v))
     batch2d_kernel(const BatchArgs<TS> B) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   sweep<EQ, TC, TS, TX, TY, 1, WENO>(B, smem_raw);

@@ -33,13 +33,12 @@
 
 namespace dgk {
 
-// Shared-memory layout: one region that holds the staged averages [NV][R2], then in
-// place the centroid primitives, then the face fluxes [NF][NFX*NGF], [NF][NFY*NGF]; the
-// staged coefficients [NS][R1], replaced in place by the limited primitive gradients;
+// Shared-memory layout: one region that holds the centroid primitives [NP][R2], then
+// the face fluxes [NF][NFX*NGF], [NF][NFY*NGF]; the staged coefficients [NS][R1], replaced in place by the limited primitive gradients;
 // the limited conserved coefficients of the tile's own cells [NS][NT]; the predicted
 // centroid values [NP][R1].  The kernel is bound by latency and issue, so what counts is
 // the number of resident CTAs: 44 KB instead of 57 KB for the FP32 16x16 MHD tile (no
-// second copy of the averages, no limited coefficients of the ring) are 5 CTAs per SM
+// averages beside the primitives, no limited coefficients of the ring) are 5 CTAs per SM
 // instead of 3.
 template <int EQ, int TX, int TY, int NGF>
 struct MhTile2D {
@@ -47,9 +46,8 @@ struct MhTile2D {
   static constexpr int NV = T::NV, NS = T::NS, NP = T::NP, NF = T::NF, NT = T::NT;
   static constexpr int R2 = T::R2, R1 = T::R1, NFX = T::NFX, NFY = T::NFY;
   static constexpr int FSZ = NF * NGF * (NFX + NFY);
-  static constexpr int WSZ = NV * R2 > FSZ ? NV * R2 : FSZ;
+  static constexpr int WSZ = NP * R2 > FSZ ? NP * R2 : FSZ;
   static constexpr int ELEMS = WSZ + NS * R1 + NS * NT + NP * R1;
-  static_assert(NV == NP, "the primitives replace the averages in place");
 };
 
 template <int EQ, int TX, int TY, int NGF, class TC, int NT = TX * TY>
@@ -61,7 +59,7 @@ __host__ __device__ constexpr size_t mh2d_smem_bytes() {
 
 template <class TC>
 struct MhMem2D {
-  TileMem<TC> m;  // c0 = w (averages, primitives, fluxes), sl (gradients), gx, gy
+  TileMem<TC> m;  // w (primitives, fluxes), sl (gradients), gx, gy
   TC* wp;         // predicted centroid primitives [NP][R1]
   TC* ls;         // limited conserved coefficients of the tile [NS][NT]
 };
@@ -243,7 +241,7 @@ __device__ __forceinline__ void face_flux_prim2d(const Gas<TC>& G, int dir, cons
 template <int EQ, class TC, class TS, int TX, int TY, int NGF, bool WENO, int NT>
 __device__ __forceinline__ void mh2d_compute(const Stage2DArgs<TS>& A, int i0, int j0,
                                              unsigned nblk, const MhMem2D<TC>& MM,
-                                             TileScalars<NT>& S) {
+                                             TileScalars<NT>& S, unsigned err) {
   using Tr = Tr2<EQ>;
   constexpr int NV = Tr::NV, NS = Tr::NS, NP = Tr::NP, NF = Tr::NF;
   constexpr int R2X = TX + 4, R2Y = TY + 4, R2 = R2X * R2Y;
@@ -267,21 +265,9 @@ __device__ __forceinline__ void mh2d_compute(const Stage2DArgs<TS>& A, int i0, i
   const int nx = A.nx, ny = A.ny;
   const size_t ncell = (size_t)A.ncell;
   const Gas<TC> G = gas_of<TC>(A.gas);
-  unsigned err = 0;
   const double dt = S.dt;
   const TC dtc = Cvt<TC>::to_tc(dt);
   const TC hdt = TC(0.5) * dtc;
-
-  // ---- 1. centroid primitives of every staged cell, in place of its averages
-  for (int r = tid; r < R2; r += NT) {
-    TC c[NV], W[NP];
-#pragma unroll
-    for (int v = 0; v < NV; ++v) c[v] = s_w[v * R2 + r];
-    prims2d<EQ, TC>(G, c, W, err);
-#pragma unroll
-    for (int q = 0; q < NP; ++q) s_w[q * R2 + r] = W[q];
-  }
-  __syncthreads();
 
   const Geo2D<TS>& geo = A.geo;
   const TC hh[2] = {geo.hx, geo.hy};
@@ -380,7 +366,7 @@ __device__ __forceinline__ void mh2d_compute(const Stage2DArgs<TS>& A, int i0, i
   double o0[NV];
   if (mine) {
   const int r1 = (ly + 1) * R1X + lx + 1;
-  const size_t gc = (size_t)s_gy[ly + 2] + s_gx[lx + 2];
+  const unsigned gc = (unsigned)(s_gy[ly + 2] + s_gx[lx + 2]);
 
   TC sFx[NF], sFy[NF];
 #pragma unroll
@@ -436,14 +422,14 @@ __device__ __forceinline__ void mh2d_compute(const Stage2DArgs<TS>& A, int i0, i
   // U^{n+1} = U^n + dt L, U^n the limited step input
   TC os[NS];
 #pragma unroll
-  for (int v = 0; v < NV; ++v) o0[v] = fma(dt, Cvt<TC>::to_f64(rc0[v]), A.in.c0[v * ncell + gc]);
+  for (int v = 0; v < NV; ++v) o0[v] = fma(dt, Cvt<TC>::to_f64(rc0[v]), (A.in.c0 + v * ncell)[gc]);
 #pragma unroll
   for (int k = 0; k < NS; ++k) os[k] = s_ls[k * NC + tid] + dtc * rs[k];
   if (owner) {
 #pragma unroll
-    for (int v = 0; v < NV; ++v) A.out.c0[v * ncell + gc] = o0[v];
+    for (int v = 0; v < NV; ++v) (A.out.c0 + v * ncell)[gc] = o0[v];
 #pragma unroll
-    for (int k = 0; k < NS; ++k) A.out.sl[k * ncell + gc] = (TS)os[k];
+    for (int k = 0; k < NS; ++k) (A.out.sl + k * ncell)[gc] = (TS)os[k];
   }
   }  // mine
   courant_commit2d<EQ, TC, TS, NT>(A, G, owner, o0, dt, nblk, err, S);
@@ -469,9 +455,10 @@ __global__ void __launch_bounds__(NT, (MhMinBlocks<EQ, NT, NGF, WENO, TC>::v))
   __syncthreads();
   griddep_wait();
   stage2d_take_dt(A, S);
-  stage2d_load<EQ, TC, TS, TX, TY, NT>(A, M.m);
+  unsigned err = 0;
+  stage2d_load<EQ, TC, TS, TX, TY, NT, false>(A, M.m, gas_of<TC>(A.gas), err);
   __syncthreads();
-  mh2d_compute<EQ, TC, TS, TX, TY, NGF, WENO, NT>(A, i0, j0, gridDim.x * gridDim.y, M, S);
+  mh2d_compute<EQ, TC, TS, TX, TY, NGF, WENO, NT>(A, i0, j0, gridDim.x * gridDim.y, M, S, err);
 }
 
 }  // namespace dgk

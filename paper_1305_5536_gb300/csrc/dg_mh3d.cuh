@@ -141,10 +141,10 @@ __device__ __forceinline__ void prim_flux3d(const Gas<TC>& G, const TC* W, int d
   F[4] = (E + p) * vd;
 }
 
-// Exact-solver flux along axis d between primitive states (selects, as face_flux3d).
-template <class TC>
-__device__ __forceinline__ void face_flux_prim3d(const Gas<TC>& G, int d, const TC* WL,
-                                                 const TC* WR, TC* F, unsigned& err) {
+// Exact-solver flux along axis d between primitive states.
+template <int d, class TC>
+__device__ __forceinline__ void face_flux_prim3d(const Gas<TC>& G, const TC* WL, const TC* WR,
+                                                 TC* F, unsigned& err) {
   const TC nl = d == 0 ? WL[1] : (d == 1 ? WL[2] : WL[3]);
   const TC nr = d == 0 ? WR[1] : (d == 1 ? WR[2] : WR[3]);
   TC tl[2] = {d == 0 ? WL[2] : WL[1], d == 2 ? WL[2] : WL[3]};
@@ -217,14 +217,14 @@ __global__ void __launch_bounds__(TX * TY * TZ) mh3d_kernel(const Stage3DArgs<TS
   }
 
   // ---- 1. primitives of the halo-2 box; coefficients of the halo-1 box
-  stage3d_issue<5, 15, TX, TY, TZ>(A.in, ncell, s_gx, s_gy, s_gz, s_g);
+  stage3d_issue<5, 15, TX, TY, TZ, TS, TC, 0, 0, false>(A.in, ncell, s_gx, s_gy, s_gz, s_g);
   for (int r = tid; r < R2; r += NT) {
     int rz = r / (R2X * R2Y), rr = r - rz * (R2X * R2Y);
     int ry = rr / R2X, rx = rr - ry * R2X;
-    size_t g = (size_t)s_gz[rz] + s_gy[ry] + s_gx[rx];
+    const unsigned g = (unsigned)(s_gz[rz] + s_gy[ry] + s_gx[rx]);
     TC c[5], W[5];
 #pragma unroll
-    for (int v = 0; v < 5; ++v) c[v] = Cvt<TC>::to_tc(__ldg(&A.in.c0[v * ncell + g]));
+    for (int v = 0; v < 5; ++v) c[v] = Cvt<TC>::to_tc(__ldg(&(A.in.c0 + v * ncell)[g]));
     prims3d<TC>(G, c, W, err);
 #pragma unroll
     for (int q = 0; q < 5; ++q) s_w[q * R2 + r] = W[q];
@@ -297,21 +297,18 @@ __global__ void __launch_bounds__(TX * TY * TZ) mh3d_kernel(const Stage3DArgs<TS
       for (int d = 0; d < 3; ++d) rs[3 * v + d] = geo.cs[d] * sF[d][v];
   }
 
-  // ---- 4. faces, one orientation at a time (rolled loop: one copy of the solver)
-#pragma unroll 1
-  for (int d = 0; d < 3; ++d) {
-    const int FX = TX + (d == 0), FY = TY + (d == 1), FZ = TZ + (d == 2);
-    const int NFACE = FX * FY * FZ;
-    static_assert((TX + 1) * (TY + 1) * (TZ + 1) < 16384 && (TX + 1) * (TY + 1) <= 1024,
-                  "face indices within the exact range of div_by_magic");
-    const unsigned mXY = div_magic(FX * FY), mX = div_magic(FX);
-    const int step = d == 0 ? 1 : (d == 1 ? R1X : R1X * R1Y);
+  // ---- 4. faces, one orientation at a time
+  auto orient = [&](auto dc) {
+    constexpr int d = dc;
+    constexpr int FX = TX + (d == 0), FY = TY + (d == 1), FZ = TZ + (d == 2);
+    constexpr int NFACE = FX * FY * FZ;
+    constexpr int step = d == 0 ? 1 : (d == 1 ? R1X : R1X * R1Y);
     const TC hn = d == 0 ? hh[0] : (d == 1 ? hh[1] : hh[2]);
     const TC o1 = d == 0 ? oo[1] : oo[0], o2 = d == 2 ? oo[1] : oo[2];
     for (int e = tid; e < NPT * NFACE; e += NT) {
       const int f = NPT == 4 ? (e >> 2) : e, g = NPT == 4 ? (e & 3) : 0;
-      const int fz = div_by_magic(f, mXY), fr = f - fz * (FX * FY);
-      const int fy = div_by_magic(fr, mX), fx = fr - fy * FX;
+      const int fz = f / (FX * FY), fr = f - fz * (FX * FY);
+      const int fy = fr / FX, fx = fr - fy * FX;
       // + side cell: halo-1 coordinates (fx+1, fy+1, fz+1); - side one step back
       const int r1r = ((fz + 1) * R1Y + (fy + 1)) * R1X + (fx + 1);
       const int r1l = r1r - step;
@@ -323,7 +320,7 @@ __global__ void __launch_bounds__(TX * TY * TZ) mh3d_kernel(const Stage3DArgs<TS
       TC WL[5], WR[5], F[5];
       mh_eval3d<TC>(s_wp + r1l, s_g + r1l, R1, xl, yl, zl, WL);
       mh_eval3d<TC>(s_wp + r1r, s_g + r1r, R1, xr, yr, zr, WR);
-      face_flux_prim3d<TC>(G, d, WL, WR, F, err);
+      face_flux_prim3d<d, TC>(G, WL, WR, F, err);
 #pragma unroll
       for (int v = 0; v < 5; ++v) s_f[(v * FMAX + f) * NPT + g] = F[v];
     }
@@ -332,46 +329,45 @@ __global__ void __launch_bounds__(TX * TY * TZ) mh3d_kernel(const Stage3DArgs<TS
       const int fm = (lz * FY + ly) * FX + lx;
       const int fp = fm + (d == 0 ? 1 : (d == 1 ? FX : FX * FY));
       if (NPT == 4) {
-        if (d == 0) gather3d<0, TC>(s_f, FMAX, fm, fp, geo, rc0, rs);
-        else if (d == 1) gather3d<1, TC>(s_f, FMAX, fm, fp, geo, rc0, rs);
-        else gather3d<2, TC>(s_f, FMAX, fm, fp, geo, rc0, rs);
+        gather3d<d, TC>(s_f, FMAX, fm, fp, geo, rc0, rs);
       } else {
-        if (d == 0) gather3d_centroid<0, TC>(s_f, FMAX, fm, fp, geo, rc0, rs);
-        else if (d == 1) gather3d_centroid<1, TC>(s_f, FMAX, fm, fp, geo, rc0, rs);
-        else gather3d_centroid<2, TC>(s_f, FMAX, fm, fp, geo, rc0, rs);
+        gather3d_centroid<d, TC>(s_f, FMAX, fm, fp, geo, rc0, rs);
       }
     }
     __syncthreads();
-  }
+  };
+  orient(std::integral_constant<int, 0>{});
+  orient(std::integral_constant<int, 1>{});
+  orient(std::integral_constant<int, 2>{});
 
   // ---- 5. update of the limited coefficients, Courant speed of the new state
   const int gi = i0 + lx, gj = j0 + ly, gk = k0 + lz;
   const bool owner = gi < nx && gj < ny && gk < nz;
-  const size_t gc = (size_t)s_gz[lz + 2] + s_gy[ly + 2] + s_gx[lx + 2];
+  const unsigned gc = (unsigned)(s_gz[lz + 2] + s_gy[ly + 2] + s_gx[lx + 2]);
   TC sn[15];
   if (A.limiter) {
     TC c[5], W[5], g[15];
 #pragma unroll
-    for (int v = 0; v < 5; ++v) c[v] = Cvt<TC>::to_tc(A.in.c0[v * ncell + gc]);
+    for (int v = 0; v < 5; ++v) c[v] = Cvt<TC>::to_tc((A.in.c0 + v * ncell)[gc]);
     prims3d<TC>(G, c, W, err);
 #pragma unroll
     for (int k = 0; k < 15; ++k) g[k] = s_g[k * R1 + r1c];
     mh_cons3d<TC>(G, W, g, sn);
   } else {
 #pragma unroll
-    for (int k = 0; k < 15; ++k) sn[k] = (TC)A.in.sl[k * ncell + gc];
+    for (int k = 0; k < 15; ++k) sn[k] = (TC)(A.in.sl + k * ncell)[gc];
   }
   double o0[5];
   TC os[15];
 #pragma unroll
-  for (int v = 0; v < 5; ++v) o0[v] = fma(dt, Cvt<TC>::to_f64(rc0[v]), A.in.c0[v * ncell + gc]);
+  for (int v = 0; v < 5; ++v) o0[v] = fma(dt, Cvt<TC>::to_f64(rc0[v]), (A.in.c0 + v * ncell)[gc]);
 #pragma unroll
   for (int k = 0; k < 15; ++k) os[k] = sn[k] + dtc * rs[k];
   if (owner) {
 #pragma unroll
-    for (int v = 0; v < 5; ++v) A.out.c0[v * ncell + gc] = o0[v];
+    for (int v = 0; v < 5; ++v) (A.out.c0 + v * ncell)[gc] = o0[v];
 #pragma unroll
-    for (int k = 0; k < 15; ++k) A.out.sl[k * ncell + gc] = (TS)os[k];
+    for (int k = 0; k < 15; ++k) (A.out.sl + k * ncell)[gc] = (TS)os[k];
   }
 
   TC sp = TC(0);

@@ -202,10 +202,10 @@ __global__ void __launch_bounds__(TX * TY * TZ) mh3m_kernel(const Stage3DArgs<TS
   for (int r = tid; r < R2; r += NT) {
     int rz = r / (R2X * R2Y), rr = r - rz * (R2X * R2Y);
     int ry = rr / R2X, rx = rr - ry * R2X;
-    size_t g = (size_t)s_gz[rz] + s_gy[ry] + s_gx[rx];
+    const unsigned g = (unsigned)(s_gz[rz] + s_gy[ry] + s_gx[rx]);
     TC c[8], W[8];
 #pragma unroll
-    for (int v = 0; v < 8; ++v) c[v] = Cvt<TC>::to_tc(__ldg(&A.in.c0[v * ncell + g]));
+    for (int v = 0; v < 8; ++v) c[v] = Cvt<TC>::to_tc(__ldg(&(A.in.c0 + v * ncell)[g]));
     prims3m<TC>(G, c, W, err);
 #pragma unroll
     for (int q = 0; q < 8; ++q) s_w[q * R2 + r] = W[q];
@@ -279,21 +279,18 @@ __global__ void __launch_bounds__(TX * TY * TZ) mh3m_kernel(const Stage3DArgs<TS
     }
   }
 
-  // ---- 4. faces, one orientation at a time (rolled loop: one copy of the solver)
-#pragma unroll 1
-  for (int d = 0; d < 3; ++d) {
-    const int FX = TX + (d == 0), FY = TY + (d == 1), FZ = TZ + (d == 2);
-    const int NFACE = FX * FY * FZ;
-    static_assert((TX + 1) * (TY + 1) * (TZ + 1) < 16384 && (TX + 1) * (TY + 1) <= 1024,
-                  "face indices within the exact range of div_by_magic");
-    const unsigned mXY = div_magic(FX * FY), mX = div_magic(FX);
-    const int step = d == 0 ? 1 : (d == 1 ? R1X : R1X * R1Y);
+  // ---- 4. faces, one orientation at a time
+  auto orient = [&](auto dc) {
+    constexpr int d = dc;
+    constexpr int FX = TX + (d == 0), FY = TY + (d == 1), FZ = TZ + (d == 2);
+    constexpr int NFACE = FX * FY * FZ;
+    constexpr int step = d == 0 ? 1 : (d == 1 ? R1X : R1X * R1Y);
     const TC hn = d == 0 ? hh[0] : (d == 1 ? hh[1] : hh[2]);
     const TC o1 = d == 0 ? oo[1] : oo[0], o2 = d == 2 ? oo[1] : oo[2];
     for (int e = tid; e < NPT * NFACE; e += NT) {
       const int f = NPT == 4 ? (e >> 2) : e, g = NPT == 4 ? (e & 3) : 0;
-      const int fz = div_by_magic(f, mXY), fr = f - fz * (FX * FY);
-      const int fy = div_by_magic(fr, mX), fx = fr - fy * FX;
+      const int fz = f / (FX * FY), fr = f - fz * (FX * FY);
+      const int fy = fr / FX, fx = fr - fy * FX;
       // + side cell: halo-1 coordinates (fx+1, fy+1, fz+1); - side one step back
       const int r1r = ((fz + 1) * R1Y + (fy + 1)) * R1X + (fx + 1);
       const int r1l = r1r - step;
@@ -305,7 +302,7 @@ __global__ void __launch_bounds__(TX * TY * TZ) mh3m_kernel(const Stage3DArgs<TS
       TC WL[8], WR[8], F[8];
       mh_eval3m<TC>(s_wp + r1l, s_g + r1l, R1, xl, yl, zl, WL);
       mh_eval3m<TC>(s_wp + r1r, s_g + r1r, R1, xr, yr, zr, WR);
-      face_flux_prim3m<TC>(G, d, WL, WR, F, err);
+      face_flux_prim3m<d, TC>(G, WL, WR, F, err);
 #pragma unroll
       for (int v = 0; v < 8; ++v) s_f[(v * FMAX + f) * NPT + g] = F[v];
     }
@@ -315,31 +312,18 @@ __global__ void __launch_bounds__(TX * TY * TZ) mh3m_kernel(const Stage3DArgs<TS
       const int fp = fm + (d == 0 ? 1 : (d == 1 ? FX : FX * FY));
       const TC* s_fb = s_f + 5 * FMAX * NPT;  // the three field components
       if (NPT == 4) {
-        if (d == 0) {
-          gather3d<0, TC>(s_f, FMAX, fm, fp, geo, rc0, rs);
-          gather3d<0, TC, 3>(s_fb, FMAX, fm, fp, geo, rc0 + 5, rs + 15);
-        } else if (d == 1) {
-          gather3d<1, TC>(s_f, FMAX, fm, fp, geo, rc0, rs);
-          gather3d<1, TC, 3>(s_fb, FMAX, fm, fp, geo, rc0 + 5, rs + 15);
-        } else {
-          gather3d<2, TC>(s_f, FMAX, fm, fp, geo, rc0, rs);
-          gather3d<2, TC, 3>(s_fb, FMAX, fm, fp, geo, rc0 + 5, rs + 15);
-        }
+        gather3d<d, TC>(s_f, FMAX, fm, fp, geo, rc0, rs);
+        gather3d<d, TC, 3>(s_fb, FMAX, fm, fp, geo, rc0 + 5, rs + 15);
       } else {
-        if (d == 0) {
-          gather3d_centroid<0, TC>(s_f, FMAX, fm, fp, geo, rc0, rs);
-          gather3d_centroid<0, TC, 3>(s_fb, FMAX, fm, fp, geo, rc0 + 5, rs + 15);
-        } else if (d == 1) {
-          gather3d_centroid<1, TC>(s_f, FMAX, fm, fp, geo, rc0, rs);
-          gather3d_centroid<1, TC, 3>(s_fb, FMAX, fm, fp, geo, rc0 + 5, rs + 15);
-        } else {
-          gather3d_centroid<2, TC>(s_f, FMAX, fm, fp, geo, rc0, rs);
-          gather3d_centroid<2, TC, 3>(s_fb, FMAX, fm, fp, geo, rc0 + 5, rs + 15);
-        }
+        gather3d_centroid<d, TC>(s_f, FMAX, fm, fp, geo, rc0, rs);
+        gather3d_centroid<d, TC, 3>(s_fb, FMAX, fm, fp, geo, rc0 + 5, rs + 15);
       }
     }
     __syncthreads();
-  }
+  };
+  orient(std::integral_constant<int, 0>{});
+  orient(std::integral_constant<int, 1>{});
+  orient(std::integral_constant<int, 2>{});
   TC rsl[23];
 #pragma unroll
   for (int k = 0; k < 15; ++k) rsl[k] = rs[k];
@@ -348,12 +332,12 @@ __global__ void __launch_bounds__(TX * TY * TZ) mh3m_kernel(const Stage3DArgs<TS
   // ---- 5. update of the limited coefficients, Courant speed of the new state
   const int gi = i0 + lx, gj = j0 + ly, gk = k0 + lz;
   const bool owner = gi < nx && gj < ny && gk < nz;
-  const size_t gc = (size_t)s_gz[lz + 2] + s_gy[ly + 2] + s_gx[lx + 2];
+  const unsigned gc = (unsigned)(s_gz[lz + 2] + s_gy[ly + 2] + s_gx[lx + 2]);
   TC sn[23];
   if (A.limiter) {
     TC c[8], W[8], g[15], gB[3][3];
 #pragma unroll
-    for (int v = 0; v < 8; ++v) c[v] = Cvt<TC>::to_tc(A.in.c0[v * ncell + gc]);
+    for (int v = 0; v < 8; ++v) c[v] = Cvt<TC>::to_tc((A.in.c0 + v * ncell)[gc]);
     prims3m<TC>(G, c, W, err);
 #pragma unroll
     for (int k = 0; k < 15; ++k) g[k] = s_g[k * R1 + r1c];
@@ -363,19 +347,19 @@ __global__ void __launch_bounds__(TX * TY * TZ) mh3m_kernel(const Stage3DArgs<TS
     mh_cons3m<TC>(G, W, g, gB, sn);
   } else {
 #pragma unroll
-    for (int k = 0; k < 23; ++k) sn[k] = (TC)A.in.sl[k * ncell + gc];
+    for (int k = 0; k < 23; ++k) sn[k] = (TC)(A.in.sl + k * ncell)[gc];
   }
   double o0[8];
   TC os[23];
 #pragma unroll
-  for (int v = 0; v < 8; ++v) o0[v] = fma(dt, Cvt<TC>::to_f64(rc0[v]), A.in.c0[v * ncell + gc]);
+  for (int v = 0; v < 8; ++v) o0[v] = fma(dt, Cvt<TC>::to_f64(rc0[v]), (A.in.c0 + v * ncell)[gc]);
 #pragma unroll
   for (int k = 0; k < 23; ++k) os[k] = sn[k] + dtc * rsl[k];
   if (owner) {
 #pragma unroll
-    for (int v = 0; v < 8; ++v) A.out.c0[v * ncell + gc] = o0[v];
+    for (int v = 0; v < 8; ++v) (A.out.c0 + v * ncell)[gc] = o0[v];
 #pragma unroll
-    for (int k = 0; k < 23; ++k) A.out.sl[k * ncell + gc] = (TS)os[k];
+    for (int k = 0; k < 23; ++k) (A.out.sl + k * ncell)[gc] = (TS)os[k];
   }
 
   TC sp = TC(0);

@@ -94,15 +94,23 @@ __global__ void __launch_bounds__(TX * TY)
       }
       phase ^= 1u;
     }
+    unsigned err = 0;
     if (use_raw) {
-      for (int e = tid; e < T::NV * T::R2; e += T::NT) M.c0[e] = Cvt<TC>::to_tc(raw_c0[e]);
+      for (int r = tid; r < T::R2; r += T::NT) {
+        TC c[T::NV], W[T::NP];
+#pragma unroll
+        for (int v = 0; v < T::NV; ++v) M.c0[v * T::R2 + r] = c[v] = Cvt<TC>::to_tc(raw_c0[v * T::R2 + r]);
+        prims2d<EQ, TC>(gas_of<TC>(A.gas), c, W, err);
+#pragma unroll
+        for (int q = 0; q < T::NP; ++q) M.w[q * T::R2 + r] = W[q];
+      }
       for (int e = tid; e < T::NS * T::R1; e += T::NT) {
         const int v = e / T::R1, r = e - v * T::R1;
         const int ry = r / T::R1X, rx = r - ry * T::R1X;
         M.sl[e] = (TC)raw_sl[(v * T::R1Y + ry) * B::SXW + rx + B::SOFF];
       }
     } else {
-      stage2d_load<EQ, TC, TS, TX, TY>(A, M);
+      stage2d_load<EQ, TC, TS, TX, TY, T::NT>(A, M, gas_of<TC>(A.gas), err);
     }
     fence_proxy_async_smem();
     __syncthreads();
@@ -110,7 +118,7 @@ __global__ void __launch_bounds__(TX * TY)
     const int tn = t + gridDim.x;
     pending = tma_ok && tn < ntiles && interior((tn % tiles_x) * TX, (tn / tiles_x) * TY);
     if (tid == 0 && pending) issue((tn % tiles_x) * TX, (tn / tiles_x) * TY);
-    stage2d_compute<EQ, TC, TS, TX, TY, STAGE>(A, i0, j0, (unsigned)ntiles, M, S);
+    stage2d_compute<EQ, TC, TS, TX, TY, STAGE>(A, i0, j0, (unsigned)ntiles, M, S, err);
   }
 }
 

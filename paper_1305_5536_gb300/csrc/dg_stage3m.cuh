@@ -268,42 +268,33 @@ __device__ __forceinline__ void phys_flux3m(const Gas<TC>& G, const TC* c, int d
   F[4] = (c[4] + pT) * vd - Bd * vB;
 }
 
-// HLLD flux through a face along axis d (uniform across the CTA) between the
-// primitive states Wl, Wr (rho, v, p, B), with the normal field replaced by the
-// average of both sides (Sec. 2.6); lab frame, component order of phys_flux3m.
-// The face frame is (n, t1, t2) = (d, d+1, d+2) cyclically, picked with selects.
-template <class TC>
-__device__ __forceinline__ void face_flux_prim3m(const Gas<TC>& G, int d, const TC* Wl,
-                                                 const TC* Wr, TC* F, unsigned& err) {
-  auto pick = [&](const TC* W, int o, int k) {  // component k (0 n, 1 t1, 2 t2) of W[o..o+2]
-    const int a = d + k >= 3 ? d + k - 3 : d + k;
-    return a == 0 ? W[o] : (a == 1 ? W[o + 1] : W[o + 2]);
-  };
-  const TC bn = TC(0.5) * (pick(Wl, 5, 0) + pick(Wr, 5, 0));
+// HLLD flux through a face along axis d between the primitive states Wl, Wr (rho, v, p,
+// B), with the normal field replaced by the average of both sides (Sec. 2.6); lab frame,
+// component order of phys_flux3m.  The face frame is (n, t1, t2) = (d, d+1, d+2)
+// cyclically.  d is a template parameter, as in face_flux3d.
+template <int d, class TC>
+__device__ __forceinline__ void face_flux_prim3m(const Gas<TC>& G, const TC* Wl, const TC* Wr,
+                                                 TC* F, unsigned& err) {
+  constexpr int e = (d + 1) % 3, f = (d + 2) % 3;
+  const TC bn = TC(0.5) * (Wl[5 + d] + Wr[5 + d]);
   TC Ff[7];
-  hlld_flux3<TC>(G, Wl[0], pick(Wl, 1, 0), pick(Wl, 1, 1), pick(Wl, 1, 2), Wl[4], pick(Wl, 5, 1),
-                 pick(Wl, 5, 2), Wr[0], pick(Wr, 1, 0), pick(Wr, 1, 1), pick(Wr, 1, 2), Wr[4],
-                 pick(Wr, 5, 1), pick(Wr, 5, 2), bn, Ff, err);
-  // lab component a is face component k = a - d (mod 3)
+  hlld_flux3<TC>(G, Wl[0], Wl[1 + d], Wl[1 + e], Wl[1 + f], Wl[4], Wl[5 + e], Wl[5 + f], Wr[0],
+                 Wr[1 + d], Wr[1 + e], Wr[1 + f], Wr[4], Wr[5 + e], Wr[5 + f], bn, Ff, err);
   F[0] = Ff[0];
   F[4] = Ff[4];
-#pragma unroll
-  for (int a = 0; a < 3; ++a) {
-    const int k = a - d < 0 ? a - d + 3 : a - d;
-    F[1 + a] = k == 0 ? Ff[1] : (k == 1 ? Ff[2] : Ff[3]);
-    F[5 + a] = k == 0 ? TC(0) : (k == 1 ? Ff[5] : Ff[6]);
-  }
+  F[1 + d] = Ff[1]; F[1 + e] = Ff[2]; F[1 + f] = Ff[3];
+  F[5 + d] = TC(0); F[5 + e] = Ff[5]; F[5 + f] = Ff[6];
 }
 
 // The same between conserved states cl, cr (the solver checks positivity).
-template <class TC>
-__device__ __forceinline__ void face_flux3m(const Gas<TC>& G, int d, const TC* cl, const TC* cr,
-                                            TC* F, unsigned& err) {
+template <int d, class TC>
+__device__ __forceinline__ void face_flux3m(const Gas<TC>& G, const TC* cl, const TC* cr, TC* F,
+                                            unsigned& err) {
   TC Wl[8], Wr[8];
   unsigned e2 = 0;
   prims3m<TC>(G, cl, Wl, e2);
   prims3m<TC>(G, cr, Wr, e2);
-  face_flux_prim3m<TC>(G, d, Wl, Wr, F, err);
+  face_flux_prim3m<d, TC>(G, Wl, Wr, F, err);
 }
 
 // Field part of the right-hand side from the Taylor-like gathers r[3*(5+i)+d].
@@ -378,10 +369,10 @@ __global__ void __launch_bounds__(TX * TY * TZ, (Stage3mMinBlocks<TX * TY * TZ, 
     int rx, ry, rz;
     halo3d_cell<TX, TY, TZ>(e, rx, ry, rz);
     const int r = (rz * R2Y + ry) * R2X + rx;
-    size_t g = (size_t)s_gz[rz] + s_gy[ry] + s_gx[rx];
+    const unsigned g = (unsigned)(s_gz[rz] + s_gy[ry] + s_gx[rx]);
     TC c[8], W[8];
 #pragma unroll
-    for (int v = 0; v < 8; ++v) c[v] = Cvt<TC>::to_tc(__ldg(&A.in.c0[v * ncell + g]));
+    for (int v = 0; v < 8; ++v) c[v] = Cvt<TC>::to_tc(__ldg(&(A.in.c0 + v * ncell)[g]));
     prims3m<TC>(G, c, W, err);
 #pragma unroll
     for (int q = 0; q < 8; ++q) s_w[q * R2 + r] = W[q];
@@ -455,14 +446,11 @@ __global__ void __launch_bounds__(TX * TY * TZ, (Stage3mMinBlocks<TX * TY * TZ, 
   }
 
   // ---- faces, one orientation at a time
-#pragma unroll 1
-  for (int d = 0; d < 3; ++d) {
-    const int FX = TX + (d == 0), FY = TY + (d == 1), FZ = TZ + (d == 2);
-    const int NFACE = FX * FY * FZ;
-    static_assert((TX + 1) * (TY + 1) * (TZ + 1) < 16384 && (TX + 1) * (TY + 1) <= 1024,
-                  "face indices within the exact range of div_by_magic");
-    const unsigned mXY = div_magic(FX * FY), mX = div_magic(FX);
-    const int step = d == 0 ? 1 : (d == 1 ? R1X : R1X * R1Y);
+  auto orient = [&](auto dc) {
+    constexpr int d = dc;
+    constexpr int FX = TX + (d == 0), FY = TY + (d == 1), FZ = TZ + (d == 2);
+    constexpr int NFACE = FX * FY * FZ;
+    constexpr int step = d == 0 ? 1 : (d == 1 ? R1X : R1X * R1Y);
     const TC hn = d == 0 ? hh[0] : (d == 1 ? hh[1] : hh[2]);
     const TC o1 = d == 0 ? oo[1] : oo[0], o2 = d == 2 ? oo[1] : oo[2];
     // a thread takes the two points of a face at one side of the first transverse axis: 62
@@ -471,8 +459,8 @@ __global__ void __launch_bounds__(TX * TY * TZ, (Stage3mMinBlocks<TX * TY * TZ, 
     // with one point per thread)
     for (int e = tid; e < 2 * NFACE; e += NT) {
       const int f = e >> 1, ga = e & 1;
-      const int fz = div_by_magic(f, mXY), fr = f - fz * (FX * FY);
-      const int fy = div_by_magic(fr, mX), fx = fr - fy * FX;
+      const int fz = f / (FX * FY), fr = f - fz * (FX * FY);
+      const int fy = fr / FX, fx = fr - fy * FX;
       const int r1r = ((fz + 1) * R1Y + (fy + 1)) * R1X + (fx + 1);
       const int r1l = r1r - step;
       const TC a = ga ? o1 : -o1;
@@ -504,7 +492,7 @@ __global__ void __launch_bounds__(TX * TY * TZ, (Stage3mMinBlocks<TX * TY * TZ, 
           cl[v] = ml[v] + tl[v] * b;
           cr[v] = mr[v] + tr[v] * b;
         }
-        face_flux3m<TC>(G, d, cl, cr, F, err);
+        face_flux3m<d, TC>(G, cl, cr, F, err);
 #pragma unroll
         for (int v = 0; v < 8; ++v) s_f[(v * FMAX + f) * 4 + 2 * ga + gb] = F[v];
       }
@@ -514,19 +502,14 @@ __global__ void __launch_bounds__(TX * TY * TZ, (Stage3mMinBlocks<TX * TY * TZ, 
       const int fm = (lz * FY + ly) * FX + lx;
       const int fp = fm + (d == 0 ? 1 : (d == 1 ? FX : FX * FY));
       // gather3d for the 5 Taylor variables and the 3 field components
-      if (d == 0) {
-        gather3d<0, TC>(s_f, FMAX, fm, fp, geo, rc0, rs);
-        gather3d<0, TC, 3>(s_f + 5 * FMAX * 4, FMAX, fm, fp, geo, rc0 + 5, rs + 15);
-      } else if (d == 1) {
-        gather3d<1, TC>(s_f, FMAX, fm, fp, geo, rc0, rs);
-        gather3d<1, TC, 3>(s_f + 5 * FMAX * 4, FMAX, fm, fp, geo, rc0 + 5, rs + 15);
-      } else {
-        gather3d<2, TC>(s_f, FMAX, fm, fp, geo, rc0, rs);
-        gather3d<2, TC, 3>(s_f + 5 * FMAX * 4, FMAX, fm, fp, geo, rc0 + 5, rs + 15);
-      }
+      gather3d<d, TC>(s_f, FMAX, fm, fp, geo, rc0, rs);
+      gather3d<d, TC, 3>(s_f + 5 * FMAX * 4, FMAX, fm, fp, geo, rc0 + 5, rs + 15);
     }
     __syncthreads();
-  }
+  };
+  orient(std::integral_constant<int, 0>{});
+  orient(std::integral_constant<int, 1>{});
+  orient(std::integral_constant<int, 2>{});
   TC rsl[23];
 #pragma unroll
   for (int k = 0; k < 15; ++k) rsl[k] = rs[k];
@@ -535,33 +518,33 @@ __global__ void __launch_bounds__(TX * TY * TZ, (Stage3mMinBlocks<TX * TY * TZ, 
   // ---- Runge-Kutta combination
   const int gi = i0 + lx, gj = j0 + ly, gk = k0 + lz;
   const bool owner = gi < nx && gj < ny && gk < nz;
-  const size_t gc = (size_t)s_gz[lz + 2] + s_gy[ly + 2] + s_gx[lx + 2];
+  const unsigned gc = (unsigned)(s_gz[lz + 2] + s_gy[ly + 2] + s_gx[lx + 2]);
   const double dt = s_dt;
   const TC dtc = Cvt<TC>::to_tc(dt);
   double o0[8];
   TC os[23];
   if (STAGE == 1) {
 #pragma unroll
-    for (int v = 0; v < 8; ++v) o0[v] = fma(dt, Cvt<TC>::to_f64(rc0[v]), A.in.c0[v * ncell + gc]);
+    for (int v = 0; v < 8; ++v) o0[v] = fma(dt, Cvt<TC>::to_f64(rc0[v]), (A.in.c0 + v * ncell)[gc]);
 #pragma unroll
     for (int k = 0; k < 23; ++k) os[k] = s_sl[k * R1 + r1c] + dtc * rsl[k];
     if (A.limiter && A.lim_sl && owner) {
 #pragma unroll
-      for (int k = 0; k < 23; ++k) A.lim_sl[k * ncell + gc] = (TS)s_sl[k * R1 + r1c];
+      for (int k = 0; k < 23; ++k) (A.lim_sl + k * ncell)[gc] = (TS)s_sl[k * R1 + r1c];
     }
   } else {
     TC sn[23];
     if (A.limiter && A.lim_sl) {
 #pragma unroll
-      for (int k = 0; k < 23; ++k) sn[k] = (TC)A.lim_sl[k * ncell + gc];
+      for (int k = 0; k < 23; ++k) sn[k] = (TC)(A.lim_sl + k * ncell)[gc];
     } else {
 #pragma unroll
-      for (int k = 0; k < 23; ++k) sn[k] = (TC)A.base.sl[k * ncell + gc];
+      for (int k = 0; k < 23; ++k) sn[k] = (TC)(A.base.sl + k * ncell)[gc];
     }
     if (A.limiter && !A.lim_sl) {
       TC c[8], W[8], Wn[6][8];
 #pragma unroll
-      for (int v = 0; v < 8; ++v) c[v] = Cvt<TC>::to_tc(A.base.c0[v * ncell + gc]);
+      for (int v = 0; v < 8; ++v) c[v] = Cvt<TC>::to_tc((A.base.c0 + v * ncell)[gc]);
       prims3m<TC>(G, c, W, err);
       const size_t nb[6] = {(size_t)s_gz[lz + 2] + s_gy[ly + 2] + s_gx[lx + 1],
                             (size_t)s_gz[lz + 2] + s_gy[ly + 2] + s_gx[lx + 3],
@@ -572,24 +555,24 @@ __global__ void __launch_bounds__(TX * TY * TZ, (Stage3mMinBlocks<TX * TY * TZ, 
 #pragma unroll
       for (int k = 0; k < 6; ++k) {
 #pragma unroll
-        for (int v = 0; v < 8; ++v) c[v] = Cvt<TC>::to_tc(A.base.c0[v * ncell + nb[k]]);
+        for (int v = 0; v < 8; ++v) c[v] = Cvt<TC>::to_tc((A.base.c0 + v * ncell)[nb[k]]);
         prims3m<TC>(G, c, Wn[k], err);
       }
       limit3m<TC, WENO>(G, hh, W, Wn, sn);
     }
 #pragma unroll
     for (int v = 0; v < 8; ++v)
-      o0[v] = half_f64(A.base.c0[v * ncell + gc] +
-                       fma(dt, Cvt<TC>::to_f64(rc0[v]), A.in.c0[v * ncell + gc]));
+      o0[v] = half_f64((A.base.c0 + v * ncell)[gc] +
+                       fma(dt, Cvt<TC>::to_f64(rc0[v]), (A.in.c0 + v * ncell)[gc]));
 #pragma unroll
     for (int k = 0; k < 23; ++k)
       os[k] = TC(0.5) * sn[k] + TC(0.5) * (s_sl[k * R1 + r1c] + dtc * rsl[k]);
   }
   if (owner) {
 #pragma unroll
-    for (int v = 0; v < 8; ++v) A.out.c0[v * ncell + gc] = o0[v];
+    for (int v = 0; v < 8; ++v) (A.out.c0 + v * ncell)[gc] = o0[v];
 #pragma unroll
-    for (int k = 0; k < 23; ++k) A.out.sl[k * ncell + gc] = (TS)os[k];
+    for (int k = 0; k < 23; ++k) (A.out.sl + k * ncell)[gc] = (TS)os[k];
   }
 
   if (STAGE == 2) {

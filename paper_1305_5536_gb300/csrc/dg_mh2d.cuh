@@ -33,10 +33,11 @@
 
 namespace dgk {
 
-// Shared-memory layout: one region that holds the centroid primitives [NP][R2], then
-// the face fluxes [NF][NFX*NGF], [NF][NFY*NGF]; the staged coefficients [NS][R1], replaced in place by the limited primitive gradients;
-// the limited conserved coefficients of the tile's own cells [NS][NT]; the predicted
-// centroid values [NP][R1].  The kernel is bound by latency and issue, so what counts is
+// Shared-memory layout: a record per cell of the halo-1 region (Tile2D) that takes the
+// staged coefficients and then the predicted centroid values and the limited primitive
+// gradients; one region that holds the centroid primitives [NP][R2], then the face fluxes
+// [NF][NFX*NGF], [NF][NFY*NGF]; the limited conserved coefficients of the tile's own cells
+// [8][NT] (the field's are its gradients, in the record).  The kernel is bound by latency and issue, so what counts is
 // the number of resident CTAs: 44 KB instead of 57 KB for the FP32 16x16 MHD tile (no
 // averages beside the primitives, no limited coefficients of the ring) are 5 CTAs per SM
 // instead of 3.
@@ -47,7 +48,7 @@ struct MhTile2D {
   static constexpr int R2 = T::R2, R1 = T::R1, NFX = T::NFX, NFY = T::NFY;
   static constexpr int FSZ = NF * NGF * (NFX + NFY);
   static constexpr int WSZ = NP * R2 > FSZ ? NP * R2 : FSZ;
-  static constexpr int ELEMS = WSZ + NS * R1 + NS * NT + NP * R1;
+  static constexpr int ELEMS = T::REC * R1 + (WSZ + 3) / 4 * 4 + 8 * NT;
 };
 
 template <int EQ, int TX, int TY, int NGF, class TC, int NT = TX * TY>
@@ -59,9 +60,8 @@ __host__ __device__ constexpr size_t mh2d_smem_bytes() {
 
 template <class TC>
 struct MhMem2D {
-  TileMem<TC> m;  // w (primitives, fluxes), sl (gradients), gx, gy
-  TC* wp;         // predicted centroid primitives [NP][R1]
-  TC* ls;         // limited conserved coefficients of the tile [NS][NT]
+  TileMem<TC> m;  // records (predicted values, gradients), w (primitives, fluxes), gx, gy
+  TC* ls;         // limited conserved coefficients of the tile [8][NT]
 };
 
 template <int EQ, int TX, int TY, int NGF, class TC>
@@ -69,11 +69,10 @@ __device__ __forceinline__ MhMem2D<TC> mh2d_mem(unsigned char* base) {
   using T = Tile2D<EQ, TX, TY>;
   using M = MhTile2D<EQ, TX, TY, NGF>;
   MhMem2D<TC> r;
-  r.m.c0 = r.m.w = reinterpret_cast<TC*>(base);
-  r.m.sl = r.m.w + M::WSZ;
-  r.ls = r.m.sl + T::NS * T::R1;
-  r.wp = r.ls + T::NS * T::NT;
-  r.m.gx = reinterpret_cast<int*>(r.wp + T::NP * T::R1);
+  r.m.rec = reinterpret_cast<TC*>(base);
+  r.m.w = r.m.rec + T::REC * T::R1;
+  r.ls = r.m.w + (M::WSZ + 3) / 4 * 4;
+  r.m.gx = reinterpret_cast<int*>(r.ls + 8 * T::NT);
   r.m.gy = r.m.gx + T::R2X;
   return r;
 }
@@ -177,15 +176,15 @@ __device__ __forceinline__ void mh_rates2d(const Gas<TC>& G, const TC* W, const 
 }
 
 // Predicted primitive state at local point (x, y) of a cell: wp[] its predicted
-// centroid values, g[] its limited primitive gradients (both strided by `st`).
+// centroid values, g[] its limited primitive gradients.
 template <int EQ, class TC>
-__device__ __forceinline__ void mh_eval2d(const TC* wp, const TC* g, int st, TC x, TC y, TC* W) {
+__device__ __forceinline__ void mh_eval2d(const TC* wp, const TC* g, TC x, TC y, TC* W) {
 #pragma unroll
-  for (int q = 0; q < 4; ++q) W[q] = wp[q * st] + g[(2 * q) * st] * x + g[(2 * q + 1) * st] * y;
+  for (int q = 0; q < 4; ++q) W[q] = wp[q] + g[2 * q] * x + g[2 * q + 1] * y;
   if (EQ == 1) {
-    const TC a1 = g[8 * st], a2 = g[9 * st], a3 = g[10 * st];
-    W[4] = wp[4 * st] + a3 * x + a1 * y;
-    W[5] = wp[5 * st] + a2 * x - a3 * y;
+    const TC a1 = g[8], a2 = g[9], a3 = g[10];
+    W[4] = wp[4] + a3 * x + a1 * y;
+    W[5] = wp[5] + a2 * x - a3 * y;
   }
 }
 
@@ -253,9 +252,9 @@ __device__ __forceinline__ void mh2d_compute(const Stage2DArgs<TS>& A, int i0, i
   (void)R2Y;
   (void)R1Y;
   TC* s_w = MM.m.w;
-  TC* s_g = MM.m.sl;  // staged coefficients, then limited primitive gradients
+  constexpr int REC = Tile2D<EQ, TX, TY>::REC;
+  TC* s_rec = MM.m.rec;  // staged coefficients, then predicted values and gradients
   TC* s_ls = MM.ls;
-  TC* s_wp = MM.wp;
   TC* s_fx = MM.m.w;
   TC* s_fy = MM.m.w + NF * NGF * NFX;
   const int* s_gx = MM.m.gx;
@@ -276,7 +275,8 @@ __device__ __forceinline__ void mh2d_compute(const Stage2DArgs<TS>& A, int i0, i
   for (int r1 = tid; r1 < R1; r1 += NT) {
     int ry = r1 / R1X, rx = r1 - ry * R1X;
     int r2 = (ry + 1) * R2X + (rx + 1);
-    TC W[NP], Wn[4][NP], s[NS], g[NS], Wt[NP];
+    TC W[NP], Wn[4][NP], s[NS], rec[REC], Wt[NP];
+    TC* g = rec + NP;
 #pragma unroll
     for (int q = 0; q < NP; ++q) {
       W[q] = s_w[q * R2 + r2];
@@ -285,19 +285,19 @@ __device__ __forceinline__ void mh2d_compute(const Stage2DArgs<TS>& A, int i0, i
       Wn[2][q] = s_w[q * R2 + r2 - R2X];
       Wn[3][q] = s_w[q * R2 + r2 + R2X];
     }
+    vec_get<REC>(s_rec + r1 * REC, rec);
 #pragma unroll
-    for (int k = 0; k < NS; ++k) s[k] = s_g[k * R1 + r1];
+    for (int k = 0; k < NS; ++k) s[k] = g[k];
     mh_grads2d<EQ, TC, WENO>(G, hh, W, Wn, A.limiter, s, g);
     mh_rates2d<EQ, TC>(G, W, g, Wt);
-#pragma unroll
-    for (int k = 0; k < NS; ++k) s_g[k * R1 + r1] = g[k];
     if ((unsigned)(rx - 1) < (unsigned)TX && (unsigned)(ry - 1) < (unsigned)TY) {
       const int t = (ry - 1) * TX + rx - 1;
 #pragma unroll
-      for (int k = 0; k < NS; ++k) s_ls[k * NC + t] = s[k];
+      for (int k = 0; k < 8; ++k) s_ls[k * NC + t] = s[k];
     }
 #pragma unroll
-    for (int q = 0; q < NP; ++q) s_wp[q * R1 + r1] = W[q] + hdt * Wt[q];
+    for (int q = 0; q < NP; ++q) rec[q] = W[q] + hdt * Wt[q];
+    vec_put<REC>(s_rec + r1 * REC, rec);
   }
   __syncthreads();  // the primitives are dead from here: their space takes the fluxes
 
@@ -323,9 +323,11 @@ __device__ __forceinline__ void mh2d_compute(const Stage2DArgs<TS>& A, int i0, i
       TC t = NGF == 2 ? (gp ? ox : -ox) : TC(0);
       yl = hh[1]; yr = -hh[1]; xl = t; xr = t;
     }
-    TC WL[NP], WR[NP], F[NF];
-    mh_eval2d<EQ, TC>(s_wp + r1l, s_g + r1l, R1, xl, yl, WL);
-    mh_eval2d<EQ, TC>(s_wp + r1r, s_g + r1r, R1, xr, yr, WR);
+    TC WL[NP], WR[NP], F[NF], rec[REC];
+    vec_get<REC>(s_rec + r1l * REC, rec);
+    mh_eval2d<EQ, TC>(rec, rec + NP, xl, yl, WL);
+    vec_get<REC>(s_rec + r1r * REC, rec);
+    mh_eval2d<EQ, TC>(rec, rec + NP, xr, yr, WR);
     face_flux_prim2d<EQ, TC>(G, xf ? 0 : 1, WL, WR, F, err);
     if (xf) {
 #pragma unroll
@@ -342,8 +344,9 @@ __device__ __forceinline__ void mh2d_compute(const Stage2DArgs<TS>& A, int i0, i
   if constexpr (SPLIT) {
     const int cell = tid >> 2, qp = tid & 3, cy = cell / TX, cx = cell - cy * TX;
     const int q1 = (cy + 1) * R1X + cx + 1;
-    TC W[NP], Fx[NF], Fy[NF];
-    mh_eval2d<EQ, TC>(s_wp + q1, s_g + q1, R1, (qp & 1) ? ox : -ox, (qp & 2) ? oy : -oy, W);
+    TC W[NP], Fx[NF], Fy[NF], rec[REC];
+    vec_get<REC>(s_rec + q1 * REC, rec);
+    mh_eval2d<EQ, TC>(rec, rec + NP, (qp & 1) ? ox : -ox, (qp & 2) ? oy : -oy, W);
     prim_flux2d<EQ, TC>(G, W, Fx, Fy, err);
 #pragma unroll
     for (int q = 0; q < NF; ++q) {
@@ -375,10 +378,12 @@ __device__ __forceinline__ void mh2d_compute(const Stage2DArgs<TS>& A, int i0, i
 #pragma unroll
     for (int q = 0; q < NF; ++q) { sFx[q] = s_vol[q * NC + tid]; sFy[q] = s_vol[(NF + q) * NC + tid]; }
   } else {
+    TC rec[REC];
+    vec_get<REC>(s_rec + r1 * REC, rec);
 #pragma unroll
     for (int qp = 0; qp < 4; ++qp) {
       TC W[NP], Fx[NF], Fy[NF];
-      mh_eval2d<EQ, TC>(s_wp + r1, s_g + r1, R1, (qp & 1) ? ox : -ox, (qp & 2) ? oy : -oy, W);
+      mh_eval2d<EQ, TC>(rec, rec + NP, (qp & 1) ? ox : -ox, (qp & 2) ? oy : -oy, W);
       prim_flux2d<EQ, TC>(G, W, Fx, Fy, err);
 #pragma unroll
       for (int q = 0; q < NF; ++q) { sFx[q] += Fx[q]; sFy[q] += Fy[q]; }
@@ -424,7 +429,7 @@ __device__ __forceinline__ void mh2d_compute(const Stage2DArgs<TS>& A, int i0, i
 #pragma unroll
   for (int v = 0; v < NV; ++v) o0[v] = fma(dt, Cvt<TC>::to_f64(rc0[v]), (A.in.c0 + v * ncell)[gc]);
 #pragma unroll
-  for (int k = 0; k < NS; ++k) os[k] = s_ls[k * NC + tid] + dtc * rs[k];
+  for (int k = 0; k < NS; ++k) os[k] = (k < 8 ? s_ls[k * NC + tid] : s_rec[r1 * REC + NP + k]) + dtc * rs[k];
   if (owner) {
 #pragma unroll
     for (int v = 0; v < NV; ++v) (A.out.c0 + v * ncell)[gc] = o0[v];

@@ -114,16 +114,6 @@ __device__ __forceinline__ void mh_rates3d(const Gas<TC>& G, const TC* W, const 
   Wt[4] = -(v[0] * g[12] + v[1] * g[13] + v[2] * g[14]) - G.g * p * divv;
 }
 
-// Predicted primitive state of a cell at local point (x, y, z): wp[] its predicted
-// centroid values, g[] its limited primitive gradients (strided by `st`).
-template <class TC>
-__device__ __forceinline__ void mh_eval3d(const TC* wp, const TC* g, int st, TC x, TC y, TC z,
-                                          TC* W) {
-#pragma unroll
-  for (int q = 0; q < 5; ++q)
-    W[q] = wp[q * st] + g[(3 * q) * st] * x + g[(3 * q + 1) * st] * y + g[(3 * q + 2) * st] * z;
-}
-
 // Physical flux along axis d of a primitive state (rho, v, p).
 template <class TC>
 __device__ __forceinline__ void prim_flux3d(const Gas<TC>& G, const TC* W, int d, TC* F,
@@ -188,9 +178,11 @@ __global__ void __launch_bounds__(TX * TY * TZ) mh3d_kernel(const Stage3DArgs<TS
   extern __shared__ __align__(16) unsigned char smem_raw[];
   TC* s_w = reinterpret_cast<TC*>(smem_raw);  // 5 x R2 primitives, then face fluxes
   TC* s_f = s_w;
-  TC* s_wp = s_w + WS;                        // 5 x R1 predicted centroid values
-  TC* s_g = s_wp + 5 * R1;                    // 15 x R1 coefficients -> limited gradients
-  int* s_gx = reinterpret_cast<int*>(s_g + 15 * R1);
+  // R1 records (kRec3d): the staged coefficients, then the predicted centroid values and
+  // the limited gradients, read with 16-byte loads
+  TC* s_rec = s_w + WS;
+  static_assert(WS % 4 == 0, "records are 16-byte aligned");
+  int* s_gx = reinterpret_cast<int*>(s_rec + kRec3d * R1);
   int* s_gy = s_gx + R2X;
   int* s_gz = s_gy + R2Y;
   __shared__ double s_dt;
@@ -217,7 +209,7 @@ __global__ void __launch_bounds__(TX * TY * TZ) mh3d_kernel(const Stage3DArgs<TS
   }
 
   // ---- 1. primitives of the halo-2 box; coefficients of the halo-1 box
-  stage3d_issue<5, 15, TX, TY, TZ, TS, TC, 0, 0, false>(A.in, ncell, s_gx, s_gy, s_gz, s_g);
+    stage3d_issue<15, TX, TY, TZ, TS, TC, kRec3d, 5>(A.in, ncell, s_gx, s_gy, s_gz, s_rec);
   for (int r = tid; r < R2; r += NT) {
     int rz = r / (R2X * R2Y), rr = r - rz * (R2X * R2Y);
     int ry = rr / R2X, rx = rr - ry * R2X;
@@ -240,9 +232,10 @@ __global__ void __launch_bounds__(TX * TY * TZ) mh3d_kernel(const Stage3DArgs<TS
   const TC oo[3] = {geo.oo[0], geo.oo[1], geo.oo[2]};
 
   // ---- 2. gradients, limiter, half-step prediction on the halo-1 box
-  for (int r1 = tid; r1 < R1; r1 += NT) {
-    int rz = r1 / (R1X * R1Y), rr = r1 - rz * (R1X * R1Y);
-    int ry = rr / R1X, rx = rr - ry * R1X;
+  for (int e = tid; e < ring3d_count<TX, TY, TZ>(); e += NT) {
+    int rx, ry, rz;
+    ring3d_cell<TX, TY, TZ>(e, rx, ry, rz);
+    const int r1 = (rz * R1Y + ry) * R1X + rx;
     int r2 = ((rz + 1) * R2Y + (ry + 1)) * R2X + (rx + 1);
     TC W[5], Wn[6][5], s[15], g[15], Wt[5];
 #pragma unroll
@@ -255,14 +248,19 @@ __global__ void __launch_bounds__(TX * TY * TZ) mh3d_kernel(const Stage3DArgs<TS
       Wn[4][q] = s_w[q * R2 + r2 - R2X * R2Y];
       Wn[5][q] = s_w[q * R2 + r2 + R2X * R2Y];
     }
+    {
+      TC v[kRec3d];
+      rec_get<TC>(s_rec + r1 * kRec3d, v);
 #pragma unroll
-    for (int k = 0; k < 15; ++k) s[k] = s_g[k * R1 + r1];
-    mh_grads3d<TC, WENO>(G, hh, W, Wn, A.limiter, s, g);
-    mh_rates3d<TC>(G, W, g, Wt);
+      for (int k = 0; k < 15; ++k) s[k] = v[5 + k];
+      mh_grads3d<TC, WENO>(G, hh, W, Wn, A.limiter, s, g);
+      mh_rates3d<TC>(G, W, g, Wt);
 #pragma unroll
-    for (int k = 0; k < 15; ++k) s_g[k * R1 + r1] = g[k];
+      for (int q = 0; q < 5; ++q) v[q] = W[q] + hdt * Wt[q];
 #pragma unroll
-    for (int q = 0; q < 5; ++q) s_wp[q * R1 + r1] = W[q] + hdt * Wt[q];
+      for (int k = 0; k < 15; ++k) v[5 + k] = g[k];
+      rec_put<TC>(s_rec + r1 * kRec3d, v);
+    }
   }
   __syncthreads();  // the primitives are dead from here: their space takes the fluxes
 
@@ -273,6 +271,8 @@ __global__ void __launch_bounds__(TX * TY * TZ) mh3d_kernel(const Stage3DArgs<TS
 #pragma unroll
   for (int v = 0; v < 5; ++v) rc0[v] = TC(0);
   {
+    TC vc[kRec3d];
+    rec_get<TC>(s_rec + r1c * kRec3d, vc);
     TC sF[3][5];
 #pragma unroll
     for (int d = 0; d < 3; ++d)
@@ -281,8 +281,7 @@ __global__ void __launch_bounds__(TX * TY * TZ) mh3d_kernel(const Stage3DArgs<TS
 #pragma unroll
     for (int qp = 0; qp < 8; ++qp) {
       TC W[5];
-      mh_eval3d<TC>(s_wp + r1c, s_g + r1c, R1, (qp & 1) ? oo[0] : -oo[0],
-                    (qp & 2) ? oo[1] : -oo[1], (qp & 4) ? oo[2] : -oo[2], W);
+      eval3d<TC>(vc, vc + 5, (qp & 1) ? oo[0] : -oo[0], (qp & 2) ? oo[1] : -oo[1], (qp & 4) ? oo[2] : -oo[2], W);
 #pragma unroll
       for (int d = 0; d < 3; ++d) {
         TC F[5];
@@ -318,8 +317,13 @@ __global__ void __launch_bounds__(TX * TY * TZ) mh3d_kernel(const Stage3DArgs<TS
       const TC yl = d == 1 ? hn : (d == 0 ? a : b), yr = d == 1 ? -hn : (d == 0 ? a : b);
       const TC zl = d == 2 ? hn : b, zr = d == 2 ? -hn : b;
       TC WL[5], WR[5], F[5];
-      mh_eval3d<TC>(s_wp + r1l, s_g + r1l, R1, xl, yl, zl, WL);
-      mh_eval3d<TC>(s_wp + r1r, s_g + r1r, R1, xr, yr, zr, WR);
+      {
+        TC v[kRec3d];
+        rec_get<TC>(s_rec + r1l * kRec3d, v);
+        eval3d<TC>(v, v + 5, xl, yl, zl, WL);
+        rec_get<TC>(s_rec + r1r * kRec3d, v);
+        eval3d<TC>(v, v + 5, xr, yr, zr, WR);
+      }
       face_flux_prim3d<d, TC>(G, WL, WR, F, err);
 #pragma unroll
       for (int v = 0; v < 5; ++v) s_f[(v * FMAX + f) * NPT + g] = F[v];
@@ -351,7 +355,7 @@ __global__ void __launch_bounds__(TX * TY * TZ) mh3d_kernel(const Stage3DArgs<TS
     for (int v = 0; v < 5; ++v) c[v] = Cvt<TC>::to_tc((A.in.c0 + v * ncell)[gc]);
     prims3d<TC>(G, c, W, err);
 #pragma unroll
-    for (int k = 0; k < 15; ++k) g[k] = s_g[k * R1 + r1c];
+    for (int k = 0; k < 15; ++k) g[k] = s_rec[r1c * kRec3d + 5 + k];
     mh_cons3d<TC>(G, W, g, sn);
   } else {
 #pragma unroll

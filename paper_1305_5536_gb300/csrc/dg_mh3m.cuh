@@ -198,7 +198,7 @@ __global__ void __launch_bounds__(TX * TY * TZ) mh3m_kernel(const Stage3DArgs<TS
   }
 
   // ---- 1. primitives of the halo-2 box; coefficients of the halo-1 box
-  stage3d_issue<8, 23, TX, TY, TZ>(A.in, ncell, s_gx, s_gy, s_gz, s_g);
+  stage3d_issue<23, TX, TY, TZ>(A.in, ncell, s_gx, s_gy, s_gz, s_g);
   for (int r = tid; r < R2; r += NT) {
     int rz = r / (R2X * R2Y), rr = r - rz * (R2X * R2Y);
     int ry = rr / R2X, rx = rr - ry * R2X;

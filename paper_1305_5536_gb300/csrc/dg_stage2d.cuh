@@ -43,7 +43,9 @@ template <> struct Tr2<1> {  // planar MHD: (rho, mx, my, E, b1, b2) + (.., a1, 
 };
 
 // Shared-memory working set of one tile (element counts of the arithmetic type
-// TC): averages [NV][R2], derivative coefficients [NS][R1], and one region that
+// TC): a record of REC elements per cell of the halo-1 region (averages, then derivative
+// coefficients; 16-byte aligned, read with vector loads: at strides of 12 and 20 words
+// the 8 threads of each phase of a 16-byte load hit disjoint banks), and one region that
 // first holds the centroid primitives [NP][R2] and, once the limiter is done with
 // them, the face fluxes [NF][(TX+1)TY][2] and [NF][TX(TY+1)][2].
 template <int EQ, int TX, int TY>
@@ -55,8 +57,38 @@ struct Tile2D {
   static constexpr int NFX = (TX + 1) * TY, NFY = TX * (TY + 1);
   static constexpr int NT = TX * TY;
   static constexpr int WSZ = NP * R2 > NF * 2 * (NFX + NFY) ? NP * R2 : NF * 2 * (NFX + NFY);
-  static constexpr int ELEMS = NV * R2 + NS * R1 + WSZ;
+  static constexpr int REC = (NV + NS + 3) / 4 * 4;
+  static constexpr int ELEMS = REC * R1 + WSZ;
 };
+
+// The N elements of a record.
+template <int N, class TC>
+__device__ __forceinline__ void vec_get(const TC* rec, TC* v) {
+  if constexpr (sizeof(TC) == 4) {
+#pragma unroll
+    for (int i = 0; i < N / 4; ++i) {
+      const float4 q = reinterpret_cast<const float4*>(rec)[i];
+      v[4 * i] = q.x; v[4 * i + 1] = q.y; v[4 * i + 2] = q.z; v[4 * i + 3] = q.w;
+    }
+  } else {
+#pragma unroll
+    for (int i = 0; i < N / 2; ++i) {
+      const double2 q = reinterpret_cast<const double2*>(rec)[i];
+      v[2 * i] = q.x; v[2 * i + 1] = q.y;
+    }
+  }
+}
+template <int N, class TC>
+__device__ __forceinline__ void vec_put(TC* rec, const TC* v) {
+  if constexpr (sizeof(TC) == 4) {
+#pragma unroll
+    for (int i = 0; i < N / 4; ++i)
+      reinterpret_cast<float4*>(rec)[i] = make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
+  } else {
+#pragma unroll
+    for (int i = 0; i < N / 2; ++i) reinterpret_cast<double2*>(rec)[i] = make_double2(v[2 * i], v[2 * i + 1]);
+  }
+}
 
 // NT = 4 TX TY (four threads per cell): also the volume sums [2 NF][TX TY].
 template <int EQ, int TX, int TY, class TC, int NT = TX * TY>
@@ -68,9 +100,8 @@ __host__ __device__ constexpr size_t stage2d_smem_bytes() {
 
 template <class TC>
 struct TileMem {
-  TC* c0;
-  TC* sl;
-  TC* w;  // primitives, then face fluxes
+  TC* rec;  // records of the halo-1 cells
+  TC* w;    // primitives, then face fluxes
   int* gx;
   int* gy;
 };
@@ -79,9 +110,8 @@ template <int EQ, int TX, int TY, class TC>
 __device__ __forceinline__ TileMem<TC> tile_mem(unsigned char* base) {
   using T = Tile2D<EQ, TX, TY>;
   TileMem<TC> m;
-  m.c0 = reinterpret_cast<TC*>(base);
-  m.sl = m.c0 + T::NV * T::R2;
-  m.w = m.sl + T::NS * T::R1;
+  m.rec = reinterpret_cast<TC*>(base);
+  m.w = m.rec + T::REC * T::R1;
   m.gx = reinterpret_cast<int*>(m.w + T::WSZ);
   m.gy = m.gx + T::R2X;
   return m;
@@ -289,10 +319,10 @@ __device__ __forceinline__ void stage2d_load(const Stage2DArgs<TS>& A, const Til
       const int ry = r / T::R2X, rx = r - ry * T::R2X;
       const unsigned g = (unsigned)(M.gy[ry] + M.gx[rx]);
       if ((unsigned)(rx - 1) < (unsigned)T::R1X && (unsigned)(ry - 1) < (unsigned)T::R1Y) {
-        TC* dst = M.sl + (ry - 1) * T::R1X + rx - 1;
+        TC* dst = M.rec + ((ry - 1) * T::R1X + rx - 1) * T::REC + T::NV;
 #pragma unroll
         for (int k = 0; k < T::NS; ++k)
-          cp_async_elem<sizeof(TS)>(dst + k * T::R1, A.in.sl + k * ncell + g);
+          cp_async_elem<sizeof(TS)>(dst + k, A.in.sl + k * ncell + g);
       }
 #pragma unroll
       for (int v = 0; v < T::NV; ++v) a[i][v] = __ldg(A.in.c0 + v * ncell + g);
@@ -306,31 +336,19 @@ __device__ __forceinline__ void stage2d_load(const Stage2DArgs<TS>& A, const Til
 #pragma unroll
       for (int v = 0; v < T::NV; ++v) c[v] = Cvt<TC>::to_tc(a[i][v]);
       prims2d<EQ, TC>(G, c, W, err);
+      if (C0) {
+        const int ry = r / T::R2X, rx = r - ry * T::R2X;
+        if ((unsigned)(rx - 1) < (unsigned)T::R1X && (unsigned)(ry - 1) < (unsigned)T::R1Y) {
+          TC* dst = M.rec + ((ry - 1) * T::R1X + rx - 1) * T::REC;
 #pragma unroll
-      for (int v = 0; v < T::NV; ++v)
-        if (C0) M.c0[v * T::R2 + r] = c[v];
+          for (int v = 0; v < T::NV; ++v) dst[v] = c[v];
+        }
+      }
 #pragma unroll
       for (int q = 0; q < T::NP; ++q) M.w[q * T::R2 + r] = W[q];
     }
   }
   cp_async_wait_all();
-}
-
-// Stage 2 reads the step's input state U^n of its own cell only at the end (the
-// Runge-Kutta combination): request those lines into L2 while the tile stages.
-template <int EQ, class TC, class TS, int TX, int TY>
-__device__ __forceinline__ void stage2d_prefetch_base(const Stage2DArgs<TS>& A,
-                                                      const TileMem<TC>& M) {
-  using T = Tile2D<EQ, TX, TY>;
-  const size_t ncell = (size_t)A.ncell;
-  if (threadIdx.x >= T::NT) return;
-  const int lx = threadIdx.x % TX, ly = threadIdx.x / TX;
-  const unsigned gc = (unsigned)(M.gy[ly + 2] + M.gx[lx + 2]);
-  const TS* sl = A.limiter && A.lim_sl ? A.lim_sl : A.base.sl;
-#pragma unroll
-  for (int v = 0; v < T::NV; ++v) prefetch_l2(&(A.base.c0 + v * ncell)[gc]);
-#pragma unroll
-  for (int k = 0; k < T::NS; ++k) prefetch_l2(&(sl + k * ncell)[gc]);
 }
 
 // End of a step on one tile: the Courant signal speed of the new averages o0[]
@@ -418,9 +436,9 @@ __device__ __forceinline__ void stage2d_compute(const Stage2DArgs<TS>& A, int i0
   static_assert(NC % 32 == 0 && NT % 32 == 0 && NT >= NC, "tile must be whole warps");
   (void)R2Y;
   (void)R1Y;
-  TC* s_c0 = M.c0;
+  constexpr int REC = Tile2D<EQ, TX, TY>::REC;
+  TC* s_rec = M.rec;
   TC* s_w = M.w;
-  TC* s_sl = M.sl;
   TC* s_fx = M.w;
   TC* s_fy = M.w + NF * 2 * NFX;
   const int* s_gx = M.gx;
@@ -440,7 +458,8 @@ __device__ __forceinline__ void stage2d_compute(const Stage2DArgs<TS>& A, int i0
     for (int r1 = tid; r1 < R1; r1 += NT) {
       int ry = r1 / R1X, rx = r1 - ry * R1X;
       int r2 = (ry + 1) * R2X + (rx + 1);
-      TC W[NP], Wn[4][NP], s[NS];
+      TC W[NP], Wn[4][NP], rec[REC];
+      TC* s = rec + NV;
 #pragma unroll
       for (int q = 0; q < NP; ++q) {
         W[q] = s_w[q * R2 + r2];
@@ -449,12 +468,10 @@ __device__ __forceinline__ void stage2d_compute(const Stage2DArgs<TS>& A, int i0
         Wn[2][q] = s_w[q * R2 + r2 - R2X];
         Wn[3][q] = s_w[q * R2 + r2 + R2X];
       }
-#pragma unroll
-      for (int k = 0; k < NS; ++k) s[k] = s_sl[k * R1 + r1];
+      vec_get<REC>(s_rec + r1 * REC, rec);
       if (WENO && A.limiter == 2) weno_cell2d<EQ, TC>(G, hh, W, Wn, s, nullptr);
       else limit_cell2d<EQ, TC>(G, hh, W, Wn, s);
-#pragma unroll
-      for (int k = 0; k < NS; ++k) s_sl[k * R1 + r1] = s[k];
+      vec_put<REC>(s_rec + r1 * REC, rec);
     }
   }
   __syncthreads();  // the primitives are dead from here: their space takes the fluxes
@@ -476,16 +493,12 @@ __device__ __forceinline__ void stage2d_compute(const Stage2DArgs<TS>& A, int i0
       const int fy = f / W1, fx = f - fy * W1;
       const int r1l = d == 0 ? (fy + 1) * R1X + fx : fy * R1X + fx + 1;
       const int r1r = r1l + (d == 0 ? 1 : R1X);
-      const int r2l = d == 0 ? (fy + 2) * R2X + fx + 1 : (fy + 1) * R2X + fx + 2;
-      const int r2r = r2l + (d == 0 ? 1 : R2X);
       const TC t = d == 0 ? (g ? oy : -oy) : (g ? ox : -ox);
-      TC c0l[NV], c0r[NV], sl[NS], sr[NS], cl[NV], cr[NV], F[NF];
-#pragma unroll
-      for (int v = 0; v < NV; ++v) { c0l[v] = s_c0[v * R2 + r2l]; c0r[v] = s_c0[v * R2 + r2r]; }
-#pragma unroll
-      for (int k = 0; k < NS; ++k) { sl[k] = s_sl[k * R1 + r1l]; sr[k] = s_sl[k * R1 + r1r]; }
-      eval2d<EQ, TC>(c0l, sl, d == 0 ? hh[0] : t, d == 0 ? t : hh[1], cl);
-      eval2d<EQ, TC>(c0r, sr, d == 0 ? -hh[0] : t, d == 0 ? t : -hh[1], cr);
+      TC cl[NV], cr[NV], F[NF], rec[REC];
+      vec_get<REC>(s_rec + r1l * REC, rec);
+      eval2d<EQ, TC>(rec, rec + NV, d == 0 ? hh[0] : t, d == 0 ? t : hh[1], cl);
+      vec_get<REC>(s_rec + r1r * REC, rec);
+      eval2d<EQ, TC>(rec, rec + NV, d == 0 ? -hh[0] : t, d == 0 ? t : -hh[1], cr);
       face_flux2d<EQ, TC>(G, d, cl, cr, F, err);
 #pragma unroll
       for (int q = 0; q < NF; ++q) s_f[(q * NF1 + f) * 2 + g] = F[q];
@@ -499,13 +512,10 @@ __device__ __forceinline__ void stage2d_compute(const Stage2DArgs<TS>& A, int i0
   static_assert(!SPLIT || (R2X + R2Y) % 2 == 0, "FP64 sums behind the offset tables");
   if constexpr (SPLIT) {
     const int cell = tid >> 2, qp = tid & 3, cy = cell / TX, cx = cell - cy * TX;
-    const int q2 = (cy + 2) * R2X + cx + 2, q1 = (cy + 1) * R1X + cx + 1;
-    TC a0[NV], s[NS], c[NV], Fx[NF], Fy[NF];
-#pragma unroll
-    for (int v = 0; v < NV; ++v) a0[v] = s_c0[v * R2 + q2];
-#pragma unroll
-    for (int k = 0; k < NS; ++k) s[k] = s_sl[k * R1 + q1];
-    eval2d<EQ, TC>(a0, s, (qp & 1) ? ox : -ox, (qp & 2) ? oy : -oy, c);
+    const int q1 = (cy + 1) * R1X + cx + 1;
+    TC rec[REC], c[NV], Fx[NF], Fy[NF];
+    vec_get<REC>(s_rec + q1 * REC, rec);
+    eval2d<EQ, TC>(rec, rec + NV, (qp & 1) ? ox : -ox, (qp & 2) ? oy : -oy, c);
     phys_flux2d<EQ, TC>(G, c, Fx, Fy, err);
 #pragma unroll
     for (int q = 0; q < NF; ++q) {
@@ -528,15 +538,13 @@ __device__ __forceinline__ void stage2d_compute(const Stage2DArgs<TS>& A, int i0
   const bool owner = mine && gi < nx && gj < ny;
   double o0[NV];
   if (mine) {
-  const int r2 = (ly + 2) * R2X + lx + 2, r1 = (ly + 1) * R1X + lx + 1;
+  const int r1 = (ly + 1) * R1X + lx + 1;
   const unsigned gc = (unsigned)(s_gy[ly + 2] + s_gx[lx + 2]);
   const TC dtc = Cvt<TC>::to_tc(S.dt);
   const double dt = S.dt;
-  TC c0[NV], s[NS];
-#pragma unroll
-  for (int v = 0; v < NV; ++v) c0[v] = s_c0[v * R2 + r2];
-#pragma unroll
-  for (int k = 0; k < NS; ++k) s[k] = s_sl[k * R1 + r1];
+  TC rec[REC];
+  vec_get<REC>(s_rec + r1 * REC, rec);
+  const TC *c0 = rec, *s = rec + NV;
 
   TC sFx[NF], sFy[NF];
 #pragma unroll
@@ -664,7 +672,6 @@ __device__ __forceinline__ void stage2d_tile(const Stage2DArgs<TS>& A, int i0, i
   __syncthreads();
   griddep_wait();
   stage2d_take_dt(A, S);
-  if (STAGE == 2) stage2d_prefetch_base<EQ, TC, TS, TX, TY>(A, M);
   unsigned err = 0;
   stage2d_load<EQ, TC, TS, TX, TY, NT>(A, M, gas_of<TC>(A.gas), err);
   __syncthreads();

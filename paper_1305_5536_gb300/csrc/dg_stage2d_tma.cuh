@@ -99,7 +99,13 @@ __global__ void __launch_bounds__(TX * TY)
       for (int r = tid; r < T::R2; r += T::NT) {
         TC c[T::NV], W[T::NP];
 #pragma unroll
-        for (int v = 0; v < T::NV; ++v) M.c0[v * T::R2 + r] = c[v] = Cvt<TC>::to_tc(raw_c0[v * T::R2 + r]);
+        for (int v = 0; v < T::NV; ++v) c[v] = Cvt<TC>::to_tc(raw_c0[v * T::R2 + r]);
+        const int ry = r / T::R2X, rx = r - ry * T::R2X;
+        if ((unsigned)(rx - 1) < (unsigned)T::R1X && (unsigned)(ry - 1) < (unsigned)T::R1Y) {
+          TC* dst = M.rec + ((ry - 1) * T::R1X + rx - 1) * T::REC;
+#pragma unroll
+          for (int v = 0; v < T::NV; ++v) dst[v] = c[v];
+        }
         prims2d<EQ, TC>(gas_of<TC>(A.gas), c, W, err);
 #pragma unroll
         for (int q = 0; q < T::NP; ++q) M.w[q * T::R2 + r] = W[q];
@@ -107,7 +113,7 @@ __global__ void __launch_bounds__(TX * TY)
       for (int e = tid; e < T::NS * T::R1; e += T::NT) {
         const int v = e / T::R1, r = e - v * T::R1;
         const int ry = r / T::R1X, rx = r - ry * T::R1X;
-        M.sl[e] = (TC)raw_sl[(v * T::R1Y + ry) * B::SXW + rx + B::SOFF];
+        M.rec[r * T::REC + T::NV + v] = (TC)raw_sl[(v * T::R1Y + ry) * B::SXW + rx + B::SOFF];
       }
     } else {
       stage2d_load<EQ, TC, TS, TX, TY, T::NT>(A, M, gas_of<TC>(A.gas), err);

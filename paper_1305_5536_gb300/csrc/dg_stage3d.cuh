@@ -212,28 +212,20 @@ __device__ __forceinline__ void gather3d(const TC* s_f, int FMAX, int fm, int fp
   }
 }
 
-// Start of the staging of a 3D tile: the NS derivative coefficients of the
-// halo-1 box are copied with cp.async (in flight while the averages are read),
-// and every average of the halo-2 box that this thread reads next is requested
-// into L2, so that the DRAM latencies of the staging overlap.  The caller then
-// reads the averages, calls cp_async_wait_all() and synchronises.
+// Start of the staging of a 3D tile: the NS derivative coefficients of the halo-1 box are
+// copied with cp.async, in flight while the caller reads the averages; it then calls
+// cp_async_wait_all() and synchronises.  A thread takes whole cells, so that a cell's
+// offset is formed once for its coefficients (walking planes cost a dozen instructions a
+// copy: 3D Euler 128^3 1188 -> 1115 us a step).
 // REC > 0: the coefficients go into per-cell records of REC elements, coefficient
 // k of halo-1 cell r1 at s_sl[r1 * REC + OFF + k]; else planes s_sl[k * R1 + r1].
-// PREFETCH = false leaves out the L2 requests for the averages (the 3D Euler
-// kernel, which reads them two cells at a time, measured 1 % faster without);
-// HALO = true requests only the cells of halo3d_cell, the ones a kernel whose
-// limiter covers the tile and its face slabs reads.
-template <int NV, int NS, int TX, int TY, int TZ, class TS, class TC, int REC = 0, int OFF = 0,
-          bool PREFETCH = true, bool HALO = false>
+template <int NS, int TX, int TY, int TZ, class TS, class TC, int REC = 0, int OFF = 0>
 __device__ __forceinline__ void stage3d_issue(const StateBuf<TS>& in, size_t ncell,
                                               const int* s_gx, const int* s_gy, const int* s_gz,
                                               TC* s_sl) {
-  constexpr int R2X = TX + 4, R2Y = TY + 4, R2 = R2X * R2Y * (TZ + 4);
-  constexpr int R1X = TX + 2, R1Y = TY + 2;
+  constexpr int R1X = TX + 2, R1Y = TY + 2, R1 = R1X * R1Y * (TZ + 2);
   constexpr int NT = TX * TY * TZ;
   static_assert(sizeof(TS) == sizeof(TC), "derivative coefficients are staged as stored");
-  // whole cells of the box: a cell's offset once for its NS coefficients
-  constexpr int R1 = R1X * R1Y * (TZ + 2);
   for (int r = threadIdx.x; r < R1; r += NT) {
     const int rz = r / (R1X * R1Y), rr = r - rz * (R1X * R1Y);
     const int ry = rr / R1X, rx = rr - ry * R1X;
@@ -242,22 +234,6 @@ __device__ __forceinline__ void stage3d_issue(const StateBuf<TS>& in, size_t nce
 #pragma unroll
     for (int k = 0; k < NS; ++k)
       cp_async_elem<sizeof(TS)>(dst + k * (REC > 0 ? 1 : R1), in.sl + k * ncell + g);
-  }
-  if (PREFETCH) {
-    for (int r = threadIdx.x; r < (HALO ? halo3d_count<TX, TY, TZ>() : R2); r += NT) {
-      int rx, ry, rz;
-      if (HALO) {
-        halo3d_cell<TX, TY, TZ>(r, rx, ry, rz);
-      } else {
-        rz = r / (R2X * R2Y);
-        const int rr = r - rz * (R2X * R2Y);
-        ry = rr / R2X;
-        rx = rr - ry * R2X;
-      }
-      const const unsigned g = (unsigned)(s_gz[rz] + s_gy[ry] + s_gx[rx]);
-#pragma unroll
-      for (int v = 0; v < NV; ++v) prefetch_l2(&(in.c0 + v * ncell)[g]);
-    }
   }
 }
 
@@ -332,7 +308,7 @@ __global__ void __launch_bounds__(TX * TY * TZ, (Stage3dMinBlocks<TX * TY * TZ, 
 
   // ---- primitives where the limiter reads them; averages of the halo-1 box
   if (STAGE == 2) stage3d_prefetch_base<5, 15, TX, TY>(A, ncell, s_gx, s_gy, s_gz);
-  stage3d_issue<5, 15, TX, TY, TZ, TS, TC, kRec3d, 5, false>(A.in, ncell, s_gx, s_gy, s_gz, s_rec);
+  stage3d_issue<15, TX, TY, TZ, TS, TC, kRec3d, 5>(A.in, ncell, s_gx, s_gy, s_gz, s_rec);
   // the halo-2 cells the limiter reads (the halo-1 box and the six outer face
   // layers), two per pass, all ten FP64 loads in flight before the first is
   // converted (the second cell of the last pass re-reads the first if it is past

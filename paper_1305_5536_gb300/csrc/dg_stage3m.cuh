@@ -361,7 +361,7 @@ __global__ void __launch_bounds__(TX * TY * TZ, (Stage3mMinBlocks<TX * TY * TZ, 
 
   // ---- primitives where the limiter reads them; averages of the halo-1 box
   if (STAGE == 2) stage3d_prefetch_base<8, 23, TX, TY>(A, ncell, s_gx, s_gy, s_gz);
-  stage3d_issue<8, 23, TX, TY, TZ, TS, TC, 0, 0, true, true>(A.in, ncell, s_gx, s_gy, s_gz, s_sl);
+  stage3d_issue<23, TX, TY, TZ>(A.in, ncell, s_gx, s_gy, s_gz, s_sl);
   // the halo-2 cells the limiter reads: the halo-1 box, then the six outer face
   // layers (e < R1 is the cell's halo-1 index)
 #pragma unroll 1

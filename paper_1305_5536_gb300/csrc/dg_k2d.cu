@@ -134,6 +134,8 @@ static cudaError_t launch2d_tma(int stage, const Stage2DArgs<TS>& a, cudaStream_
 // FP64 variants 5 and 6 are small tiles with four threads per cell: a grid of a few
 // thousand cells then covers every SM, and the four FP64 pipes of each share a tile's
 // faces and volume points (one warp keeps one pipe busy for 64 cycles an instruction).
+// us a step, 8x8 with one thread per cell / 8x4 and 8x8 with four: 32^2 123 / 65 / 81,
+// 64^2 122 / 72 / 80, 96^2 124 / 102 / 90, 128^2 136 / 153 / 140; the tuner picks.
 int stage2d_variants(int, int fp32) { return fp32 ? 5 : 7; }
 
 const char* stage2d_variant_name(int, int fp32, int v) {

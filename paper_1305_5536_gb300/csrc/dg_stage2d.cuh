@@ -1,10 +1,10 @@
 // dg_stage2d.cuh -- one SSP-RK2 stage of the 2D P1 DG scheme (Euler or planar
 // ideal MHD) as a single fused kernel.
 //
-// One CTA owns a TX x TY tile of cells.  It stages in shared memory the cell
-// averages of the tile plus a halo of 2 cells and the derivative coefficients of
-// the tile plus a halo of 1 cell (periodic wrap), then
-//   1. centroid primitives of every staged cell,
+// One CTA owns a TX x TY tile of cells.  It stages in shared memory, as records, the cell
+// averages and derivative coefficients of the tile plus a halo of 1 cell (periodic wrap),
+// then
+//   1. (while staging) centroid primitives of the tile plus a halo of 2 cells,
 //   2. the min/max limiter (Sec. 2.5) of the tile and its 1-cell ring, in place,
 //   3. every face of the tile once: the two one-sided polynomials at the 2 Gauss
 //      points, the Riemann flux (exact solver, or HLLD with the averaged normal
@@ -47,7 +47,8 @@ template <> struct Tr2<1> {  // planar MHD: (rho, mx, my, E, b1, b2) + (.., a1, 
 // coefficients; 16-byte aligned, read with vector loads: at strides of 12 and 20 words
 // the 8 threads of each phase of a 16-byte load hit disjoint banks), and one region that
 // first holds the centroid primitives [NP][R2] and, once the limiter is done with
-// them, the face fluxes [NF][(TX+1)TY][2] and [NF][TX(TY+1)][2].
+// them, the face fluxes [NF][(TX+1)TY][2] and [NF][TX(TY+1)][2].  (Planes instead of
+// records, 34 scalar loads a face point: 62.7 against 60.3 us a step at 512^2.)
 template <int EQ, int TX, int TY>
 struct Tile2D {
   using Tr = Tr2<EQ>;
@@ -254,7 +255,7 @@ __device__ __forceinline__ void face_flux2d(const Gas<TC>& G, int dir, const TC*
   }
   TC pl = G.gm1 * (cl[3] - TC(0.5) * (cl[1] * vxl + cl[2] * vyl) - magl);
   TC pr = G.gm1 * (cr[3] - TC(0.5) * (cr[1] * vxr + cr[2] * vyr) - magr);
-  // the face frame's normal and transverse components (dir is a constant at the callers)
+  // the face frame's normal and transverse components
   const bool xd = dir == 0;
   const TC unl = xd ? vxl : vyl, utl = xd ? vyl : vxl;
   const TC unr = xd ? vxr : vyr, utr = xd ? vyr : vxr;
@@ -301,7 +302,9 @@ __device__ __forceinline__ void stage2d_take_dt(const Stage2DArgs<TS>& A, TileSc
 // thread takes whole cells of the halo-2 region, so that a cell's offset is formed once
 // for its averages and (inside the halo-1 region) its derivative coefficients.  The
 // coefficients are copied with cp.async and the averages of all of a thread's cells are
-// loaded before the first is converted, so that their DRAM latencies overlap.  C0: the
+// loaded before the first is converted, so that their DRAM latencies overlap.  (Walking
+// rows element by element and forming the primitives in a pass of their own: 2D MHD 512^2
+// FP32 68.4 against 62.7 us a step.)  C0: the
 // averages are kept beside the primitives (the MUSCL-Hancock kernel needs only the
 // latter).  The caller synchronises.
 template <int EQ, class TC, class TS, int TX, int TY, int NT, bool C0 = true>
@@ -479,33 +482,57 @@ __device__ __forceinline__ void stage2d_compute(const Stage2DArgs<TS>& A, int i0
 
   // ---- faces: Riemann fluxes at the Gauss points, each face once
   const TC ox = geo.ox, oy = geo.oy;
-  // One loop per orientation with its own copy of the solver: no selects between the
-  // two (2D MHD 512^2 FP32: 70.5 -> 68.4 us a step).
-  auto faces = [&](auto dc) {
-    constexpr int d = dc;
-    constexpr int NF1 = d == 0 ? NFX : NFY;
-    TC* s_f = d == 0 ? s_fx : s_fy;
-    // the y faces start with the threads that had fewest x faces
-    const int t0 = d == 0 ? tid : (tid >= NT / 2 ? tid - NT / 2 : tid + NT / 2);
-    for (int e = t0; e < 2 * NF1; e += NT) {
-      constexpr int W1 = d == 0 ? TX + 1 : TX;
-      const int f = e >> 1, g = e & 1;
-      const int fy = f / W1, fx = f - fy * W1;
-      const int r1l = d == 0 ? (fy + 1) * R1X + fx : fy * R1X + fx + 1;
-      const int r1r = r1l + (d == 0 ? 1 : R1X);
-      const TC t = d == 0 ? (g ? oy : -oy) : (g ? ox : -ox);
+  // FP64: one loop over the faces of both orientations, so that the points divide evenly
+  // among the warps (each keeps an FP64 pipe busy; us a step, one loop against two: 2D
+  // Euler 256^2 412 / 463, 2D MHD 256^2 436 / 460, 512^2 1437 / 1428).
+  if constexpr (sizeof(TC) == 8) {
+    for (int e = tid; e < 2 * (NFX + NFY); e += NT) {
+      const bool xf = e < 2 * NFX;
+      const int ee = xf ? e : e - 2 * NFX, f = ee >> 1, g = ee & 1;
+      const int fy = xf ? f / (TX + 1) : f / TX, fx = f - fy * (xf ? TX + 1 : TX);
+      const int r1l = xf ? (fy + 1) * R1X + fx : fy * R1X + fx + 1;
+      const int r1r = r1l + (xf ? 1 : R1X);
+      const TC t = xf ? (g ? oy : -oy) : (g ? ox : -ox);
       TC cl[NV], cr[NV], F[NF], rec[REC];
       vec_get<REC>(s_rec + r1l * REC, rec);
-      eval2d<EQ, TC>(rec, rec + NV, d == 0 ? hh[0] : t, d == 0 ? t : hh[1], cl);
+      eval2d<EQ, TC>(rec, rec + NV, xf ? hh[0] : t, xf ? t : hh[1], cl);
       vec_get<REC>(s_rec + r1r * REC, rec);
-      eval2d<EQ, TC>(rec, rec + NV, d == 0 ? -hh[0] : t, d == 0 ? t : -hh[1], cr);
-      face_flux2d<EQ, TC>(G, d, cl, cr, F, err);
+      eval2d<EQ, TC>(rec, rec + NV, xf ? -hh[0] : t, xf ? t : -hh[1], cr);
+      face_flux2d<EQ, TC>(G, xf ? 0 : 1, cl, cr, F, err);
+      TC* s_f = xf ? s_fx : s_fy;
+      const int NF1 = xf ? NFX : NFY;
 #pragma unroll
       for (int q = 0; q < NF; ++q) s_f[(q * NF1 + f) * 2 + g] = F[q];
     }
-  };
-  faces(std::integral_constant<int, 0>{});
-  faces(std::integral_constant<int, 1>{});
+  } else {
+    // FP32: one loop per orientation with its own copy of the solver: no selects between the
+    // two (2D MHD 512^2: 70.5 -> 68.4 us a step).
+    auto faces = [&](auto dc) {
+      constexpr int d = dc;
+      constexpr int NF1 = d == 0 ? NFX : NFY;
+      TC* s_f = d == 0 ? s_fx : s_fy;
+      // the y faces start with the threads that had fewest x faces
+      const int t0 = d == 0 ? tid : (tid >= NT / 2 ? tid - NT / 2 : tid + NT / 2);
+      for (int e = t0; e < 2 * NF1; e += NT) {
+        constexpr int W1 = d == 0 ? TX + 1 : TX;
+        const int f = e >> 1, g = e & 1;
+        const int fy = f / W1, fx = f - fy * W1;
+        const int r1l = d == 0 ? (fy + 1) * R1X + fx : fy * R1X + fx + 1;
+        const int r1r = r1l + (d == 0 ? 1 : R1X);
+        const TC t = d == 0 ? (g ? oy : -oy) : (g ? ox : -ox);
+        TC cl[NV], cr[NV], F[NF], rec[REC];
+        vec_get<REC>(s_rec + r1l * REC, rec);
+        eval2d<EQ, TC>(rec, rec + NV, d == 0 ? hh[0] : t, d == 0 ? t : hh[1], cl);
+        vec_get<REC>(s_rec + r1r * REC, rec);
+        eval2d<EQ, TC>(rec, rec + NV, d == 0 ? -hh[0] : t, d == 0 ? t : -hh[1], cr);
+        face_flux2d<EQ, TC>(G, d, cl, cr, F, err);
+  #pragma unroll
+        for (int q = 0; q < NF; ++q) s_f[(q * NF1 + f) * 2 + g] = F[q];
+      }
+    };
+    faces(std::integral_constant<int, 0>{});
+    faces(std::integral_constant<int, 1>{});
+  }
   // ---- four threads per cell: one volume Gauss point each, summed over the four lanes
   constexpr bool SPLIT = NT == 4 * NC;
   TC* s_vol = reinterpret_cast<TC*>(M.gy + R2Y);

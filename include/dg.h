@@ -120,7 +120,8 @@ const char* dg_last_error(const dg_ctx* ctx);
 
 /* Copy a state in (interchange layout, float64).  on_device != 0: `coeffs` is a
  * device pointer, else host memory (page-locked host memory is read in place by
- * the layout kernels; pageable memory is staged plane by plane).  Resets time and
+ * the layout kernel; pageable memory is staged through a device buffer kept by the
+ * context, at once up to 64 MB, else plane by plane).  Resets time and
  * step counters, clears the device error word and computes the first Courant
  * time step.  Synchronises the stream. */
 dg_status dg_set_state(dg_ctx* ctx, const double* coeffs, int on_device);
@@ -232,7 +233,7 @@ dg_status dg_profile(dg_ctx* ctx, int enable);
  * per-element staging) summed over their CTAs since profiling was last enabled.
  * Only the library's profiling build (compiled with DG_PHASE_PROFILE) counts
  * them; the normal build returns DG_EINVAL.  cycles[s * 16 + k] for stage s = 0, 1
- * and phase k; n >= 32.  2D phases: 0 staging, 1 primitives, 2 limiter, 3 faces,
+ * and phase k; n >= 32.  2D phases: 0 staging and primitives, 2 limiter, 3 faces,
  * 4 per-cell right-hand side and combination, 5 Courant reduction; 3D phases:
  * 0 staging and primitives, 1 limiter, 2 volume integral, 3/5/7 x/y/z faces,
  * 4/6/8 their gathers, 9 combination, 10 Courant reduction.  Synchronises. */

@@ -15,7 +15,7 @@ import os
 
 import numpy as np
 
-PHASES_2D = ["staging", "primitives", "limiter", "faces", "per-cell rhs + combination",
+PHASES_2D = ["staging + primitives", "(none)", "limiter", "faces", "per-cell rhs + combination",
              "Courant reduction"]
 PHASES_3D = ["staging + primitives", "limiter", "volume integral", "x faces", "x gather",
              "y faces", "y gather", "z faces", "z gather", "combination + store",

@@ -391,10 +391,11 @@ __device__ __forceinline__ void side_f64(const Gas<double>& G, double p, double 
   }
 }
 
-// p f''/f' of one side at x = p/pK (FP32).
+// p f''/f' of one side at x = p/pK (FP32): for a shock, f'' = -q (p + 4 B + 3 pK) /
+// (4 (p + B)^2) and f' = q (p + 2 B + pK) / (2 (p + B)); here B in units of pK.
 __device__ __forceinline__ float curvature_f32(const GasConst<float>& G, float x) {
   const float B = G.g6;
-  const float sh = -0.25f * x * (4.0f * B + 3.0f * x + 1.0f) *
+  const float sh = -0.25f * x * (4.0f * B + x + 3.0f) *
                    rcpv((x + B) * (0.5f * (x + 1.0f) + B));
   return x > 1.0f ? sh : -G.shk1;
 }

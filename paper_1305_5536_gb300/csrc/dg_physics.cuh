@@ -392,11 +392,14 @@ __device__ __forceinline__ void side_f64(const Gas<double>& G, double p, double 
 }
 
 // p f''/f' of one side at x = p/pK (FP32): for a shock, f'' = -q (p + 4 B + 3 pK) /
-// (4 (p + B)^2) and f' = q (p + 2 B + pK) / (2 (p + B)); here B in units of pK.
+// (4 (p + B)^2) and f' = q (p + 2 B + pK) / (2 (p + B)); here B in units of pK.  By
+// r = 1/x, a product of bounded factors (x^2 leaves the FP32 range from x = 1.8e19 on);
+// -1/2 for the strongest shocks, also where x itself leaves that range (r = 0).
 __device__ __forceinline__ float curvature_f32(const GasConst<float>& G, float x) {
   const float B = G.g6;
-  const float sh = -0.25f * x * (4.0f * B + x + 3.0f) *
-                   rcpv((x + B) * (0.5f * (x + 1.0f) + B));
+  const float r = rcpv(x);
+  const float sh = -0.25f * fmaf(4.0f * B + 3.0f, r, 1.0f) *
+                   rcpv(fmaf(B, r, 1.0f) * fmaf(0.5f + B, r, 0.5f));
   return x > 1.0f ? sh : -G.shk1;
 }
 

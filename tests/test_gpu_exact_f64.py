@@ -139,3 +139,21 @@ def test_random_pairs(fluxes, gamma, jump, mach):
     tol = 4 * EPS * 2 * gamma / (gamma - 1)
     d = np.abs(F - _reference(s, gamma)) / _scales(s, gamma)
     assert d.max() < tol, (float(d.max()), tol)
+
+
+@pytest.mark.parametrize("gamma", [5.0 / 3.0, 1.4, 1.1])
+def test_strong_shocks(fluxes, gamma):
+    """Pressure ratios up to 1e60 (the FP32 curvature once squared p*/pK), equal and unequal
+    densities, at rest and with the hot gas driven into the cold one, from either side."""
+    rng = np.random.default_rng(12)
+    k = np.concatenate([np.arange(2, 61), rng.uniform(15, 45, 400)])
+    r = np.exp(rng.uniform(-3, 3, k.size)) * (np.arange(k.size) % 2) + 1.0 * (np.arange(k.size) % 2 == 0)
+    u = np.sqrt(gamma) * rng.uniform(0, 2, k.size) * (np.arange(k.size) % 3 > 0)
+    one, zero = np.ones_like(k), np.zeros_like(k)
+    s = np.stack([one, u, one, zero, r, zero, 10.0 ** -k, 0.5 * one], 1)
+    m = s[:, [4, 5, 6, 7, 0, 1, 2, 3]] * np.array([1, -1, 1, 1, 1, -1, 1, 1])
+    s = np.concatenate([s, m])
+    F, err = fluxes(s, gamma)
+    assert (err == 0).all() and np.isfinite(F).all()
+    d = np.abs(F - _reference(s, gamma)) / _scales(s, gamma)
+    assert d.max() < 4 * EPS * 2 * gamma / (gamma - 1), float(d.max())

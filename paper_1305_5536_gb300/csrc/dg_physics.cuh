@@ -432,7 +432,7 @@ __device__ __forceinline__ Star64 star_f64(const Gas<double>& G, double rL, doub
     // relative Newton step, then Halley's correction 1 / (1 + step H), H = p f''/(2 f')
     const double dS = dfL + dfR, idS = rcpv(dS);
     double x = -(fL + fR + du) * idS * ip;
-    const float xf = Cvt<float>::to_tc(x);
+    float xf = Cvt<float>::to_tc(x);
     const float tL = Cvt<float>::to_tc(dfL * idS), tR = 1.0f - tL;  // shares of f'
     const float kL = tL * curvature_f32(H, Cvt<float>::to_tc(xL));
     const float kR = tR * curvature_f32(H, Cvt<float>::to_tc(xR));
@@ -440,7 +440,11 @@ __device__ __forceinline__ Star64 star_f64(const Gas<double>& G, double rL, doub
     if (!(fabsf(c) < 0.05f)) c = 0.0f;
     x = fma(-x, Cvt<float>::to_f64(c), x);
     double pn = fma(p, x, p);
-    if (!(pn > pfloor)) { pn = pfloor; x = fma(pn, ip, -1.0); }
+    if (!(pn > pfloor)) {  // held at the floor: the step that is taken, 0 once it rests there
+      pn = pfloor;
+      x = fma(pn, ip, -1.0);
+      xf = Cvt<float>::to_tc(x);
+    }
     R.p = pn;
     R.step = x;
     const double d = pn - p;

@@ -368,7 +368,7 @@ __device__ __forceinline__ void exact_flux_f32(const Gas<float>& G, float rL, fl
 //   * the pressure functions at p* for u* by their second-order Taylor expansion about
 //     the last point (error of order 1e-18), and p/p_K^z at p* likewise;
 //   * one power per side, (p/p_K)^z = w: the isentropic density is rho_K (p/p_K) / w^2;
-//   * wave-speed signs that FP32 decides (margin 1e-4 c) are not formed in FP64.
+//   * a shock speed whose sign FP32 decides (margin 1e-5 of it) is not formed in FP64.
 // About 200 FP64 operations a solve instead of above 2000 (pow in three or more Newton
 // evaluations, a re-evaluation and the sampling): 3D Euler 64^3 step 29.0 -> 5.3 ms, 2D
 // Euler 64^2 step 772 -> 154 us.
@@ -484,10 +484,13 @@ __device__ __forceinline__ void exact_flux_f64(const Gas<double>& G, double rL, 
   bool unpert, fan = false;
   double q = 1.0;  // (p/pK)^z at p*
   if (shock) {
-    const float cf = Cvt<float>::to_tc(cK);
-    const float s = Cvt<float>::to_tc(w) - cf * sqrtv(G.lo.shk1 * Cvt<float>::to_tc(x) + G.lo.z);
-    unpert = s >= 0.0f;
-    if (!(fabsf(s) > 1e-4f * cf)) unpert = w - cK * sqrt64(fma(G.shk1, x, G.z)) >= 0.0;
+    // w against the shock's speed m: decided in FP32 where the two differ by 1e-5, some 25
+    // times the rounding of both, and neither has left the FP32 range (m = inf fails too)
+    const float wf = Cvt<float>::to_tc(w);
+    const float m = Cvt<float>::to_tc(cK) * sqrtv(G.lo.shk1 * Cvt<float>::to_tc(x) + G.lo.z);
+    unpert = wf >= m;
+    if (!(m > 1e-30f && fabsf(wf - m) > 1e-5f * (fabsf(wf) + m)))
+      unpert = w - cK * sqrt64(fma(G.shk1, x, G.z)) >= 0.0;
   } else {
     // from the last evaluation by the relative step since then; from 1 (p = pK) where
     // that evaluation was on the shock side, less than a step away from pK

@@ -157,3 +157,30 @@ def test_strong_shocks(fluxes, gamma):
     assert (err == 0).all() and np.isfinite(F).all()
     d = np.abs(F - _reference(s, gamma)) / _scales(s, gamma)
     assert d.max() < 4 * EPS * 2 * gamma / (gamma - 1), float(d.max())
+
+
+@pytest.mark.parametrize("gamma", [5.0 / 3.0, 1.4, 1.1])
+def test_sign_of_the_shock_speed(fluxes, gamma):
+    """Shocks nearly at rest on the face (relative speeds down to 1e-13, Mach numbers up to
+    3e5) and cold gas (pressure ratios up to 1e60) streaming against hot gas about as fast as
+    the shock runs into it: on the wrong side of the shock the flux is off by its speed times
+    the jump."""
+    mach = np.array([1.5, 3, 30, 300, 3e3, 3e4, 3e5])
+    eps = np.array([0] + [q * 10.0 ** -k for k in range(6, 14) for q in (1, -1, 3, -3)])
+    m, e = (a.ravel() for a in np.meshgrid(mach, eps))
+    u1 = m * np.sqrt(gamma)
+    r2 = (gamma + 1) * m * m / ((gamma - 1) * m * m + 2)
+    p2 = 1 + 2 * gamma / (gamma + 1) * (m * m - 1)
+    one, zero = np.ones_like(m), np.zeros_like(m)
+    stat = np.stack([one, u1 * (1 - e), one, zero, r2, u1 / r2 - e * u1, p2, zero], 1)
+    rng = np.random.default_rng(13)
+    n = 2000
+    one, zero = np.ones(n), np.zeros(n)
+    cold = np.stack([np.exp(rng.uniform(-2, 2, n)), rng.uniform(0, 6, n), 10.0 ** -rng.uniform(5, 60, n),
+                     zero, one, zero, one, zero], 1)
+    s = np.concatenate([stat, cold])
+    s = np.concatenate([s, s[:, [4, 5, 6, 7, 0, 1, 2, 3]] * np.array([1, -1, 1, 1, 1, -1, 1, 1])])
+    F, err = fluxes(s, gamma)
+    assert (err == 0).all()
+    d = np.abs(F - _reference(s, gamma)) / _scales(s, gamma)
+    assert d.max() < 4 * EPS * 2 * gamma / (gamma - 1), float(d.max())

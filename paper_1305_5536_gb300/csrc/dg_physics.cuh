@@ -209,8 +209,10 @@ __device__ __forceinline__ double exact_guess(const Gas<double>& G, double rL, d
 // from the adaptive PVRS / TRRS / TSRS guess, sampled at x/t = 0) with the
 // arithmetic arranged for the FP32 pipes:
 //   * per side, the constants of the pressure function are formed once:
-//       shock       f = (p - pK) q,  q = (A_K / (p + B_K))^(1/2),
-//                   f' = q (1 - (p - pK) / (2 (p + B_K))) = q (1 - (p - pK) q^2 / (2 A_K)),
+//       shock       f = (p - pK) q,  q = A_K^(1/2) y,  y = (p + B_K)^(-1/2),
+//                   f' = q (1 - (p - pK) / (2 (p + B_K))) = q (1 - (p - pK) y^2 / 2)
+//                   (two roots, so that density times pressure need not be in range: in
+//                   cgs units it is 1e-40 in diffuse interstellar gas),
 //       rarefaction f = 2 cK / (g - 1) ((p/pK)^z - 1),  f' = (p/pK)^z cK / (g p),
 //     with A_K = 2 / ((g + 1) rho_K), B_K = (g - 1) / (g + 1) pK, z = (g - 1) / (2g);
 //     divisions become approximate reciprocals, square roots reciprocal square
@@ -239,7 +241,7 @@ __device__ __forceinline__ Star32 star_f32(const GasConst<float>& G, float rL, f
                                            float cL, float rR, float pR, float ipR, float cR,
                                            float du) {
   constexpr float accept = 2e-4f;
-  const float AiL = 0.5f * G.gp1 * rL, AiR = 0.5f * G.gp1 * rR;  // 1 / A_K
+  const float AL = rsqrtp(0.5f * G.gp1 * rL), AR = rsqrtp(0.5f * G.gp1 * rR);  // A_K^(1/2)
   const float BL = G.g6 * pL, BR = G.g6 * pR;
   const float CL = G.two_gm1 * cL, CR = G.two_gm1 * cR;          // 2 cK / (g - 1)
   const float DL = cL * G.inv_g, DR = cR * G.inv_g;              // cK / g
@@ -254,7 +256,7 @@ __device__ __forceinline__ Star32 star_f32(const GasConst<float>& G, float rL, f
       const float den = cL * ex2v(-G.z * lg2v(pL)) + cR * ex2v(-G.z * lg2v(pR));
       p = ex2v(G.inv_z * lg2v(num * rcpv(den)));
     } else {  // two shocks
-      const float gL = rsqrtp((BL + pv) * AiL), gR = rsqrtp((BR + pv) * AiR);
+      const float gL = AL * rsqrtp(BL + pv), gR = AR * rsqrtp(BR + pv);
       p = (gL * pL + gR * pR - du) * rcpv(gL + gR);
     }
   }
@@ -265,8 +267,8 @@ __device__ __forceinline__ Star32 star_f32(const GasConst<float>& G, float rL, f
     const float rp = rcpv(p);
     {
       const float dp = p - pL;
-      const float q = rsqrtp((p + BL) * AiL);
-      const float fs = dp * q, dfs = q * (1.0f - 0.5f * dp * q * q * AiL);
+      const float y = rsqrtp(p + BL), q = AL * y;
+      const float fs = dp * q, dfs = q * (1.0f - 0.5f * dp * y * y);
       const float qr = ex2v(G.z * lg2v(p * ipL));
       const float fr = CL * (qr - 1.0f), dfr = qr * DL * rp;
       const bool sh = p > pL;
@@ -275,8 +277,8 @@ __device__ __forceinline__ Star32 star_f32(const GasConst<float>& G, float rL, f
     }
     {
       const float dp = p - pR;
-      const float q = rsqrtp((p + BR) * AiR);
-      const float fs = dp * q, dfs = q * (1.0f - 0.5f * dp * q * q * AiR);
+      const float y = rsqrtp(p + BR), q = AR * y;
+      const float fs = dp * q, dfs = q * (1.0f - 0.5f * dp * y * y);
       const float qr = ex2v(G.z * lg2v(p * ipR));
       const float fr = CR * (qr - 1.0f), dfr = qr * DR * rp;
       const bool sh = p > pR;

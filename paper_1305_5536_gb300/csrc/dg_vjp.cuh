@@ -26,6 +26,18 @@ __device__ __forceinline__ float pow_m1v(float x, float z, float& w) {
 }
 __device__ __forceinline__ double pow_m1v(double x, double z, double& w) { return pow_m1(x, z, w); }
 
+// q = (Ai pb)^(-1/2) and 1/pb: in FP32 by two roots, as in star_f32.
+__device__ __forceinline__ float shock_q(float pb, float Ai, float& ipb) {
+  const float y = rsqrtp(pb);
+  ipb = y * y;
+  return y * rsqrtp(Ai);
+}
+__device__ __forceinline__ double shock_q(double pb, double Ai, double& ipb) {
+  const double q = rsqrtp(pb * Ai);
+  ipb = q * q * Ai;
+  return q;
+}
+
 // Pressure function of side K (Toro's f_K) and its partial derivatives with
 // respect to p, rho_K and p_K (c_K = sqrt(g p_K / rho_K) taken into account); i* are
 // reciprocals, qz = (p/p_K)^z on a rarefaction side.
@@ -35,8 +47,8 @@ __device__ __forceinline__ void pressure_fn_partials(const Gas<T>& G, T p, T ip,
                                                      T& qz) {
   if (gt_pos(p, pK)) {  // shock: f = (p - pK) q, q = (Ai (p + B))^(-1/2), 1/Ai = 2/((g+1) rho_K)
     const T Ai = T(0.5) * G.gp1 * rK;
-    const T q = rsqrtp((p + G.g6 * pK) * Ai);
-    const T ipb = q * q * Ai;
+    T ipb;
+    const T q = shock_q(p + G.g6 * pK, Ai, ipb);
     f = (p - pK) * q;
     df = q - T(0.5) * f * ipb;
     dpk = -q - T(0.5) * f * G.g6 * ipb;

@@ -150,6 +150,8 @@ __device__ __forceinline__ Dn<T, N>& operator+=(Dn<T, N>& a, const Dn<T, N>& b) 
 template <class T, int N>
 __device__ __forceinline__ Dn<T, N> sqrtv(const Dn<T, N>& a) { return dsqrt(a); }
 template <class T, int N>
+__device__ __forceinline__ Dn<T, N> sqrts(const Dn<T, N>& a) { return dsqrt(a); }
+template <class T, int N>
 __device__ __forceinline__ Dn<T, N> rcpv(const Dn<T, N>& a) { return T(1) / a; }
 template <class T, int N>
 __device__ __forceinline__ Dn<T, N> rsqrtp(const Dn<T, N>& a) { return T(1) / dsqrt(a); }

@@ -129,6 +129,12 @@ __device__ __forceinline__ float sqrtv(float x) {
   asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
   return r;
 }
+// A root whose operand may be subnormal (a fourth power of velocities is, from 3e-10 on).
+__device__ __forceinline__ float sqrts(float x) {
+  float r;
+  asm("sqrt.approx.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+}
 __device__ __forceinline__ float rsqrtp(float x) {
   float r;
   asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
@@ -145,6 +151,7 @@ __device__ __forceinline__ float lg2v(float x) {
   return r;
 }
 __device__ __forceinline__ double sqrtv(double x) { return sqrt64(x); }
+__device__ __forceinline__ double sqrts(double x) { return sqrt64(x); }
 __device__ __forceinline__ double rsqrtp(double x) { return rsqrt64(x); }
 
 // The smallest normal number of a type: slopes below it count as zero.

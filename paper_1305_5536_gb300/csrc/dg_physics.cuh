@@ -167,7 +167,7 @@ __device__ __forceinline__ T fast_speed2(const Gas<T>& G, T ir, T p, T b2, T bn)
   const T s = a2 + b2 * ir;
   T disc = s * s - T(4) * a2 * (bn * bn * ir);
   disc = negv(disc) ? T(0) : disc;
-  return T(0.5) * (s + sqrtv(disc));
+  return T(0.5) * (s + sqrts(disc));
 }
 template <class T>
 __device__ __forceinline__ T fast_speed(const Gas<T>& G, T rho, T p, T b2, T bn) {

@@ -216,7 +216,7 @@ __global__ void __launch_bounds__(TX * TY * TZ) mh3d_kernel(const Stage3DArgs<TS
     const unsigned g = (unsigned)(s_gz[rz] + s_gy[ry] + s_gx[rx]);
     TC c[5], W[5];
 #pragma unroll
-    for (int v = 0; v < 5; ++v) c[v] = Cvt<TC>::to_tc(__ldg(&(A.in.c0 + v * ncell)[g]));
+    for (int v = 0; v < 5; ++v) c[v] = Cvt<TC>::to_tc((A.in.c0 + v * ncell)[g]);
     prims3d<TC>(G, c, W, err);
 #pragma unroll
     for (int q = 0; q < 5; ++q) s_w[q * R2 + r] = W[q];

@@ -304,9 +304,11 @@ __device__ __forceinline__ void stage2d_take_dt(const Stage2DArgs<TS>& A, TileSc
 // coefficients are copied with cp.async and the averages of all of a thread's cells are
 // loaded before the first is converted, so that their DRAM latencies overlap.  (Walking
 // rows element by element and forming the primitives in a pass of their own: 2D MHD 512^2
-// FP32 68.4 against 62.7 us a step.)  C0: the
-// averages are kept beside the primitives (the MUSCL-Hancock kernel needs only the
-// latter).  The caller synchronises.
+// FP32 68.4 against 62.7 us a step.)  Plain loads: the batched kernel reads in stage 2 what
+// other CTAs of the same launch wrote in stage 1, and a dependent launch starts before the
+// kernel that writes its input has ended; the non-coherent path is for data that nothing
+// writes while the kernel runs.  C0: the averages are kept beside the primitives (the
+// MUSCL-Hancock kernel needs only the latter).  The caller synchronises.
 template <int EQ, class TC, class TS, int TX, int TY, int NT, bool C0 = true>
 __device__ __forceinline__ void stage2d_load(const Stage2DArgs<TS>& A, const TileMem<TC>& M,
                                              const Gas<TC>& G, unsigned& err) {
@@ -328,7 +330,7 @@ __device__ __forceinline__ void stage2d_load(const Stage2DArgs<TS>& A, const Til
           cp_async_elem<sizeof(TS)>(dst + k, A.in.sl + k * ncell + g);
       }
 #pragma unroll
-      for (int v = 0; v < T::NV; ++v) a[i][v] = __ldg(A.in.c0 + v * ncell + g);
+      for (int v = 0; v < T::NV; ++v) a[i][v] = (A.in.c0 + v * ncell)[g];
     }
   }
 #pragma unroll

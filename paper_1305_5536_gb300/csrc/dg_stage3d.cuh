@@ -342,8 +342,8 @@ __global__ void __launch_bounds__(TX * TY * TZ, (Stage3dMinBlocks<TX * TY * TZ, 
     double a[5], b[5];
 #pragma unroll
     for (int v = 0; v < 5; ++v) {
-      a[v] = __ldg(&(A.in.c0 + v * ncell)[ga]);
-      b[v] = __ldg(&(A.in.c0 + v * ncell)[gb]);
+      a[v] = (A.in.c0 + v * ncell)[ga];
+      b[v] = (A.in.c0 + v * ncell)[gb];
     }
     put(e, ra, oka, a);
     if (two) put(eb, rb, okb, b);

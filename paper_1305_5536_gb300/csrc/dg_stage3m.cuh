@@ -372,7 +372,7 @@ __global__ void __launch_bounds__(TX * TY * TZ, (Stage3mMinBlocks<TX * TY * TZ, 
     const unsigned g = (unsigned)(s_gz[rz] + s_gy[ry] + s_gx[rx]);
     TC c[8], W[8];
 #pragma unroll
-    for (int v = 0; v < 8; ++v) c[v] = Cvt<TC>::to_tc(__ldg(&(A.in.c0 + v * ncell)[g]));
+    for (int v = 0; v < 8; ++v) c[v] = Cvt<TC>::to_tc((A.in.c0 + v * ncell)[g]);
     prims3m<TC>(G, c, W, err);
 #pragma unroll
     for (int q = 0; q < 8; ++q) s_w[q * R2 + r] = W[q];

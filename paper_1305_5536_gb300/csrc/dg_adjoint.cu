@@ -1091,7 +1091,7 @@ void adjoint_reset(AdjointStore& s) {
 }
 
 dg_status adjoint_reserve(AdjointStore& s, int nplanes, long ncell, int k, long long nsteps,
-                          std::string& msg) {
+                          cudaStream_t st, std::string& msg) {
   if (nsteps <= s.cap_steps && s.ncell == ncell && s.nplanes == nplanes) return DG_OK;
   long long cap = std::max<long long>(nsteps, 2 * s.cap_steps);
   const size_t plane = (size_t)nplanes * ncell;
@@ -1107,8 +1107,16 @@ dg_status adjoint_reserve(AdjointStore& s, int nplanes, long ncell, int k, long 
   }
   if (s.nrec > 0 && s.ckpt && s.ncell == ncell && s.nplanes == nplanes) {
     const size_t old = (size_t)((s.nrec + k - 1) / k + 1);
-    cudaMemcpy(ck, s.ckpt, std::min(old, nck) * plane * sizeof(double), cudaMemcpyDeviceToDevice);
-    cudaMemcpy(dh, s.dt_hist, (size_t)s.nrec * sizeof(double), cudaMemcpyDeviceToDevice);
+    if (cudaMemcpyAsync(ck, s.ckpt, std::min(old, nck) * plane * sizeof(double),
+                        cudaMemcpyDeviceToDevice, st) != cudaSuccess ||
+        cudaMemcpyAsync(dh, s.dt_hist, (size_t)s.nrec * sizeof(double), cudaMemcpyDeviceToDevice, st) !=
+            cudaSuccess ||
+        cudaStreamSynchronize(st) != cudaSuccess) {
+      cudaFree(ck);
+      cudaFree(dh);
+      msg = "adjoint checkpoint store: copying the recorded checkpoints failed";
+      return DG_ECUDA;
+    }
   } else {
     s.nrec = 0;
   }

@@ -40,7 +40,7 @@ struct AdjointCall {
 void adjoint_free(AdjointStore& s);
 void adjoint_reset(AdjointStore& s);
 dg_status adjoint_reserve(AdjointStore& s, int nplanes, long ncell, int k, long long nsteps,
-                          std::string& msg);
+                          cudaStream_t st, std::string& msg);
 dg_status adjoint_step(AdjointStore& s, const AdjointCall& c, const double* u_n,
                        const double* lam_next, double* lam_prev, double dt, std::string& msg);
 dg_status adjoint_run(AdjointStore& s, const AdjointCall& c, int nplanes, int k,

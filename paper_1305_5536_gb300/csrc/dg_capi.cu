@@ -179,6 +179,10 @@ StateBuf<TS> sbuf(dg_ctx* c, int b, const Prob& p) {
   return s;
 }
 
+// Device memory of the context and its first contents.  Those are written on the caller's
+// stream: nothing orders the legacy stream before a non-blocking one, and a copy or a
+// memset there may run after the first launch.  (A copy from pageable memory returns once
+// its source has been read.)
 dg_status alloc_ctx(dg_ctx* c) {
   size_t c0n = 0, sln = 0;
   for (auto& p : c->probs) {
@@ -201,7 +205,7 @@ dg_status alloc_ctx(dg_ctx* c) {
   c->scratch_elems = std::max<size_t>((size_t)maxcell, 256 * 2 * 8);
   CK(c, cudaMalloc(&c->scratch, c->scratch_elems * sizeof(double)));
   CK(c, cudaMalloc(&c->ctl, c->probs.size() * sizeof(Ctl)));
-  CK(c, cudaMemset(c->ctl, 0, c->probs.size() * sizeof(Ctl)));
+  CK(c, cudaMemsetAsync(c->ctl, 0, c->probs.size() * sizeof(Ctl), c->stream));
   CK(c, cudaMallocHost(&c->ctl_host, c->probs.size() * sizeof(Ctl)));
   CK(c, cudaMalloc(&c->totals_dev, 16 * sizeof(double)));
   std::vector<LoadProb> tab;
@@ -220,9 +224,10 @@ dg_status alloc_ctx(dg_ctx* c) {
     tab.push_back(l);
   }
   CK(c, cudaMalloc(&c->ltab, tab.size() * sizeof(LoadProb)));
-  CK(c, cudaMemcpy(c->ltab, tab.data(), tab.size() * sizeof(LoadProb), cudaMemcpyHostToDevice));
+  CK(c, cudaMemcpyAsync(c->ltab, tab.data(), tab.size() * sizeof(LoadProb), cudaMemcpyHostToDevice,
+                        c->stream));
   CK(c, cudaMalloc(&c->lacc, tab.size() * sizeof(LoadAcc)));
-  CK(c, cudaMemset(c->lacc, 0, tab.size() * sizeof(LoadAcc)));
+  CK(c, cudaMemsetAsync(c->lacc, 0, tab.size() * sizeof(LoadAcc), c->stream));
   return DG_OK;
 }
 
@@ -711,10 +716,11 @@ dg_status build_batch(dg_ctx* c) {
     }
     c->btiles[v] = begin;
     CK(c, cudaMalloc(&c->btab[v], tab.size() * sizeof(BatchProb)));
-    CK(c, cudaMemcpy(c->btab[v], tab.data(), tab.size() * sizeof(BatchProb), cudaMemcpyHostToDevice));
+    CK(c, cudaMemcpyAsync(c->btab[v], tab.data(), tab.size() * sizeof(BatchProb), cudaMemcpyHostToDevice,
+                          c->stream));
   }
   CK(c, cudaMalloc(&c->bar, 2 * sizeof(unsigned)));
-  CK(c, cudaMemset(c->bar, 0, 2 * sizeof(unsigned)));
+  CK(c, cudaMemsetAsync(c->bar, 0, 2 * sizeof(unsigned), c->stream));
   // test hook (no GPU fault, no hang): the barrier expects one CTA more than is
   // launched, so every wait runs out after a short bounded spin
   const char* t = getenv("DG_TEST_BARRIER_TIMEOUT");
@@ -958,7 +964,7 @@ dg_status dg_profile(dg_ctx* c, int enable) {
 #ifdef DG_PHASE_PROFILE
     const size_t bytes = 2 * kPhaseSlots * sizeof(unsigned long long);
     if (!c->phase_dev) CK(c, cudaMalloc(&c->phase_dev, bytes));
-    CK(c, cudaMemset(c->phase_dev, 0, bytes));
+    CK(c, cudaMemsetAsync(c->phase_dev, 0, bytes, c->stream));
 #endif
   }
   c->prof = enable != 0;
@@ -971,8 +977,8 @@ dg_status dg_phase_cycles(dg_ctx* c, double* cycles, int n) {
 #ifdef DG_PHASE_PROFILE
   if (!c->phase_dev) return fail(c, DG_ESTATE, "enable profiling (dg_profile) first");
   unsigned long long h[2 * kPhaseSlots];
+  CK(c, cudaMemcpyAsync(h, c->phase_dev, sizeof(h), cudaMemcpyDeviceToHost, c->stream));
   CK(c, cudaStreamSynchronize(c->stream));
-  CK(c, cudaMemcpy(h, c->phase_dev, sizeof(h), cudaMemcpyDeviceToHost));
   for (int k = 0; k < 2 * kPhaseSlots; ++k) cycles[k] = (double)h[k];
   return DG_OK;
 #else
@@ -1073,7 +1079,7 @@ dg_status dg_record(dg_ctx* c, int nsteps, double dt_override, double* t_out) {
   std::string msg;
   // grow the store: checkpoints of the interchange state + time-step history
   dg_status s = adjoint_reserve(c->adj, c->nplanes, p.ncell, c->ckpt_every,
-                                c->adj.nrec + nsteps, msg);
+                                c->adj.nrec + nsteps, c->stream, msg);
   if (s != DG_OK) return fail(c, s, "%s", msg.c_str());
   // point the control block at the history
   Ctl h;

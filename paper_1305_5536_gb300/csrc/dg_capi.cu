@@ -58,13 +58,13 @@ struct dg_ctx {
   int cur = 0, nxt = 2;
   Ctl* ctl = nullptr;       // device, one per problem
   Ctl* ctl_host = nullptr;  // pinned mirror for readback
-  double* scratch = nullptr;  // device, one interchange plane (host transfers, totals)
-  double* stage = nullptr;    // device, all interchange planes (pageable host transfers of
-                              // states up to kStageElems; allocated by the first one)
-  LoadProb* ltab = nullptr;   // device, work list of the state load and save launches
-  LoadAcc* lacc = nullptr;    // device, one per problem
-  int lblocks = 0;
+  char* slab = nullptr;       // device: ctl, lacc, ltab, totals_dev and scratch
+  double* scratch = nullptr;  // host transfers, totals: all interchange planes of states up
+                              // to kStageElems, else one plane
   size_t scratch_elems = 0;
+  LoadProb* ltab = nullptr;   // work list of the state load and save launches
+  LoadAcc* lacc = nullptr;    // one per problem
+  int lblocks = 0;
   double* totals_dev = nullptr;
   int variant = -1;  // tile shape (-1: not tuned yet)
   bool state_set = false;
@@ -179,6 +179,10 @@ StateBuf<TS> sbuf(dg_ctx* c, int b, const Prob& p) {
   return s;
 }
 
+// Pageable host states up to this many elements (64 MB) cross in one copy through the
+// scratch buffer, larger ones plane by plane.
+constexpr size_t kStageElems = size_t(8) << 20;
+
 // Device memory of the context and its first contents.  Those are written on the caller's
 // stream: nothing orders the legacy stream before a non-blocking one, and a copy or a
 // memset there may run after the first launch.  (A copy from pageable memory returns once
@@ -200,14 +204,6 @@ dg_status alloc_ctx(dg_ctx* c) {
                   3.0 * (c0n * 8.0 + sln * ts) / 1e9);
     }
   }
-  long maxcell = 0;
-  for (auto& p : c->probs) maxcell = std::max(maxcell, p.ncell);
-  c->scratch_elems = std::max<size_t>((size_t)maxcell, 256 * 2 * 8);
-  CK(c, cudaMalloc(&c->scratch, c->scratch_elems * sizeof(double)));
-  CK(c, cudaMalloc(&c->ctl, c->probs.size() * sizeof(Ctl)));
-  CK(c, cudaMemsetAsync(c->ctl, 0, c->probs.size() * sizeof(Ctl), c->stream));
-  CK(c, cudaMallocHost(&c->ctl_host, c->probs.size() * sizeof(Ctl)));
-  CK(c, cudaMalloc(&c->totals_dev, 16 * sizeof(double)));
   std::vector<LoadProb> tab;
   for (auto& p : c->probs) {
     LoadProb l;
@@ -223,11 +219,32 @@ dg_status alloc_ctx(dg_ctx* c) {
     c->lblocks += l.nblk;
     tab.push_back(l);
   }
-  CK(c, cudaMalloc(&c->ltab, tab.size() * sizeof(LoadProb)));
-  CK(c, cudaMemcpyAsync(c->ltab, tab.data(), tab.size() * sizeof(LoadProb), cudaMemcpyHostToDevice,
-                        c->stream));
-  CK(c, cudaMalloc(&c->lacc, tab.size() * sizeof(LoadAcc)));
-  CK(c, cudaMemsetAsync(c->lacc, 0, tab.size() * sizeof(LoadAcc), c->stream));
+  // everything small in one allocation, and in it the staging buffer of pageable host
+  // transfers: a cudaMalloc is a good part of what a small context costs
+  long maxcell = 0;
+  for (auto& p : c->probs) maxcell = std::max(maxcell, p.ncell);
+  const size_t np = c->probs.size(), all = (size_t)c->nplanes * c->ncell_total;
+  const size_t plane = std::max<size_t>((size_t)maxcell, 256 * 2 * 8);
+  auto pad = [](size_t bytes) { return (bytes + 255) / 256 * 256; };
+  const size_t ctl_b = pad(np * sizeof(Ctl)), acc_b = pad(np * sizeof(LoadAcc)),
+               tab_b = pad(np * sizeof(LoadProb)), tot_b = pad(16 * sizeof(double));
+  const size_t small = ctl_b + acc_b + tab_b + tot_b;
+  c->scratch_elems = all <= kStageElems ? std::max(all, plane) : plane;
+  if (cudaMalloc(&c->slab, small + c->scratch_elems * sizeof(double)) != cudaSuccess) {
+    cudaGetLastError();  // no room to stage a whole state: plane by plane
+    c->slab = nullptr;
+    c->scratch_elems = plane;
+    CK(c, cudaMalloc(&c->slab, small + plane * sizeof(double)));
+  }
+  char* b = c->slab;
+  c->ctl = reinterpret_cast<Ctl*>(b);
+  c->lacc = reinterpret_cast<LoadAcc*>(b += ctl_b);
+  c->ltab = reinterpret_cast<LoadProb*>(b += acc_b);
+  c->totals_dev = reinterpret_cast<double*>(b += tab_b);
+  c->scratch = reinterpret_cast<double*>(b + tot_b);
+  CK(c, cudaMallocHost(&c->ctl_host, np * sizeof(Ctl)));
+  CK(c, cudaMemsetAsync(c->slab, 0, ctl_b + acc_b, c->stream));
+  CK(c, cudaMemcpyAsync(c->ltab, tab.data(), np * sizeof(LoadProb), cudaMemcpyHostToDevice, c->stream));
   return DG_OK;
 }
 
@@ -615,17 +632,9 @@ static void* mapped_view(const void* host) {
   return a.type == cudaMemoryTypeHost ? a.devicePointer : nullptr;
 }
 
-// Pageable host memory up to this many elements (64 MB) crosses in one copy through a
-// device buffer kept by the context; larger states plane by plane through `scratch`.
-constexpr size_t kStageElems = size_t(8) << 20;
+// The scratch buffer, if it takes the whole state.
 static double* stage_buffer(dg_ctx* c) {
-  const size_t n = (size_t)c->nplanes * c->ncell_total;
-  if (n > kStageElems) return nullptr;
-  if (!c->stage && cudaMalloc(&c->stage, n * sizeof(double)) != cudaSuccess) {
-    cudaGetLastError();
-    c->stage = nullptr;
-  }
-  return c->stage;
+  return (size_t)c->nplanes * c->ncell_total <= c->scratch_elems ? c->scratch : nullptr;
 }
 
 template <class TS>
@@ -836,12 +845,7 @@ void dg_destroy(dg_ctx* c) {
     cudaFree(c->c0[b]);
     cudaFree(c->sl[b]);
   }
-  cudaFree(c->scratch);
-  cudaFree(c->stage);
-  cudaFree(c->ltab);
-  cudaFree(c->lacc);
-  cudaFree(c->ctl);
-  cudaFree(c->totals_dev);
+  cudaFree(c->slab);
   for (int v = 0; v < 3; ++v) cudaFree(c->btab[v]);
   cudaFree(c->bar);
   cudaFree(c->phase_dev);

@@ -514,10 +514,16 @@ bool g_tune_loaded = false;
 // time (this also keeps concurrent trial steps from timing each other)
 std::mutex g_tune_mutex;
 
+// Number of the set of tile shapes, part of every key: raised when an index changes its
+// shape or a table grows, so that a file written before is tuned anew instead of being
+// read as other tiles (1, without a number in the key: FP64 3D Euler 1 was 8x4x2, FP64 2D
+// had no tiles with four threads per cell).
+constexpr int kTileSet = 2;
+
 std::string tune_key(dg_ctx* c) {
   char b[128];
   const Prob& p = c->probs[0];
-  snprintf(b, sizeof(b), "eq%d_d%d_fp%d_lim%d_%dx%dx%d_np%zu", c->eq, c->dim, c->fp32 ? 32 : 64,
+  snprintf(b, sizeof(b), "t%d_eq%d_d%d_fp%d_lim%d_%dx%dx%d_np%zu", kTileSet, c->eq, c->dim, c->fp32 ? 32 : 64,
            c->limiter, p.nx, p.ny, p.nz, c->probs.size());
   std::string k = b;
   if (c->integrator == DG_MUSCL_HANCOCK) k += "_mh" + std::to_string(c->face_points);

@@ -36,8 +36,9 @@ def _deps_mtime():
     return t
 
 
-# Forward stage kernels: FP32 division and square root to within 2 ulp (the
-# single-precision path only; double precision is always IEEE-exact).
+# Forward stage kernels: FP32 division and square root to within 2 ulp.  These flags leave
+# double precision alone; where the kernels call rcpv, sqrt64 or rsqrt64 of dg_f64.cuh it is
+# good to about 1 ulp, a plain / or sqrt is IEEE-exact.
 FAST_FP32 = ["-prec-div=false", "-prec-sqrt=false"]
 FAST_FP32_SOURCES = ("dg_k2d.cu", "dg_k3d.cu", "dg_k3m.cu", "dg_kmh.cu", "dg_kmh3d.cu", "dg_kmh3m.cu",
                      "dg_batch.cu")

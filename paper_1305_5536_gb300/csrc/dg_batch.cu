@@ -98,8 +98,9 @@ __device__ __forceinline__ void sweep(const BatchArgs<TS>& B, unsigned char* sme
   }
 }
 
-// FP32: 80 registers a thread (the tile code plus the work list's; at the stage kernels'
-// 64 it spills: 48 problems 638 against 630 us a step).
+// FP32: 80 registers a thread (48 problems 630 us a step, against 638 at the stage kernels'
+// 64).  It still spills there (16x16 MHD: 240 bytes stored, 216 loaded): the arguments of a
+// tile, which the single-problem kernels read from the constant bank, are formed per tile.
 template <int NT, class TC>
 struct BatchMinBlocks {
   static constexpr int v = sizeof(TC) == 4 ? 65536 / (80 * NT) : 1;

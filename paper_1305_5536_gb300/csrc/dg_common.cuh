@@ -233,7 +233,7 @@ __host__ __device__ __forceinline__ void halo3d_cell(int e, int& rx, int& ry, in
 // face count of a rolled loop over orientations): floor(n / d) = (n * m) >> 32
 // with m = ceil(2^32 / d), exact for n < 2^14 and 2 <= d <= 1024 (checked for
 // every such pair; d = 1 would need m = 2^32); two instructions instead of a full
-// integer division.
+// integer division.  (The present stage kernels know their face counts at compile time.)
 __host__ __device__ __forceinline__ unsigned div_magic(unsigned d) {
   return (unsigned)((0x100000000ull + d - 1) / d);
 }

@@ -441,7 +441,8 @@ __device__ __forceinline__ void mh2d_compute(const Stage2DArgs<TS>& A, int i0, i
 }
 
 // FP32: as many resident CTAs as the shared memory of the face-centroid rule allows
-// (5 of 256 threads: 48 registers a thread, where nothing spills).
+// (5 of 256 threads: 48 registers a thread, where the 16x8 and 32x8 tiles spill nothing and
+// the 16x16 MHD tile 16 bytes).
 template <int EQ, int NT, int NGF, bool WENO, class TC>
 struct MhMinBlocks {
   static constexpr int R = NGF == 1 && !(EQ == 1 && WENO) ? 48 : 64;

@@ -126,7 +126,6 @@ struct GasConst {
   T g, gm1, gp1, inv_gm1;
   T z;        // (g-1)/(2g)
   T inv_z;    // 2g/(g-1)
-  T mzp;      // -(g+1)/(2g)
   T g6;       // (g-1)/(g+1)
   T shk1;     // (g+1)/(2g)
   T inv_g;    // 1/g
@@ -139,7 +138,6 @@ struct GasConst {
     inv_gm1 = T(1.0 / (gamma - 1.0));
     z = T((gamma - 1.0) / (2.0 * gamma));
     inv_z = T(2.0 * gamma / (gamma - 1.0));
-    mzp = T(-(gamma + 1.0) / (2.0 * gamma));
     g6 = T((gamma - 1.0) / (gamma + 1.0));
     shk1 = T((gamma + 1.0) / (2.0 * gamma));
     inv_g = T(1.0 / gamma);

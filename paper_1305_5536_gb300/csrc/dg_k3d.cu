@@ -32,19 +32,21 @@ static cudaError_t launch3d(int stage, const Stage3DArgs<TS>& a, cudaStream_t st
   return launch3d_w<TC, TS, TX, TY, TZ, false>(stage, a, st);
 }
 
-// FP64: 8x4x4 has less halo per cell (64^3 4422 against 4561 us a step), 4x4x4 spreads a
-// small grid wider (24^3 446 against 512 us).
-int stage3d_variants(int) { return 2; }
+// FP64: 8x4x4 has less halo per cell (64^3 4422 us a step, 8x4x2 4561), 4x4x4 spreads a
+// small grid wider (24^3 446 against 512 us), 8x4x2 leaves no tile half empty on grids of one
+// or two planes (256x256x2 2375 against 4278 us).
+int stage3d_variants(int fp32) { return fp32 ? 2 : 3; }
 
 const char* stage3d_variant_name(int fp32, int v) {
-  static const char* n64[] = {"4x4x4", "8x4x4"};
+  static const char* n64[] = {"4x4x4", "8x4x4", "8x4x2"};
   static const char* n32[] = {"8x8x4", "8x4x4"};
-  if (v < 0 || v > 1) return "?";
+  if (v < 0 || v > (fp32 ? 1 : 2)) return "?";
   return fp32 ? n32[v] : n64[v];
 }
 
 cudaError_t launch_stage3d(int variant, int stage, const Stage3DArgs<double>& a, cudaStream_t st) {
   if (variant == 1) return launch3d<double, double, 8, 4, 4>(stage, a, st);
+  if (variant == 2) return launch3d<double, double, 8, 4, 2>(stage, a, st);
   return launch3d<double, double, 4, 4, 4>(stage, a, st);
 }
 

@@ -31,6 +31,9 @@ static cudaError_t launch_mh3d_ngf(int face_points, const Stage3DArgs<TS>& a, cu
   return launch_mh3d_t<TC, TS, TX, TY, TZ, 1, false>(a, st);
 }
 
+// FP64: 4x4x4 has less halo per cell (64^3 971 against 1045 us a step, 96^3 3156 against
+// 3485), 8x4x2 leaves no tile half empty on grids of one or two planes (256x256x2 517 against
+// 913 us).
 int mh3d_variants(int) { return 2; }
 
 const char* mh3d_variant_name(int fp32, int v) {

@@ -114,7 +114,7 @@ __device__ __forceinline__ Dn<T, N> operator/(T a, const Dn<T, N>& b) {
 template <class T, int N>
 __device__ __forceinline__ Dn<T, N> dsqrt(const Dn<T, N>& a) {
   Dn<T, N> r;
-  r.v = sqrtv(a.v);
+  r.v = sqrts(a.v);
   T k = r.v > T(0) ? T(0.5) / r.v : T(0);
 #pragma unroll
   for (int i = 0; i < N; ++i) r.d[i] = a.d[i] * k;

@@ -131,7 +131,8 @@ __device__ __forceinline__ float sqrtv(float x) {
   asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
   return r;
 }
-// A root whose operand may be subnormal (a fourth power of velocities is, from 3e-10 on).
+// A root whose operand may be subnormal: a square of velocities (from 1e-19 on), a fourth
+// power of them (from 3e-10 on).
 __device__ __forceinline__ float sqrts(float x) {
   float r;
   asm("sqrt.approx.f32 %0, %1;" : "=f"(r) : "f"(x));

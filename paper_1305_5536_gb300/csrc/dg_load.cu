@@ -63,7 +63,7 @@ __device__ __forceinline__ TC signal_speed(const Gas<TC>& G, const double* a, co
   else if constexpr (EQ == 0) prims3d<TC>(G, c, W, err);
   else prims3m<TC>(G, c, W, err);
   if constexpr (EQ == 0) {
-    s[0] = sqrtv(G.g * W[DIM + 1] * rcpv(W[0]));
+    s[0] = sqrts(G.g * W[DIM + 1] * rcpv(W[0]));
 #pragma unroll
     for (int d = 1; d < DIM; ++d) s[d] = s[0];
   } else {

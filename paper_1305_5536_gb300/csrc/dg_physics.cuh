@@ -305,7 +305,7 @@ __device__ __forceinline__ void exact_flux_f32(const Gas<float>& G, float rL, fl
   }
   const float ipL = rcpv(pL), ipR = rcpv(pR);
   const float aL = G.g * pL * rcpv(rL), aR = G.g * pR * rcpv(rR);
-  const float cL = sqrtv(aL), cR = sqrtv(aR);
+  const float cL = sqrts(aL), cR = sqrts(aR);
   const float du = uR - uL;
   if (G.two_gm1 * cL + G.two_gm1 * cR <= du) err |= ERR_VACUUM;
   const Star32 S = star_f32(G, rL, pL, ipL, cL, rR, pR, ipR, cR, du);

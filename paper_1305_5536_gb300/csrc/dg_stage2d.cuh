@@ -377,7 +377,7 @@ __device__ __forceinline__ void courant_commit2d(const Stage2DArgs<TS>& A, const
     prims2d<EQ, TC>(G, c, W, err);
     TC cx, cy;
     if (EQ == 0) {
-      cx = cy = sqrtv(G.g * W[3] * rcpv(W[0]));
+      cx = cy = sqrts(G.g * W[3] * rcpv(W[0]));
     } else {
       TC b2 = W[4] * W[4] + W[5] * W[5];
       cx = fast_speed(G, W[0], W[3], b2, W[4]);

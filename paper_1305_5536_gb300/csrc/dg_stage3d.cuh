@@ -548,7 +548,7 @@ __global__ void __launch_bounds__(TX * TY * TZ, (Stage3dMinBlocks<TX * TY * TZ, 
 #pragma unroll
       for (int v = 0; v < 5; ++v) c[v] = Cvt<TC>::to_tc(o0[v]);
       prims3d<TC>(G, c, W, err);
-      TC cs = sqrtv(G.g * W[4] * rcpv(W[0]));
+      TC cs = sqrts(G.g * W[4] * rcpv(W[0]));
       sp = (fabs(W[1]) + cs) * geo.ih[0] + (fabs(W[2]) + cs) * geo.ih[1] +
            (fabs(W[3]) + cs) * geo.ih[2];
       if (!courant_ok(sp, W[0], W[4])) { err |= ERR_NONPHYS; sp = TC(0); }

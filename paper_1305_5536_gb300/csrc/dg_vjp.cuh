@@ -92,7 +92,7 @@ __device__ void exact_flux_vjp(const Gas<T>& G, T rL, T uL, T vL, T pL, T rR, T 
     return;
   }
   const T irL = rcpv(rL), irR = rcpv(rR), ipL = rcpv(pL), ipR = rcpv(pR);
-  const T cL = sqrtv(G.g * pL * irL), cR = sqrtv(G.g * pR * irR);
+  const T cL = sqrts(G.g * pL * irL), cR = sqrts(G.g * pR * irR);
   const T du = uR - uL;
   if (G.two_gm1 * (cL + cR) <= du) err |= ERR_VACUUM;
   const T p = vjp_pstar(G, rL, pL, ipL, cL, rR, pR, ipR, cR, du, err);

@@ -89,3 +89,25 @@ def test_euler_adjoint_step(rho0, c0):
         out.append(s.adjoint_step(lam, torch.from_numpy(u).cuda(), dt).cpu().numpy() / w)
     # 1e-4 of the adjoint's scale: the bar of the FP32 adjoint
     assert np.abs(out[1] - out[0]).max() < 1e-4 * np.abs(out[0]).max()
+
+
+@pytest.mark.parametrize("gamma", [5.0 / 3.0, 1.4])
+@pytest.mark.parametrize("integrator,limiter,jump,mach", [("mh", 0, 0.3, 0.5), ("rk2", 1, 0.3, 0.5)])
+def test_euler_step_with_a_subnormal_square_of_the_sound_speed(jump, mach, integrator, limiter, gamma):
+    _one_step(_state(gamma, 1e25, 4e-20, jump, mach), gamma, integrator, limiter)
+
+
+@pytest.mark.parametrize("rho0,c0", [(1.0, 1.0), (1.0, 1e-9), (1.0, 3e-10)])
+def test_mhd_adjoint_step(rho0, c0):
+    """The fast speed's root and its derivative where the operand is subnormal."""
+    gamma = 1.4
+    u = _state(gamma, rho0, c0, 0.3, 0.5, mhd=True)
+    dt = 0.2 * O.Problem(O.MHD, 2, N, gamma=gamma, limiter=0).cfl_dt(u)[0]
+    w = np.concatenate([np.repeat([1.0, 1 / c0, 1 / c0, 1 / c0 ** 2], 3), np.full(5, 1 / c0)])[:, None, None]
+    lam = torch.from_numpy(np.random.default_rng(3).normal(size=u.shape) * w).cuda()
+    out = []
+    for prec in ("fp64", "fp32"):
+        s = dg.DGSolver("mhd", 2, N, gamma=gamma, limiter=0, precision=prec)
+        out.append(s.adjoint_step(lam, torch.from_numpy(u).cuda(), dt).cpu().numpy() / w)
+    # 1e-4 of the adjoint's scale: the bar of the FP32 adjoint
+    assert np.abs(out[1] - out[0]).max() < 1e-4 * np.abs(out[0]).max()

@@ -63,6 +63,7 @@ struct dg_ctx {
                               // to kStageElems, else one plane
   size_t scratch_elems = 0;
   LoadProb* ltab = nullptr;   // work list of the state load and save launches
+  std::vector<LoadProb> ltab_host;  // its source, kept while a copy on the stream may read it
   LoadAcc* lacc = nullptr;    // one per problem
   int lblocks = 0;
   double* totals_dev = nullptr;
@@ -79,6 +80,7 @@ struct dg_ctx {
   // batched 2D problems: one persistent launch per step over a tile work list
   bool batch2d = false;
   BatchProb* btab[3] = {nullptr, nullptr, nullptr};  // per tile variant of the batch kernel
+  std::vector<BatchProb> btab_host[3];
   int btiles[3] = {0, 0, 0};
   unsigned* bar = nullptr;
   long long spin_limit = 1LL << 24;
@@ -185,8 +187,7 @@ constexpr size_t kStageElems = size_t(8) << 20;
 
 // Device memory of the context and its first contents.  Those are written on the caller's
 // stream: nothing orders the legacy stream before a non-blocking one, and a copy or a
-// memset there may run after the first launch.  (A copy from pageable memory returns once
-// its source has been read.)
+// memset there may run after the first launch.
 dg_status alloc_ctx(dg_ctx* c) {
   size_t c0n = 0, sln = 0;
   for (auto& p : c->probs) {
@@ -204,7 +205,7 @@ dg_status alloc_ctx(dg_ctx* c) {
                   3.0 * (c0n * 8.0 + sln * ts) / 1e9);
     }
   }
-  std::vector<LoadProb> tab;
+  std::vector<LoadProb>& tab = c->ltab_host;
   for (auto& p : c->probs) {
     LoadProb l;
     l.ncell = p.ncell;
@@ -244,7 +245,8 @@ dg_status alloc_ctx(dg_ctx* c) {
   c->scratch = reinterpret_cast<double*>(b + tot_b);
   CK(c, cudaMallocHost(&c->ctl_host, np * sizeof(Ctl)));
   CK(c, cudaMemsetAsync(c->slab, 0, ctl_b + acc_b, c->stream));
-  CK(c, cudaMemcpyAsync(c->ltab, tab.data(), np * sizeof(LoadProb), cudaMemcpyHostToDevice, c->stream));
+  CK(c, cudaMemcpyAsync(c->ltab, c->ltab_host.data(), np * sizeof(LoadProb), cudaMemcpyHostToDevice,
+                        c->stream));
   return DG_OK;
 }
 
@@ -710,7 +712,7 @@ dg_status build_batch(dg_ctx* c) {
   c->batch2d = true;
   for (int v = 0; v < 3; ++v) {
     const int tx = batch2d_tile_x(c->fp32, v), ty = batch2d_tile_y(c->fp32, v);
-    std::vector<BatchProb> tab;
+    std::vector<BatchProb>& tab = c->btab_host[v];
     int begin = 0;
     for (const Prob& p : c->probs) {
       BatchProb b{};
@@ -731,8 +733,8 @@ dg_status build_batch(dg_ctx* c) {
     }
     c->btiles[v] = begin;
     CK(c, cudaMalloc(&c->btab[v], tab.size() * sizeof(BatchProb)));
-    CK(c, cudaMemcpyAsync(c->btab[v], tab.data(), tab.size() * sizeof(BatchProb), cudaMemcpyHostToDevice,
-                          c->stream));
+    CK(c, cudaMemcpyAsync(c->btab[v], c->btab_host[v].data(), tab.size() * sizeof(BatchProb),
+                          cudaMemcpyHostToDevice, c->stream));
   }
   CK(c, cudaMalloc(&c->bar, 2 * sizeof(unsigned)));
   CK(c, cudaMemsetAsync(c->bar, 0, 2 * sizeof(unsigned), c->stream));

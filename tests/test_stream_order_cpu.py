@@ -21,3 +21,12 @@ def test_no_copy_or_memset_on_the_legacy_stream(name):
     # the asynchronous forms name a stream
     for call in re.findall(r"\bcudaMem(?:set|cpy)Async\s*\(((?:[^()]|\((?:[^()]|\([^()]*\))*\))*)\)", code):
         assert re.search(r"(stream|\bst)\s*$", call.strip()), call
+
+
+def test_sources_of_copies_to_the_device_outlive_them():
+    """A copy enqueued from pageable memory may read it later (the host's page tables are the
+    device's on Grace-Blackwell): tables are copied from vectors that the context keeps."""
+    with open(os.path.join(CSRC, "dg_capi.cu")) as f:
+        code = re.sub(r"//[^\n]*", "", f.read())
+    for src in re.findall(r"cudaMemcpyAsync\(\s*[^,]+,\s*([^,]+?),[^;]*cudaMemcpyHostToDevice", code):
+        assert ".data()" not in src or src.startswith("c->"), src
